@@ -71,17 +71,14 @@
 // and lambda_i = 1 - sum of the others (exact 64-bit integers).
 #include <math.h>
 
-#include <type_traits>
-
 #include "ac_internal.cuh"
 
 namespace ac {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int STAGE = 32;
-constexpr int PAIR_CHUNK = 128;
-constexpr int CAND_CAP = 256;  // triangle or tetrahedron candidates written out per batch
-constexpr int PL_CAP = 256;    // Sigma^2 pairs listed during the triangle phase
+constexpr int CAND_CAP = 256;  // triangle candidates written out per batch
+constexpr unsigned TET_OPEN = 1u << 31;  // of a code in tl: AC3 not decided yet
 
 template <int WORDS>
 struct WarpSmem {
@@ -89,24 +86,17 @@ struct WarpSmem {
     // row positions take 8 bits up to 256 neighbours, 10 bits beyond
     static constexpr int SH = WORDS > 8 ? 10 : 8;
     static constexpr unsigned PM = (1u << SH) - 1u;
-    using Pos = typename std::conditional<(WORDS > 8), unsigned short, unsigned char>::type;
-    using Pair = typename std::conditional<(WORDS > 8), unsigned, unsigned short>::type;
     float4 qf[M];   // (qx, qy, qz, a_x): coordinates exact, a_x rounded once
     int ai[M];      // a_x exact
     float rs[M];    // sqrt(W_x + A) rounded up
     int idx[M];     // sorted position
     unsigned Mrow[M][WORDS];
-    unsigned Trow[M][WORDS];
-    unsigned up[WORDS];
-    Pos uplist[M];
-    unsigned char upf[M];  // edge (i, x) in Sigma^1, by position
-    int n_up;
+    unsigned kup[WORDS];   // the upper edges (positions below n_up) not shown to be outside K^1
     int n_tet, n_tri, n_edge;
-    int rowpre[M + 1];                // prefix sums of candidate counts per row of up
-    int pairpre[PAIR_CHUNK + 1];      // prefix sums of tetrahedron candidates per Sigma^2 pair
-    Pair plist[PL_CAP];               // Sigma^2 pairs (p | k << SH) in enumeration order
-    int n_pl;                         // pairs found (the list holds them while n_pl <= PL_CAP)
-    unsigned cand[CAND_CAP];          // candidate codes (p | k << SH [| l << 2 SH]) of the current batch
+    int n_tl;                         // tetrahedra pushed (the list holds the first TL_CAP)
+    unsigned cand[CAND_CAP];          // triangle candidate codes (p | k << SH) of the current batch
+    static constexpr int TL_CAP = WORDS > 2 ? 256 : 128;
+    unsigned tl[TL_CAP];              // tetrahedra to settle: p | k << SH | l << 2 SH [| TET_OPEN]
     int4 st_tet[STAGE];
     int4 st_tri[STAGE];
     int2 st_edge[STAGE];
@@ -126,6 +116,8 @@ struct Bounds {
     R g3s;    // gamma_3 (1 + gamma_3)
     R up1;    // >= 1 + 1.01 u
     R two_up; // >= 2 / (1 - delta_r): 1/|X~| <= |rcp(2 X~)| two_up
+    R K2, K3; // error of the line test beyond that of its Delta: K2 (2 S) + K3
+    R inv_lo; // 1 - 64 u: takes an upper bound of 1/det~ below it
 };
 
 struct LocalArgs {
@@ -148,6 +140,7 @@ struct LocalArgs {
     PredConst pc;
     Bounds<float> b32;
     Bounds<double> b64;
+    float perp_err;  // >= the rounding errors of |q_x|^2 - (q_x.u)^2 (edge discs)
     // FP64 thresholds of the resolve kernel (y from exact minors)
     double tet_eps64, tri_k0_64, tri_k1_64;
     int4* tet_out;
@@ -188,8 +181,12 @@ struct Ar<float> {
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
         return r;
     }
+    static __device__ __forceinline__ float fma_dn(float a, float b, float c) { return __fmaf_rd(a, b, c); }
+    static __device__ __forceinline__ float to_f32_up(float a) { return a; }
+    static __device__ __forceinline__ float to_f32_dn(float a) { return a; }
     static __device__ __forceinline__ float abs(float a) { return fabsf(a); }
     static __device__ __forceinline__ float max(float a, float b) { return fmaxf(a, b); }
+    static __device__ __forceinline__ float min(float a, float b) { return fminf(a, b); }
 };
 
 template <>
@@ -202,8 +199,12 @@ struct Ar<double> {
     static __device__ __forceinline__ double add_up(double a, double b) { return __dadd_ru(a, b); }
     static __device__ __forceinline__ double sub_dn(double a, double b) { return __dsub_rd(a, b); }
     static __device__ __forceinline__ double rcp(double a) { return __drcp_rn(a); }
+    static __device__ __forceinline__ double fma_dn(double a, double b, double c) { return __fma_rd(a, b, c); }
+    static __device__ __forceinline__ float to_f32_up(double a) { return __double2float_ru(a); }
+    static __device__ __forceinline__ float to_f32_dn(double a) { return __double2float_rd(a); }
     static __device__ __forceinline__ double abs(double a) { return fabs(a); }
     static __device__ __forceinline__ double max(double a, double b) { return fmax(a, b); }
+    static __device__ __forceinline__ double min(double a, double b) { return a < b ? a : b; }
 };
 
 template <class R>
@@ -227,22 +228,6 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
     return m;
-}
-
-// position of the r-th (0-based) set bit of m; requires r < popc(m)
-__device__ __forceinline__ int nth_set_bit(unsigned m, int r) {
-    int pos = 0;
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        unsigned low = (1u << w) - 1u;
-        int c = __popc(m & low);
-        if (r >= c) {
-            r -= c;
-            m >>= w;
-            pos += w;
-        }
-    }
-    return pos;
 }
 
 template <class T>
@@ -303,17 +288,6 @@ __device__ __forceinline__ void stage_push(const int lane, bool want, const T& i
     __syncwarp();
 }
 
-// largest r in [0, n) with pre[r] <= j (pre non-decreasing, pre[0] = 0 <= j)
-__device__ __forceinline__ int row_of(const int* pre, int n, int j) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre[mid] <= j) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 // warp-wide exclusive prefix sum of per-lane counts c; the total goes to *tot
 __device__ __forceinline__ int warp_excl(int lane, int c, int* tot) {
     int incl = c;
@@ -326,23 +300,27 @@ __device__ __forceinline__ int warp_excl(int lane, int c, int* tot) {
     return incl - c;
 }
 
-// bits of word w of a row that lie above position p
+// Rows of positions are bitmasks with position e at bit 31 - (e & 31) of word
+// e / 32: the lowest position of a word is its highest set bit, which one
+// instruction finds (the lowest set bit takes two).
+__device__ __forceinline__ int first_pos(unsigned b) {
+    int r;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(r) : "r"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned pos_bit(int e) { return 0x80000000u >> (e & 31); }
+
+// bits of word w of a row that lie below, above position p
+__device__ __forceinline__ unsigned below_mask(int w, int p) {
+    if (32 * w + 31 < p) return FULL;
+    if (32 * w >= p) return 0u;
+    return ~(FULL >> (p & 31));
+}
+
 __device__ __forceinline__ unsigned above_mask(int w, int p) {
     if (32 * w + 31 <= p) return 0u;
     if (32 * w > p) return FULL;
-    return ~((2u << (p & 31)) - 1u);
-}
-
-// position of the rank-th set bit of the multi-word mask f(w), w < nw
-template <class F>
-__device__ __forceinline__ int nth_in_words(int nw, int rank, F&& f) {
-    for (int w = 0; w < nw; w++) {
-        const unsigned mw = f(w);
-        const int pc = __popc(mw);
-        if (rank < pc) return 32 * w + nth_set_bit(mw, rank);
-        rank -= pc;
-    }
-    return 0;
+    return 0x7fffffffu >> (p & 31);
 }
 
 // ---------------------------------------------------------------------------
@@ -355,13 +333,19 @@ struct Ortho {
     int ac3;  // +1 holds, -1 fails, 0 undecided
 };
 
-// AC3 from y~ and its bound: |y|^2 <= T (T exact)
+// |y|^2 from y~ and its bound: S~ and e_S
 template <class R>
-__device__ __forceinline__ int ac3_from(const Ortho<R>& o, R T, const Bounds<R>& B) {
+__device__ __forceinline__ void norm2(const Ortho<R>& o, const Bounds<R>& B, R& S, R& eS) {
     using A = Ar<R>;
-    const R S = A::fma(o.y2, o.y2, A::fma(o.y1, o.y1, A::mul(o.y0, o.y0)));
+    S = A::fma(o.y2, o.y2, A::fma(o.y1, o.y1, A::mul(o.y0, o.y0)));
     const R l1 = A::add_up(A::add_up(A::abs(o.y0), A::abs(o.y1)), A::abs(o.y2));
-    const R eS = A::fma_up(o.ey, A::fma_up(R(3), o.ey, A::mul_up(R(2), l1)), A::mul_up(B.g3s, S));
+    eS = A::fma_up(o.ey, A::fma_up(R(3), o.ey, A::mul_up(R(2), l1)), A::mul_up(B.g3s, S));
+}
+
+// AC3: |y|^2 <= T (T exact)
+template <class R>
+__device__ __forceinline__ int ac3_of(R S, R eS, R T) {
+    using A = Ar<R>;
     if (A::sub_dn(S, eS) > T) return -1;
     if (A::add_up(S, eS) < T) return 1;
     return 0;
@@ -416,14 +400,49 @@ __device__ __forceinline__ Ortho<R> ortho_tet(const P4<R>& q1, const P4<R>& q2, 
     const R eN = A::mul_up(B.cN, A::add_up(A::add_up(A::abs(q1.w), A::abs(q2.w)), A::abs(q3.w)));
     const R Y = A::max(A::abs(o.y0), A::max(A::abs(o.y1), A::abs(o.y2)));
     o.ey = quotient_bound(eN, inv, Y, rho, B);
-    o.ac3 = ac3_from(o, T, B);
+    R S, eS;
+    norm2(o, B, S, eS);
+    o.ac3 = ac3_of(S, eS, T);
     return o;
 }
 
+// rsqrt.approx.ftz.f32: documented within 2^-22.9 relative
+__device__ __forceinline__ float rsqrt_f32(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// sqrt.approx.ftz.f32 is documented within 2^-23 relative of the root; the
+// factors leave eight times that
+__device__ __forceinline__ float sqrt_up(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmul_ru(r, 1.0f + 0x1p-20f);
+}
+
+__device__ __forceinline__ float sqrt_dn(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmul_rd(r, 1.0f - 0x1p-20f);
+}
+
+// The triangle's line of equal power, y + s n with n = q_1 x q_2, and the part
+// of it inside the grown balls of its vertices, |s| <= S (header comment).
 template <class R>
-__device__ __forceinline__ Ortho<R> ortho_tri(const P4<R>& q1, const P4<R>& q2, R T, const Bounds<R>& B) {
+struct TriLine {
+    R z0, z1, z2, n0, n1, n2;  // z = -2 y
+    R E;           // bound on |Delta~ - Delta| at y
+    R Ei;          // bound on |(Delta~ - 2 s g~) - Delta(y + s n)|, |s| <= S
+    R s2lo;        // <= 2 S
+    float s2;      // >= 2 S
+    int ac3;
+};
+
+template <class R>
+__device__ __forceinline__ TriLine<R> tri_line(const P4<R>& q1, const P4<R>& q2, R T, const Bounds<R>& B) {
     using A = Ar<R>;
-    Ortho<R> o;
+    TriLine<R> L;
     const R g11 = A::fma(q1.z, q1.z, A::fma(q1.y, q1.y, A::mul(q1.x, q1.x)));
     const R g22 = A::fma(q2.z, q2.z, A::fma(q2.y, q2.y, A::mul(q2.x, q2.x)));
     const R g12 = A::fma(q1.z, q2.z, A::fma(q1.y, q2.y, A::mul(q1.x, q2.x)));
@@ -431,12 +450,14 @@ __device__ __forceinline__ Ortho<R> ortho_tri(const P4<R>& q1, const P4<R>& q2, 
     const R r = A::rcp(R(2) * det);
     const R inv = A::mul_up(A::abs(r), B.two_up);  // >= 1/|det~|
     const R rho = A::mul_up(B.eDet, inv);
-    if (!(rho <= R(0.125))) {
-        o.ac3 = 0;
-        o.ey = R(INFINITY);
-        o.y0 = o.y1 = o.y2 = R(0);
-        return o;
+    if (!(rho <= R(0.125))) {  // every test on this line is undecided
+        L.z0 = L.z1 = L.z2 = L.n0 = L.n1 = L.n2 = L.s2lo = R(0);
+        L.s2 = 0.0f;
+        L.E = L.Ei = R(INFINITY);
+        L.ac3 = 0;
+        return L;
     }
+    Ortho<R> o;
     const R n1 = A::fma(g22, q1.w, -A::mul(g12, q2.w));
     const R n2 = A::fma(g11, q2.w, -A::mul(g12, q1.w));
     const R m1 = A::mul(n1, r), m2 = A::mul(n2, r);
@@ -446,8 +467,25 @@ __device__ __forceinline__ Ortho<R> ortho_tri(const P4<R>& q1, const P4<R>& q2, 
     o.y1 = A::fma(m1, q1.y, A::mul(m2, q2.y));
     o.y2 = A::fma(m1, q1.z, A::mul(m2, q2.z));
     o.ey = A::mul_up(B.H, A::fma_up(R(2), emu, A::mul_up(B.ky, A::add_up(A::abs(m1), A::abs(m2)))));
-    o.ac3 = ac3_from(o, T, B);
-    return o;
+    R S, eS;
+    norm2(o, B, S, eS);
+    L.ac3 = ac3_of(S, eS, T);
+    L.z0 = R(-2) * o.y0;
+    L.z1 = R(-2) * o.y1;
+    L.z2 = R(-2) * o.y2;
+    L.n0 = cross_c(q1.y, q2.z, q1.z, q2.y);
+    L.n1 = cross_c(q1.z, q2.x, q1.x, q2.z);
+    L.n2 = cross_c(q1.x, q2.y, q1.y, q2.x);
+    // S^2 = (T - |y|^2) / det, 1 / det between inv (1 - 64 u) (1 - rho) and inv (1 + 1.2 rho)
+    const R t_up = A::max(A::add_up(A::add_up(T, -S), eS), R(0));
+    const R t_lo = A::max(A::sub_dn(A::sub_dn(T, S), eS), R(0));
+    const R s2_up = A::mul_up(A::mul_up(t_up, inv), A::fma_up(R(1.2), rho, R(1)));
+    const R s2_lo = A::mul_dn(A::mul_dn(t_lo, A::mul_dn(inv, B.inv_lo)), A::sub_dn(R(1), rho));
+    L.s2 = 2.0f * sqrt_up(A::to_f32_up(s2_up));
+    L.s2lo = R(2) * R(sqrt_dn(A::to_f32_dn(s2_lo)));
+    L.E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);
+    L.Ei = A::add_up(A::fma_up(B.K2, R(L.s2), B.K3), L.E);
+    return L;
 }
 
 template <class R>
@@ -468,27 +506,34 @@ __device__ __forceinline__ Ortho<R> ortho_edge(const P4<R>& q1, const Bounds<R>&
     return o;
 }
 
-// AC2 scan of one simplex; the candidates of word w are M[p] & M[k] & M[l]
-// (nv = 3), M[p] & M[k] (nv = 2) or M[p] (nv = 1). Returns -1 if a candidate
-// violates AC2, +1 if every test clears, 0 if none violates but some test is
-// undecided at this precision.
+// Delta at y from z = -2 y (exact): three FMAs starting from a_x
+template <class R>
+__device__ __forceinline__ R delta(const P4<R>& v, R z0, R z1, R z2) {
+    return Ar<R>::fma(v.z, z2, Ar<R>::fma(v.y, z1, Ar<R>::fma(v.x, z0, v.w)));
+}
+
+template <class R>
+__device__ __forceinline__ R dot3(const P4<R>& v, R n0, R n1, R n2) {
+    return Ar<R>::fma(v.z, n2, Ar<R>::fma(v.y, n1, Ar<R>::mul(v.x, n0)));
+}
+
+// AC2 scan of a tetrahedron (i,p,k,l) over the candidates M[p] & M[k] & M[l].
+// Returns -1 if a candidate violates AC2, +1 if every test clears, 0 if none
+// violates but some test is undecided at this precision.
 template <class R, int WORDS>
-__device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const Ortho<R>& o, const Bounds<R>& B, int nv,
-                                        int p, int k, int l, unsigned& n_ok) {
+__device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const Ortho<R>& o, const Bounds<R>& B, int p,
+                                        int k, int l, unsigned& n_ok) {
     using A = Ar<R>;
     const R E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);  // inf when o.ey is
+    const R z0 = R(-2) * o.y0, z1 = R(-2) * o.y1, z2 = R(-2) * o.y2;
     bool open = false;
 #pragma unroll 1
     for (int w = 0; w < nw; w++) {
-        unsigned b = S.Mrow[p][w];
-        if (nv >= 2) b &= S.Mrow[k][w];
-        if (nv == 3) b &= S.Mrow[l][w];
+        unsigned b = S.Mrow[p][w] & S.Mrow[k][w] & S.Mrow[l][w];
         while (b) {
-            const int x = 32 * w + __ffs(b) - 1;
-            b &= b - 1;
-            const P4<R> v = point<R>(S, x);
-            const R t = A::fma(v.z, o.y2, A::fma(v.y, o.y1, A::mul(v.x, o.y0)));
-            const R d = A::fma(R(-2), t, v.w);
+            const int e = first_pos(b);
+            b ^= pos_bit(e);
+            const R d = delta(point<R>(S, 32 * w + e), z0, z1, z2);
             n_ok++;
             if (d < -E) return -1;
             if (!(d > E)) open = true;
@@ -500,7 +545,7 @@ __device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const 
 // ---------------------------------------------------------------------------
 
 template <int WORDS, class R, bool KEEP>
-__global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using SM = WarpSmem<WORDS>;
     constexpr int MAXM = SM::M;
@@ -554,22 +599,40 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
         const int nw = (m + 31) >> 5;
         const R T = (R)si;  // W_i + A <= 2^24: exact
 
-        // ---- phase A: load L(i) in order of distance from p_i; vertex AC2
-        // (Step 5); upper edges with exact edge AC3. The order only changes
-        // the order of the AC2 tests: the nearest balls are the likeliest
-        // violators of the simplices around p_i, so scans stop sooner.
+        // ---- phase A: load L(i), the n_up neighbours with an edge of Sigma^1 owned
+        // by i first, each part in order of distance from p_i; vertex AC2 (Step
+        // 5). With the upper edges in front, their positions are 0 .. n_up - 1:
+        // a tetrahedron's masks end at word n_up / 32, one word for nine atoms
+        // in ten. The order by distance only changes the order of the AC2 tests:
+        // the nearest balls are the likeliest violators of the simplices around
+        // p_i, so scans stop sooner.
+        unsigned vert_bad = 0;
+        int n_up = 0;
 #pragma unroll 1
         for (int w = 0; w < nw; w++) {
             const int e = 32 * w + lane;
+            bool upper = false;
             if (e < m) {
                 const int x = A.nb[off + e];
                 const int4 o = A.Ps[x];
                 const int qx = o.x - Pi.x, qy = o.y - Pi.y, qz = o.z - Pi.z;
                 S.idx[e] = x;
                 const int D = qx * qx + qy * qy + qz * qz;  // in (0, 2^26]
-                // narrow rows: one 32-bit key D * 64 + e, unique (D = 2^26 wraps to e, below every other key)
-                S.ai[e] = WORDS <= 2 ? (int)((unsigned)D * 64u + (unsigned)e) : D;
+                if (x > i) {
+                    // edge AC3: (D + W_i - W_x)^2 <= 4 D (W_i + A)
+                    const long long a = (long long)D + Wi - o.w;
+                    upper = a * a <= 4ll * D * si;
+                    n_ac3e++;
+                }
+                // Delta_x = a_x at p_i; a tie goes against the larger input index
+                const int ax = D - o.w + Wi;
+                if (ax < 0 || (ax == 0 && A.order[x] < gi)) vert_bad = 1;
+                // sort key: upper edges first, then D (its lowest bit dropped); narrow rows append e,
+                // which makes it unique
+                const unsigned key = (unsigned)(D - 1) >> 1 | (upper ? 0u : 1u << 25);
+                S.ai[e] = (int)(WORDS <= 2 ? key * 64u + (unsigned)e : key);
             }
+            n_up += __popc(__ballot_sync(FULL, upper));
         }
         __syncwarp();
         int xr[WORDS], rr[WORDS];
@@ -579,15 +642,15 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
             xr[w] = -1;
             rr[w] = 0;
             if (w < nw && e < m) {
-                const int De = S.ai[e];
+                const unsigned De = (unsigned)S.ai[e];
                 int rank = 0;
                 if constexpr (WORDS <= 2) {
 #pragma unroll 4
-                    for (int f = 0; f < m; f++) rank += (unsigned)S.ai[f] < (unsigned)De ? 1 : 0;
+                    for (int f = 0; f < m; f++) rank += (unsigned)S.ai[f] < De ? 1 : 0;
                 } else {
 #pragma unroll 4
                     for (int f = 0; f < m; f++) {
-                        const int Df = S.ai[f];
+                        const unsigned Df = (unsigned)S.ai[f];
                         rank += (Df < De || (Df == De && f < e)) ? 1 : 0;
                     }
                 }
@@ -596,69 +659,35 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
             }
         }
         __syncwarp();
-        unsigned vert_bad = 0;
 #pragma unroll
         for (int w = 0; w < WORDS; w++) {
             if (xr[w] >= 0) {
                 const int x = xr[w], e = rr[w];
                 const int4 o = A.Ps[x];
                 const int qx = o.x - Pi.x, qy = o.y - Pi.y, qz = o.z - Pi.z;
-                const int D = qx * qx + qy * qy + qz * qz;  // <= 2^26
-                const int ax = D - o.w + Wi;
+                const int ax = qx * qx + qy * qy + qz * qz - o.w + Wi;
                 S.qf[e] = make_float4((float)qx, (float)qy, (float)qz, (float)ax);
                 S.ai[e] = ax;
                 S.rs[e] = __fsqrt_ru((float)((long long)o.w + Aq));  // W + A <= 2^24: exact in FP32
-                const int gx = A.order[x];
                 S.idx[e] = x;
-                // Delta_x = a_x at p_i; a tie goes against the larger input index
-                if (ax < 0 || (ax == 0 && gx < gi)) vert_bad = 1;
-                bool upper = false;
-                if (x > i) {
-                    // edge AC3: (D + W_i - W_x)^2 <= 4 D (W_i + A)
-                    const long long a = (long long)D + Wi - o.w;
-                    upper = a * a <= 4ll * D * si;
-                    n_ac3e++;
-                }
-                S.upf[e] = upper ? 1 : 0;
             }
         }
-        __syncwarp();
-#pragma unroll 1
-        for (int w = 0; w < nw; w++) {
-            const int e = 32 * w + lane;
-            const unsigned b = __ballot_sync(FULL, e < m && S.upf[e] != 0);
-            if (lane == 0) S.up[w] = b;
-        }
-        if (lane == 0)
-            for (int w = nw; w < WORDS; w++) S.up[w] = 0u;
         vert_bad = __any_sync(FULL, vert_bad);
-        if (lane == 0) A.vert_pass[i] = vert_bad ? 0 : 1;
-        __syncwarp();
-        {
-            int base = 0;
-#pragma unroll 1
-            for (int w = 0; w < nw; w++) {
-                const unsigned b = S.up[w];
-                if ((b >> lane) & 1u) S.uplist[base + __popc(b & lanemask_lt())] = (typename SM::Pos)(32 * w + lane);
-                base += __popc(b);
-            }
-            if (lane == 0) {
-                S.n_up = base;
-                n_s1 += base;
-            }
+        if (lane == 0) {
+            A.vert_pass[i] = vert_bad ? 0 : 1;
+            n_s1 += n_up;
         }
         __syncwarp();
-        const int n_up = S.n_up;
+        const int nu = (n_up + 31) >> 5;
         if (keep) {
             for (int r0 = 0; r0 < n_up; r0 += 32) {
-                const bool ok = r0 + lane < n_up;
-                const int p = ok ? S.uplist[r0 + lane] : 0;
-                append_direct(ok, make_int2(i, ok ? S.idx[p] : 0), A.cand1, &cnt->n_cand_out[1], A.cap_cand[1], &cnt->err,
-                              DERR_OVF_CAND);
+                const int p = r0 + lane;
+                append_direct(p < n_up, make_int2(i, p < n_up ? S.idx[p] : 0), A.cand1, &cnt->n_cand_out[1], A.cap_cand[1],
+                              &cnt->err, DERR_OVF_CAND);
             }
         }
 
-        // ---- phase B: adjacency rows M[p] for p in up ------------------------
+        // ---- phase B: adjacency rows M[p] of the upper edges -------------------
         // The rows only filter candidates, so they may hold more than the exact
         // relation: |q_e - q_p|^2 rounded down <= (sqrt s_p + sqrt s_e)^2 rounded up
         // keeps every pair whose grown balls meet (and a few more at the margin).
@@ -677,8 +706,7 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
                 cr[w] = S.rs[cv[w] ? e : 0];
             }
 #pragma unroll 1
-            for (int r = 0; r < n_up; r++) {
-                const int p = S.uplist[r];
+            for (int p = 0; p < n_up; p++) {
                 const float4 qp = S.qf[p];
                 const float rp = S.rs[p];
 #pragma unroll
@@ -688,16 +716,12 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
                     const float rr = __fadd_ru(rp, cr[w]);
                     const bool adj = cv[w] && 32 * w + lane != p && d2 <= __fmul_ru(rr, rr);
                     const unsigned b = __ballot_sync(FULL, adj);  // words past nw come out empty
-                    if (lane == 0) {
-                        S.Mrow[p][w] = b;
-                        S.Trow[p][w] = 0u;
-                    }
+                    if (lane == 0) S.Mrow[p][w] = __brev(b);
                 }
             }
         } else {
 #pragma unroll 1
-        for (int r = 0; r < n_up; r++) {
-            const int p = S.uplist[r];
+        for (int p = 0; p < n_up; p++) {
             const float4 qp = S.qf[p];
             const float rp = S.rs[p];
 #pragma unroll 1
@@ -712,47 +736,160 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
                     adj = d2 <= __fmul_ru(rr, rr);
                 }
                 const unsigned b = __ballot_sync(FULL, adj);
-                if (lane == 0) {
-                    S.Mrow[p][w] = b;
-                    S.Trow[p][w] = 0u;
+                if (lane == 0) S.Mrow[p][w] = __brev(b);
+            }
+        }
+        }
+        if (lane < WORDS) S.kup[lane] = 0u;
+        if (lane == 0) S.n_tl = 0;
+        __syncwarp();
+
+        // ---- phase C: edges (i,p), a lane each: AC2 at the edge's orthocentre, and
+        // whether some ball leaves nothing of the edge's disc (no K^1 then)
+#pragma unroll 1
+        for (int r0 = 0; r0 < n_up; r0 += 32) {
+            const int p = r0 + lane;
+            const bool ok = p < n_up;
+            bool pass = false, pend = false;
+            if (ok) {
+                const Ortho<R> o = ortho_edge<R>(point<R>(S, p), B);
+                R S2, eS;
+                norm2(o, B, S2, eS);
+                const R E = Ar<R>::mul_up(Ar<R>::fma_up(B.K1, o.ey, B.K0), B.up1);
+                const R z0 = R(-2) * o.y0, z1 = R(-2) * o.y1, z2 = R(-2) * o.y2;
+                // 4 rho^2, rho the disc's radius; the last factor covers the products below
+                const float r4 = 4.0f * (1.0f + 0x1p-18f) *
+                                 Ar<R>::to_f32_up(Ar<R>::max(Ar<R>::add_up(Ar<R>::add_up(T, -S2), eS), R(0)));
+                const float4 qp = S.qf[p];
+                const float ri = rsqrt_f32(__fmaf_rn(qp.z, qp.z, __fmaf_rn(qp.y, qp.y, __fmul_rn(qp.x, qp.x))));
+                const float u0 = qp.x * ri, u1 = qp.y * ri, u2 = qp.z * ri;  // unit vector along the edge
+                R dmin = R(INFINITY);
+                bool out = false;
+#pragma unroll 1
+                for (int w = 0; w < nw; w++) {
+                    unsigned b = S.Mrow[p][w];
+                    n_edge += __popc(b);
+                    while (b) {
+                        const int e = first_pos(b);
+                        b ^= pos_bit(e);
+                        const float4 q = S.qf[32 * w + e];
+                        const R d = delta(point<R>(S, 32 * w + e), z0, z1, z2);
+                        dmin = Ar<R>::min(d, dmin);
+                        if (d < -E) {
+                            // Delta_x < 0 all over the disc iff -Delta_x > 2 rho |q_x - (q_x.u) u|
+                            const float m = Ar<R>::to_f32_dn(Ar<R>::sub_dn(-d, E));
+                            const float t = __fmaf_rn(q.z, u2, __fmaf_rn(q.y, u1, __fmul_rn(q.x, u0)));
+                            const float X2 = __fmaf_rn(q.z, q.z, __fmaf_rn(q.y, q.y, __fmaf_rn(q.x, q.x, A.perp_err)));
+                            if (__fmul_rn(m, m) > __fmul_rn(r4, __fmaf_rn(-t, t, X2))) {
+                                out = true;
+                                n_edge -= __popc(b);
+                                break;
+                            }
+                        }
+                    }
+                    if (out) break;
+                }
+                if (!out) {
+                    atomicOr(&S.kup[p >> 5], pos_bit(p));
+                    pass = dmin > E;
+                    pend = !pass && !(dmin < -E);
                 }
             }
-            if (lane == 0)
-                for (int w = nw; w < WORDS; w++) {
-                    S.Mrow[p][w] = 0u;
-                    S.Trow[p][w] = 0u;
-                }
-        }
+            const int idp = ok ? S.idx[p] : 0;
+            append_direct(pend, make_int4(i, idp, -1, -1), A.pending, &cnt->n_pending, A.cap_pending, &cnt->err,
+                          DERR_OVF_PEND);
+            stage_push(lane, pass, make_int2(i, idp), S.st_edge, &S.n_edge, A.edge_out, &cnt->n_edge_pass, A.cap_edge,
+                       &cnt->err, DERR_OVF_EDGE);
         }
         __syncwarp();
 
-        if (lane == 0) S.n_pl = 0;
-        __syncwarp();
-        // ---- phase C: triangles (i,p,k): AC3, then AC2 at the orthocentre -----
-        // Candidates of row r (p = uplist[r]): k in M[p] & up, k > p. Rows are
+        // ---- phase D: triangles (i,p,k) and the tetrahedra over them ----------
+        // The tetrahedra of the list, 32 per window: AC3 where it is open, AC2.
+        auto settle_tets = [&]() {
+            __syncwarp();
+            const int n_list = min(S.n_tl, SM::TL_CAP);
+#pragma unroll 1
+            for (int base = 0; base < n_list; base += 32) {
+                const int j = base + lane;
+                const bool valid = j < n_list;
+                bool pass = false, pend = false, counted = false;
+                bool pend_ac3 = false;
+                int p3 = 0, k3 = 0, ll = 0;
+                if (valid) {
+                    const unsigned code = S.tl[j];
+                    p3 = code & SM::PM;
+                    k3 = (code >> SM::SH) & SM::PM;
+                    ll = (code >> (2 * SM::SH)) & SM::PM;
+                    const Ortho<R> o = ortho_tet<R>(point<R>(S, p3), point<R>(S, k3), point<R>(S, ll), T, B);
+                    const bool open = (code & TET_OPEN) != 0u;
+                    if (!open || o.ac3 > 0) {
+                        counted = open;
+                        n_s3 += open ? 1 : 0;
+                        const int r3 = ac2_scan<R>(S, nw, o, B, p3, k3, ll, n_tet);
+                        pass = r3 > 0;
+                        pend = r3 == 0;
+                    } else if (o.ac3 == 0) {
+                        pend = pend_ac3 = true;
+                    }
+                }
+                const int4 item = make_int4(i, valid ? S.idx[p3] : 0, valid ? S.idx[k3] : 0, valid ? S.idx[ll] : 0);
+                if (keep)
+                    append_direct(counted, item, A.cand3, &cnt->n_cand_out[3], A.cap_cand[3], &cnt->err,
+                                  DERR_OVF_CAND);
+                append_direct(pend, make_int4(pend_ac3 ? ~i : i, item.y, item.z, item.w), A.pending, &cnt->n_pending,
+                              A.cap_pending, &cnt->err, DERR_OVF_PEND);
+                stage_push(lane, pass, item, S.st_tet, &S.n_tet, A.tet_out, &cnt->n_tet_out, A.cap_tet, &cnt->err,
+                           DERR_OVF_TET);
+            }
+            __syncwarp();
+            if (lane == 0) S.n_tl = 0;
+            __syncwarp();
+        };
+        // One lane's tetrahedron for the list, or (list full) for the pending list.
+        auto push_tet = [&](int pp, int kk, int x, bool open) {
+            const int slot = atomicAdd(&S.n_tl, 1);
+            if (slot < SM::TL_CAP) {
+                S.tl[slot] = (unsigned)pp | ((unsigned)kk << SM::SH) | ((unsigned)x << (2 * SM::SH)) | (open ? TET_OPEN : 0u);
+            } else {
+                const unsigned long long at = atomicAdd(&cnt->n_pending, 1ull);
+                if ((int64_t)at < A.cap_pending) A.pending[at] = make_int4(open ? ~i : i, S.idx[pp], S.idx[kk], S.idx[x]);
+                else atomicOr(&cnt->err, DERR_OVF_PEND);
+            }
+        };
+        // Candidates of row k < n_up: p in M[k], p < k. Rows are
         // taken 32 at a time, one per lane; each writes its candidates as codes
-        // p | k << SH to cand[] in row order (CAND_CAP per batch), and windows
-        // of 32 candidates read them back.
+        // p | k << SH to cand[] (CAND_CAP per batch), first those with both edges
+        // in kup, then the rest, and windows of 32 candidates read them back. A
+        // window's candidates share a few neighbouring k, so their lanes have
+        // about the same number of x above k to test.
 #pragma unroll 1
         for (int r0 = 0; r0 < n_up; r0 += 32) {
-            const bool rv = r0 + lane < n_up;
-            const int p = rv ? S.uplist[r0 + lane] : 0;
-            int c = 0;
-            if (rv)
-                for (int w = 0; w < nw; w++) c += __popc(S.Mrow[p][w] & S.up[w] & above_mask(w, p));
-            int tot;
-            const int ex = warp_excl(lane, c, &tot);
+            const int k = r0 + lane;
+            const bool rv = k < n_up;
+            const int kw1 = rv ? (k >> 5) + 1 : 0;  // words with a position below k
+            const unsigned in_k = rv && (S.kup[k >> 5] & pos_bit(k)) ? FULL : 0u;
+            unsigned c = 0;  // candidates with both edges in kup, and (upper half) the others: below 2^15 for 32 rows
+#pragma unroll 1
+            for (int w = 0; w < kw1; w++) {
+                const unsigned b = S.Mrow[k][w] & below_mask(w, k), bk = b & S.kup[w] & in_k;
+                c += (unsigned)__popc(bk) | ((unsigned)__popc(b ^ bk) << 16);
+            }
+            int tot_;
+            const unsigned ex = (unsigned)warp_excl(lane, (int)c, &tot_);
+            const int tot0 = (int)((unsigned)tot_ & 0xffffu), tot = tot0 + (int)((unsigned)tot_ >> 16);
 #pragma unroll 1
             for (int done = 0; done < tot; done += CAND_CAP) {
-                if (c > 0 && ex < done + CAND_CAP && ex + c > done) {
-                    int t = ex;
-                    for (int w = 0; w < nw; w++) {
-                        unsigned b = S.Mrow[p][w] & S.up[w] & above_mask(w, p);
+                if (c) {
+                    int t0 = (int)(ex & 0xffffu) - done, t1 = tot0 + (int)(ex >> 16) - done;
+#pragma unroll 1
+                    for (int w = 0; w < kw1; w++) {
+                        unsigned b = S.Mrow[k][w] & below_mask(w, k);
+                        const unsigned bk = b & S.kup[w] & in_k;
                         while (b) {
-                            const int k = 32 * w + __ffs(b) - 1;
-                            b &= b - 1;
-                            if (t >= done && t < done + CAND_CAP) S.cand[t - done] = (unsigned)p | ((unsigned)k << SM::SH);
-                            t++;
+                            const int e = first_pos(b);
+                            b ^= pos_bit(e);
+                            const int t = bk & pos_bit(e) ? t0++ : t1++;
+                            if (t >= 0 && t < CAND_CAP) S.cand[t] = (unsigned)(32 * w + e) | ((unsigned)k << SM::SH);
                         }
                     }
                 }
@@ -762,252 +899,120 @@ __global__ void __launch_bounds__(256, 4) k_local(LocalArgs A) {
                 for (int base = 0; base < nbatch; base += 32) {
                     const int j = base + lane;
                     const bool valid = j < nbatch;
-                    bool pass = false, pend = false, keep_it = false;
-                    int pend_ac3 = 0;
+                    bool pass = false, pend = false;
                     int pp = 0, kk = 0;
-                    Ortho<R> o;
-                    o.ac3 = -1;
+                    TriLine<R> L;
+                    L.ac3 = -1;
                     if (valid) {
                         const unsigned code = S.cand[j];
                         pp = code & SM::PM;
                         kk = code >> SM::SH;
-                        n_ac3t++;
-                        o = ortho_tri<R>(point<R>(S, pp), point<R>(S, kk), T, B);
-                        if (o.ac3 >= 0) {
-                            // potential, or not yet excluded: tetrahedra may build on it
-                            atomicOr(&S.Trow[pp][kk >> 5], 1u << (kk & 31));
-                            if (o.ac3 > 0) {
-                                n_s2++;
-                                keep_it = true;
-                            } else {
-                                pend = true;
-                                pend_ac3 = 1;
+                        L = tri_line<R>(point<R>(S, pp), point<R>(S, kk), T, B);
+                    }
+                    const bool keep_it = L.ac3 > 0;
+                    n_ac3t += valid ? 1u : 0u;
+                    n_s2 += keep_it ? 1u : 0u;
+                    // the part of the line nearer to the triangle than to any ball: -nlo <= 2 s <= hi
+                    float hi = L.s2, nlo = L.s2;
+                    const float c = 0x1p-16f * L.s2;  // quotients are within 2^-19 relative, see below
+                    bool alive = keep_it && done + j < tot0;
+                    if (alive) {
+                        R dmin = R(INFINITY);
+#pragma unroll 1
+                        for (int w = 0; w < nw; w++) {
+                            unsigned b = S.Mrow[pp][w] & S.Mrow[kk][w];
+                            n_tri += __popc(b);
+                            while (b) {
+                                const int e = first_pos(b);
+                                b ^= pos_bit(e);
+                                const P4<R> v = point<R>(S, 32 * w + e);
+                                const R d = delta(v, L.z0, L.z1, L.z2);
+                                const R g = dot3(v, L.n0, L.n1, L.n2);
+                                dmin = Ar<R>::min(d, dmin);
+                                // 2 s g <= d + Ei
+                                const float gf = (float)g;
+                                const float s1 = Ar<R>::to_f32_up(Ar<R>::add_up(d, L.Ei)) * Ar<float>::rcp(fabsf(gf));
+                                if (gf > 0.0f) hi = fminf(hi, s1);
+                                else nlo = fminf(nlo, s1);
+                                // empty: hi and nlo are at most 2 S, and one below -4 S empties the interval
+                                // whatever its rounding, so the two errors are below c / 2
+                                if (hi + nlo < -c) {
+                                    n_tri -= __popc(b);
+                                    b = 0u;
+                                    alive = false;
+                                }
+                            }
+                            if (!alive) break;
+                        }
+                        if (alive) {
+                            pass = dmin > L.E;
+                            pend = !pass && !(dmin < -L.E);
+                            hi += c;
+                            nlo += c;
+                        }
+                    }
+                    pend = pend || (valid && L.ac3 == 0);
+                    __syncwarp();
+                    // tetrahedra (i,p,k,x), x above k: AC3 on the line, and of those in
+                    // Sigma^3 the ones whose orthocentre may be an end of the interval
+#pragma unroll 1
+                    for (int w = r0 >> 5; w < nu; w++) {  // kk >= r0
+                        unsigned b = L.ac3 >= 0 ? S.Mrow[pp][w] & S.Mrow[kk][w] & above_mask(w, kk) & ~above_mask(w, n_up - 1) : 0u;
+                        n_ac3k += __popc(b);
+                        unsigned in3 = 0u, out3 = ~b;  // x with AC3 decided
+                        while (b) {
+                            const int e = first_pos(b);
+                            const unsigned bit = pos_bit(e);
+                            b ^= bit;
+                            const P4<R> v = point<R>(S, 32 * w + e);
+                            const R ad = Ar<R>::abs(delta(v, L.z0, L.z1, L.z2));
+                            const R ag = Ar<R>::abs(dot3(v, L.n0, L.n1, L.n2));
+                            if (ad < Ar<R>::fma_dn(ag, L.s2lo, -L.Ei)) in3 |= bit;
+                            if (ad > Ar<R>::fma_up(ag, R(L.s2), L.Ei)) out3 |= bit;
+                        }
+                        n_s3 += __popc(in3);
+                        for (unsigned o = ~(in3 | out3); o;) {
+                            const int e = first_pos(o);
+                            o ^= pos_bit(e);
+                            push_tet(pp, kk, 32 * w + e, true);
+                        }
+                        for (unsigned o = alive ? in3 & S.kup[w] : 0u; o;) {
+                            const int e = first_pos(o), x = 32 * w + e;
+                            o ^= pos_bit(e);
+                            const P4<R> v = point<R>(S, x);
+                            const R d = delta(v, L.z0, L.z1, L.z2);
+                            const R g = dot3(v, L.n0, L.n1, L.n2);
+                            const R far = Ar<R>::max(Ar<R>::mul(R(hi), g), -Ar<R>::mul(R(nlo), g));
+                            if (!(Ar<R>::add_up(d, -far) > R(1.5) * L.Ei)) push_tet(pp, kk, x, false);
+                        }
+                        if (keep) {
+                            int tot3;
+                            const int first = warp_excl(lane, __popc(in3), &tot3);
+                            unsigned long long at = 0;
+                            if (lane == 0 && tot3 > 0) at = atomicAdd(&cnt->n_cand_out[3], (unsigned long long)tot3);
+                            at = __shfl_sync(FULL, at, 0) + first;
+                            for (unsigned o = in3; o; at++) {
+                                const int e = first_pos(o);
+                                o ^= pos_bit(e);
+                                if ((int64_t)at < A.cap_cand[3])
+                                    A.cand3[at] = make_int4(i, S.idx[pp], S.idx[kk], S.idx[32 * w + e]);
+                                else atomicOr(&cnt->err, DERR_OVF_CAND);
                             }
                         }
                     }
-                    {
-                        const int r2 = keep_it ? ac2_scan<R>(S, nw, o, B, 2, pp, kk, 0, n_tri) : 1;
-                        if (keep_it) {
-                            pass = r2 > 0;
-                            pend = r2 == 0;
-                        }
-                    }
-                    {
-                        // list the pair for the tetrahedron phase (the triangle is potential or undecided)
-                        const bool tp = valid && (keep_it || pend_ac3);
-                        const unsigned bt = __ballot_sync(FULL, tp);
-                        const int slot = S.n_pl + __popc(bt & lanemask_lt());
-                        if (tp && slot < PL_CAP) S.plist[slot] = (typename SM::Pair)(pp | (kk << SM::SH));
-                        __syncwarp();
-                        if (lane == 0) S.n_pl += __popc(bt);
-                        __syncwarp();
-                    }
+                    __syncwarp();
                     const int4 item = make_int4(i, valid ? S.idx[pp] : 0, valid ? S.idx[kk] : 0, 0);
                     if (keep)
                         append_direct(keep_it, item, A.cand2, &cnt->n_cand_out[2], A.cap_cand[2], &cnt->err,
                                       DERR_OVF_CAND);
-                    append_direct(pend, make_int4(pend_ac3 ? ~i : i, item.y, item.z, -1), A.pending, &cnt->n_pending,
+                    append_direct(pend, make_int4(L.ac3 == 0 ? ~i : i, item.y, item.z, -1), A.pending, &cnt->n_pending,
                                   A.cap_pending, &cnt->err, DERR_OVF_PEND);
                     stage_push(lane, pass, item, S.st_tri, &S.n_tri, A.tri_out, &cnt->n_tri_pass, A.cap_tri, &cnt->err,
                                DERR_OVF_TRI);
                 }
                 __syncwarp();
             }
-        }
-        __syncwarp();
-
-        // ---- phase D: tetrahedra (i,p,k,l): AC3, then AC2 ----------------------
-        // Sigma^2 pairs (p,k) come from the list the triangle phase wrote (or,
-        // when it overflowed, from the T rows: row r of up holds popc(T[p]) of
-        // them, located by a prefix and a binary search). Pairs are taken
-        // PAIR_CHUNK at a time with a prefix over their candidate counts
-        // popc(T[p] & T[k]); their candidates l are written as codes
-        // p | k << SH | l << 2 SH to cand[] (CAND_CAP per batch) and read back by
-        // windows of 32.
-        const bool use_list = S.n_pl <= PL_CAP;
-        if (!use_list) {
-            int run = 0;
-            for (int r0 = 0; r0 < n_up; r0 += 32) {
-                int c = 0;
-                if (r0 + lane < n_up) {
-                    const int p = S.uplist[r0 + lane];
-                    for (int w = 0; w < nw; w++) c += __popc(S.Trow[p][w]);
-                }
-                int tot;
-                const int ex = warp_excl(lane, c, &tot);
-                if (r0 + lane < n_up) S.rowpre[r0 + lane] = run + ex;
-                run += tot;
-            }
-            if (lane == 0) S.rowpre[n_up] = run;
-        }
-        __syncwarp();
-        const int n_pairs = use_list ? S.n_pl : S.rowpre[n_up];
-        // pair j of the enumeration: from the list, or located in the T rows
-        auto pair_code = [&](int j) -> unsigned {
-            if (use_list) return S.plist[j];
-            const int r = row_of(S.rowpre, n_up, j);
-            const int p = S.uplist[r];
-            const int k = nth_in_words(nw, j - S.rowpre[r], [&](int w) { return S.Trow[p][w]; });
-            return (unsigned)(p | (k << SM::SH));
-        };
-        // AC3 then AC2 for the batch of candidate codes in cand[0, nbatch), 32 per window
-        auto tet_windows = [&](int nbatch) {
-#pragma unroll 1
-            for (int base = 0; base < nbatch; base += 32) {
-                const int j = base + lane;
-                const bool valid = j < nbatch;
-                bool pass = false, pend = false, keep_it = false;
-                int pend_ac3 = 0;
-                int p3 = 0, k3 = 0, ll = 0;
-                Ortho<R> o;
-                o.ac3 = -1;
-                if (valid) {
-                    const unsigned code = S.cand[j];
-                    p3 = code & SM::PM;
-                    k3 = (code >> SM::SH) & SM::PM;
-                    ll = code >> (2 * SM::SH);
-                    n_ac3k++;
-                    o = ortho_tet<R>(point<R>(S, p3), point<R>(S, k3), point<R>(S, ll), T, B);
-                    if (o.ac3 > 0) {
-                        n_s3++;
-                        keep_it = true;
-                    } else if (o.ac3 == 0) {
-                        pend = true;
-                        pend_ac3 = 1;
-                    }
-                }
-                {
-                    const int r3 = keep_it ? ac2_scan<R>(S, nw, o, B, 3, p3, k3, ll, n_tet) : 1;
-                    if (keep_it) {
-                        pass = r3 > 0;
-                        pend = r3 == 0;
-                    }
-                }
-                const int4 item = make_int4(i, valid ? S.idx[p3] : 0, valid ? S.idx[k3] : 0, valid ? S.idx[ll] : 0);
-                if (keep)
-                    append_direct(keep_it, item, A.cand3, &cnt->n_cand_out[3], A.cap_cand[3], &cnt->err,
-                                  DERR_OVF_CAND);
-                append_direct(pend, make_int4(pend_ac3 ? ~i : i, item.y, item.z, item.w), A.pending, &cnt->n_pending,
-                              A.cap_pending, &cnt->err, DERR_OVF_PEND);
-                stage_push(lane, pass, item, S.st_tet, &S.n_tet, A.tet_out, &cnt->n_tet_out, A.cap_tet, &cnt->err,
-                           DERR_OVF_TET);
-            }
-            __syncwarp();
-        };
-        if constexpr (WORDS <= 2) {
-            // narrow rows: a lane takes PAIRS_PER_LANE consecutive pairs and keeps their
-            // candidate masks T[p] & T[k] in registers; a prefix over the lanes places
-            // its candidates in enumeration order
-            constexpr int PPL = 2;
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_pairs; c0 += 32 * PPL) {
-                unsigned code[PPL], mk0[PPL], mk1[PPL];
-                int mine = 0;
-#pragma unroll
-                for (int t = 0; t < PPL; t++) {
-                    const int j = c0 + PPL * lane + t;
-                    code[t] = 0u;
-                    mk0[t] = mk1[t] = 0u;
-                    if (j < n_pairs) {
-                        code[t] = pair_code(j);
-                        const int p = code[t] & SM::PM, k = code[t] >> SM::SH;
-                        mk0[t] = S.Trow[p][0] & S.Trow[k][0];
-                        if (WORDS > 1) mk1[t] = S.Trow[p][WORDS - 1] & S.Trow[k][WORDS - 1];
-                        mine += __popc(mk0[t]) + __popc(mk1[t]);
-                    }
-                }
-                int total;
-                const int ex = warp_excl(lane, mine, &total);
-#pragma unroll 1
-                for (int done = 0; done < total; done += CAND_CAP) {
-                    if (ex < done + CAND_CAP && ex + mine > done) {
-                        int t = ex;
-#pragma unroll
-                        for (int u = 0; u < PPL; u++) {
-#pragma unroll
-                            for (int w = 0; w < WORDS; w++) {
-                                unsigned b = w == 0 ? mk0[u] : mk1[u];
-                                while (b) {
-                                    const int l = 32 * w + __ffs(b) - 1;
-                                    b &= b - 1;
-                                    if (t >= done && t < done + CAND_CAP)
-                                        S.cand[t - done] = code[u] | ((unsigned)l << (2 * SM::SH));
-                                    t++;
-                                }
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    tet_windows(min(CAND_CAP, total - done));
-                }
-            }
-        } else {
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_pairs; c0 += PAIR_CHUNK) {
-                const int cn = min(PAIR_CHUNK, n_pairs - c0);
-                {
-                    int run = 0;
-                    for (int q0 = 0; q0 < cn; q0 += 32) {
-                        int c = 0;
-                        if (q0 + lane < cn) {
-                            const unsigned code = pair_code(c0 + q0 + lane);
-                            const int p = code & SM::PM, k = code >> SM::SH;
-                            if (!use_list) S.plist[q0 + lane] = (typename SM::Pair)code;  // chunk-local copy
-                            for (int w = 0; w < nw; w++) c += __popc(S.Trow[p][w] & S.Trow[k][w]);
-                        }
-                        int tot;
-                        const int ex = warp_excl(lane, c, &tot);
-                        if (q0 + lane < cn) S.pairpre[q0 + lane] = run + ex;
-                        run += tot;
-                    }
-                    if (lane == 0) S.pairpre[cn] = run;
-                }
-                __syncwarp();
-                const int total = S.pairpre[cn];
-#pragma unroll 1
-                for (int done = 0; done < total; done += CAND_CAP) {
-                    for (int q = lane; q < cn; q += 32) {
-                        const int a0 = S.pairpre[q], a1 = S.pairpre[q + 1];
-                        if (a1 <= done || a0 >= done + CAND_CAP) continue;
-                        const unsigned code = S.plist[(use_list ? c0 : 0) + q];
-                        const int p = code & SM::PM, k = code >> SM::SH;
-                        int t = a0;
-                        for (int w = 0; w < nw; w++) {
-                            unsigned b = S.Trow[p][w] & S.Trow[k][w];
-                            while (b) {
-                                const int l = 32 * w + __ffs(b) - 1;
-                                b &= b - 1;
-                                if (t >= done && t < done + CAND_CAP) S.cand[t - done] = code | ((unsigned)l << (2 * SM::SH));
-                                t++;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    tet_windows(min(CAND_CAP, total - done));
-                }
-            }
-        }
-
-        // ---- phase E: edges (i,p): AC2 at the edge's orthocentre ---------------
-        for (int r0 = 0; r0 < n_up; r0 += 32) {
-            const bool ok = r0 + lane < n_up;
-            const int p = ok ? S.uplist[r0 + lane] : 0;
-            bool pass = false, pend = false;
-            Ortho<R> o;
-            o.ac3 = -1;
-            if (ok) o = ortho_edge<R>(point<R>(S, p), B);
-            {
-                const int r1 = ok ? ac2_scan<R>(S, nw, o, B, 1, p, 0, 0, n_edge) : 1;
-                if (ok) {
-                    pass = r1 > 0;
-                    pend = r1 == 0;
-                }
-            }
-            const int idp = ok ? S.idx[p] : 0;
-            append_direct(pend, make_int4(i, idp, -1, -1), A.pending, &cnt->n_pending, A.cap_pending, &cnt->err,
-                          DERR_OVF_PEND);
-            stage_push(lane, pass, make_int2(i, idp), S.st_edge, &S.n_edge, A.edge_out, &cnt->n_edge_pass, A.cap_edge,
-                       &cnt->err, DERR_OVF_EDGE);
+            settle_tets();
         }
         __syncwarp();
     }
@@ -1514,8 +1519,11 @@ static void set_bounds(double u, double h, int64_t wmax, Bounds<R>& b) {
     b.eG = up(g3 * H * H * slack);
     b.eDet = up(15.01 * u * H * H * H * H * slack);
     b.cn = up(6.01 * u * H * H * slack);
-    b.K0 = up((u * Am + 2 * g3 * H * h) * slack);
+    b.K0 = up((u * Am + g3 * (Am + 2 * H * h)) * slack);
     b.K1 = up(2 * s3 * H * (1 + g3) * slack);
+    b.K2 = up(s3 * H * eC * slack);
+    b.K3 = up(12 * u * H * h * slack);
+    b.inv_lo = (R)(1.0 - 64.0 * u);
     b.k2 = up((delta_r + u) * 1.01);
     b.ky = up(2.0001 * u);
     b.ke = up(1.0001 * u);
@@ -1528,6 +1536,7 @@ static void set_bounds(double u, double h, int64_t wmax, Bounds<R>& b) {
 static void set_constants(const PredConst& pc, int64_t wmax, LocalArgs& a) {
     const double h = pc.h_d, H = 2.0 * h;
     set_bounds<float>(ldexp(1.0, -24), h, wmax, a.b32);
+    a.perp_err = (float)(64.0 * ldexp(1.0, -24) * H * H);
     set_bounds<double>(ldexp(1.0, -53), h, wmax, a.b64);
     // resolve kernel: y from exact minors with relative error <= 4.0001 u64 per component
     const double v = ldexp(1.0, -53), g3d = 3 * v / (1 - 3 * v), dy = 4.0001 * v, sf = 1.0 + 16 * v;
