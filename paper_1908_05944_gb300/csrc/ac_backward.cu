@@ -23,54 +23,57 @@ namespace ac {
 struct Ortho {
     double lam[4];
     double c[3];
-    double value;
 };
 
-// Orthocentre, barycentric coordinates and OrthoSize of K vertices (global input
-// indices, ascending) from FP64 centres (n x 3) and radii.
-__device__ Ortho ortho_fp64(const double* __restrict__ X, const double* __restrict__ R, const int4& t, int K) {
+// Orthocentre and barycentric coordinates of K vertices (global input indices,
+// ascending) from FP64 centres (n x 3) and radii. A tetrahedron's come from the
+// cross products of its edge vectors (y = N / 2D, lambda_k = C_k . y / D): about
+// 80 FP64 operations, and a condition number the Gram matrix would square.
+template <int K>
+__device__ __forceinline__ Ortho ortho_fp64(const double* __restrict__ X, const double* __restrict__ R, const int4& t) {
     Ortho o;
     const int v[4] = {t.x, t.y, t.z, t.w};
     const double p0[3] = {X[3 * v[0]], X[3 * v[0] + 1], X[3 * v[0] + 2]};
     const double w0 = R[v[0]] * R[v[0]];
-    double q[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, a[3] = {0, 0, 0};
+    double q[3][3], a[3], mu[3] = {0.0, 0.0, 0.0}, y[3] = {0.0, 0.0, 0.0}, g[3];
+#pragma unroll
     for (int k = 1; k < K; k++) {
-        double wk = R[v[k]] * R[v[k]];
+        const double rk = R[v[k]];
         for (int c = 0; c < 3; c++) q[k - 1][c] = X[3 * v[k] + c] - p0[c];
-        a[k - 1] = q[k - 1][0] * q[k - 1][0] + q[k - 1][1] * q[k - 1][1] + q[k - 1][2] * q[k - 1][2] - wk + w0;
+        g[k - 1] = q[k - 1][0] * q[k - 1][0] + q[k - 1][1] * q[k - 1][1] + q[k - 1][2] * q[k - 1][2];
+        a[k - 1] = g[k - 1] - rk * rk + w0;
     }
-    const int d = K - 1;
-    double G[3][3];
-    for (int i = 0; i < d; i++)
-        for (int j = 0; j < d; j++) G[i][j] = q[i][0] * q[j][0] + q[i][1] * q[j][1] + q[i][2] * q[j][2];
-    double mu[3] = {0, 0, 0};
-    if (d == 1) {
-        mu[0] = a[0] / (2.0 * G[0][0]);
-    } else if (d == 2) {
-        double det = G[0][0] * G[1][1] - G[0][1] * G[1][0];
-        mu[0] = (G[1][1] * a[0] - G[0][1] * a[1]) / (2.0 * det);
-        mu[1] = (G[0][0] * a[1] - G[1][0] * a[0]) / (2.0 * det);
-    } else if (d == 3) {
-        double adj[3][3];
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) {
-                int r0 = (i + 1) % 3, r1 = (i + 2) % 3, c0 = (j + 1) % 3, c1 = (j + 2) % 3;
-                adj[j][i] = G[r0][c0] * G[r1][c1] - G[r0][c1] * G[r1][c0];
-            }
-        double det = G[0][0] * adj[0][0] + G[0][1] * adj[1][0] + G[0][2] * adj[2][0];
-        for (int i = 0; i < 3; i++) mu[i] = (adj[i][0] * a[0] + adj[i][1] * a[1] + adj[i][2] * a[2]) / (2.0 * det);
+    if constexpr (K == 2) {
+        mu[0] = a[0] / (2.0 * g[0]);
+        for (int c = 0; c < 3; c++) y[c] = mu[0] * q[0][c];
+    } else if constexpr (K == 3) {
+        const double g12 = q[0][0] * q[1][0] + q[0][1] * q[1][1] + q[0][2] * q[1][2];
+        const double r = 0.5 / (g[0] * g[1] - g12 * g12);
+        mu[0] = (g[1] * a[0] - g12 * a[1]) * r;
+        mu[1] = (g[0] * a[1] - g12 * a[0]) * r;
+        for (int c = 0; c < 3; c++) y[c] = mu[0] * q[0][c] + mu[1] * q[1][c];
+    } else if constexpr (K == 4) {
+        double C[3][3], N[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const double* b = q[(k + 1) % 3];
+            const double* e = q[(k + 2) % 3];
+            C[k][0] = b[1] * e[2] - b[2] * e[1];
+            C[k][1] = b[2] * e[0] - b[0] * e[2];
+            C[k][2] = b[0] * e[1] - b[1] * e[0];
+        }
+        const double r = 1.0 / (q[0][0] * C[0][0] + q[0][1] * C[0][1] + q[0][2] * C[0][2]);
+        for (int c = 0; c < 3; c++) N[c] = a[0] * C[0][c] + a[1] * C[1][c] + a[2] * C[2][c];
+        for (int c = 0; c < 3; c++) y[c] = 0.5 * r * N[c];
+        for (int k = 0; k < 3; k++) mu[k] = (C[k][0] * y[0] + C[k][1] * y[1] + C[k][2] * y[2]) * r;
     }
-    double y[3] = {0, 0, 0};
-    for (int k = 0; k < d; k++)
-        for (int c = 0; c < 3; c++) y[c] += mu[k] * q[k][c];
     double s = 1.0;
-    for (int k = 0; k < d; k++) {
+    for (int k = 0; k < K - 1; k++) {
         o.lam[k + 1] = mu[k];
         s -= mu[k];
     }
     o.lam[0] = s;
     for (int c = 0; c < 3; c++) o.c[c] = p0[c] + y[c];
-    o.value = y[0] * y[0] + y[1] * y[1] + y[2] * y[2] - w0;
     return o;
 }
 
@@ -91,13 +94,17 @@ __device__ __forceinline__ dd two_sum(double a, double b) {
     return {s, e};
 }
 
+// the same for |a| >= |b| (Dekker's FastTwoSum)
+__device__ __forceinline__ dd fast_two_sum(double a, double b) {
+    double s = a + b;
+    return {s, b - (s - a)};
+}
+
 __device__ __forceinline__ dd dd_add(dd a, dd b) {
     dd s = two_sum(a.hi, b.hi);
     dd t = two_sum(a.lo, b.lo);
-    s.lo += t.hi;
-    s = two_sum(s.hi, s.lo);
-    s.lo += t.lo;
-    return two_sum(s.hi, s.lo);
+    s = fast_two_sum(s.hi, s.lo + t.hi);
+    return fast_two_sum(s.hi, s.lo + t.lo);
 }
 
 __device__ __forceinline__ dd dd_neg(dd a) { return {-a.hi, -a.lo}; }
@@ -105,55 +112,62 @@ __device__ __forceinline__ dd dd_neg(dd a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ dd dd_sub(dd a, dd b) { return dd_add(a, dd_neg(b)); }
 
 __device__ __forceinline__ dd dd_mul(dd a, dd b) {
-    double p = a.hi * b.hi;
-    double e = fma(a.hi, b.hi, -p);
-    e += a.hi * b.lo + a.lo * b.hi;
-    return two_sum(p, e);
+    const double p = a.hi * b.hi;
+    return fast_two_sum(p, fma(a.lo, b.hi, fma(a.hi, b.lo, fma(a.hi, b.hi, -p))));
 }
 
+__device__ __forceinline__ dd dd_sqr(dd a) {
+    const double p = a.hi * a.hi;
+    return fast_two_sum(p, fma(2.0 * a.hi, a.lo, fma(a.hi, a.hi, -p)));
+}
+
+// a (a double) times b
+__device__ __forceinline__ dd dd_scale(double a, dd b) {
+    const double p = a * b.hi;
+    return fast_two_sum(p, fma(a, b.lo, fma(a, b.hi, -p)));
+}
+
+// three quotient digits, each from the remainder of the ones before (one reciprocal)
 __device__ __forceinline__ dd dd_div(dd a, dd b) {
-    double q1 = a.hi / b.hi;
-    dd r = dd_sub(a, dd_mul(b, dd_from(q1)));
-    double q2 = r.hi / b.hi;
-    r = dd_sub(r, dd_mul(b, dd_from(q2)));
-    double q3 = r.hi / b.hi;
-    dd q = two_sum(q1, q2);
-    return dd_add(q, dd_from(q3));
+    const double r = 1.0 / b.hi;
+    const double q1 = a.hi * r;
+    dd e = dd_sub(a, dd_scale(q1, b));
+    const double q2 = e.hi * r;
+    e = dd_sub(e, dd_scale(q2, b));
+    return dd_add(fast_two_sum(q1, q2), dd_from(e.hi * r));
 }
 
-// OrthoSize of K vertices from FP64 centres/radii, evaluated in double-double.
-__device__ double orthosize_dd(const double* __restrict__ X, const double* __restrict__ R, const int4& t, int K) {
+// OrthoSize of K vertices from FP64 centres/radii, evaluated in double-double:
+// about 1,100 FP64 operations for a tetrahedron, 530 for a triangle, 210 for an edge.
+template <int K>
+__device__ __forceinline__ double orthosize_dd(const double* __restrict__ X, const double* __restrict__ R, const int4& t) {
     const int v[4] = {t.x, t.y, t.z, t.w};
-    const dd r0 = dd_from(R[v[0]]);
-    const dd w0 = dd_mul(r0, r0);
-    if (K == 1) return -w0.hi;
-    dd q[3][3], a[3];
-    for (int k = 1; k < K; k++) {
-        const dd rk = dd_from(R[v[k]]);
-        dd sq = dd_from(0.0);
-        for (int c = 0; c < 3; c++) {
-            q[k - 1][c] = two_sum(X[3 * v[k] + c], -X[3 * v[0] + c]);
-            sq = dd_add(sq, dd_mul(q[k - 1][c], q[k - 1][c]));
-        }
-        a[k - 1] = dd_add(dd_sub(sq, dd_mul(rk, rk)), w0);
-    }
+    const dd w0 = dd_sqr(dd_from(R[v[0]]));
+    if constexpr (K == 1) return -w0.hi;
+    dd q[3][3], g[3], a[3];
+    const double p0[3] = {X[3 * v[0]], X[3 * v[0] + 1], X[3 * v[0] + 2]};
     auto dot = [](const dd* x, const dd* y) {
         return dd_add(dd_add(dd_mul(x[0], y[0]), dd_mul(x[1], y[1])), dd_mul(x[2], y[2]));
     };
-    dd num, den;
-    if (K == 2) {
-        dd D = dot(q[0], q[0]);
-        num = dd_mul(a[0], a[0]);
-        den = dd_mul(dd_from(4.0), D);
-    } else if (K == 3) {
-        dd g11 = dot(q[0], q[0]), g22 = dot(q[1], q[1]), g12 = dot(q[0], q[1]);
-        dd det = dd_sub(dd_mul(g11, g22), dd_mul(g12, g12));
-        dd n1 = dd_sub(dd_mul(g22, a[0]), dd_mul(g12, a[1]));
-        dd n2 = dd_sub(dd_mul(g11, a[1]), dd_mul(g12, a[0]));
+#pragma unroll
+    for (int k = 1; k < K; k++) {
+        for (int c = 0; c < 3; c++) q[k - 1][c] = two_sum(X[3 * v[k] + c], -p0[c]);
+        g[k - 1] = dd_add(dd_add(dd_sqr(q[k - 1][0]), dd_sqr(q[k - 1][1])), dd_sqr(q[k - 1][2]));
+        a[k - 1] = dd_add(dd_sub(g[k - 1], dd_sqr(dd_from(R[v[k]]))), w0);
+    }
+    dd num = dd_from(0.0), den = dd_from(1.0);
+    if constexpr (K == 2) {
+        num = dd_sqr(a[0]);
+        den = g[0];
+    } else if constexpr (K == 3) {
+        const dd g12 = dot(q[0], q[1]);
+        const dd n1 = dd_sub(dd_mul(g[1], a[0]), dd_mul(g12, a[1]));
+        const dd n2 = dd_sub(dd_mul(g[0], a[1]), dd_mul(g12, a[0]));
         num = dd_add(dd_mul(n1, a[0]), dd_mul(n2, a[1]));
-        den = dd_mul(dd_from(4.0), det);
-    } else {
+        den = dd_sub(dd_mul(g[0], g[1]), dd_sqr(g12));
+    } else if constexpr (K == 4) {
         dd C[3][3];
+#pragma unroll
         for (int k = 0; k < 3; k++) {
             const dd* b = q[(k + 1) % 3];
             const dd* e = q[(k + 2) % 3];
@@ -161,14 +175,15 @@ __device__ double orthosize_dd(const double* __restrict__ X, const double* __res
             C[k][1] = dd_sub(dd_mul(b[2], e[0]), dd_mul(b[0], e[2]));
             C[k][2] = dd_sub(dd_mul(b[0], e[1]), dd_mul(b[1], e[0]));
         }
-        dd D = dot(q[0], C[0]);
-        dd N[3];
-        for (int c = 0; c < 3; c++)
-            N[c] = dd_add(dd_add(dd_mul(a[0], C[0][c]), dd_mul(a[1], C[1][c])), dd_mul(a[2], C[2][c]));
-        num = dot(N, N);
-        den = dd_mul(dd_from(4.0), dd_mul(D, D));
+        den = dd_sqr(dot(q[0], C[0]));
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const dd N = dd_add(dd_add(dd_mul(a[0], C[0][c]), dd_mul(a[1], C[1][c])), dd_mul(a[2], C[2][c]));
+            num = c == 0 ? dd_sqr(N) : dd_add(num, dd_sqr(N));
+        }
     }
-    dd f = dd_sub(dd_div(num, den), w0);
+    const dd y2 = dd_div(num, den);  // 4 |y|^2: scaling by 1/4 is exact
+    const dd f = dd_sub(dd{0.25 * y2.hi, 0.25 * y2.lo}, w0);
     return f.hi + f.lo;
 }
 
@@ -245,14 +260,67 @@ int eval_filtration_f32(ac_ctx* c, float* const f_out[4], cudaStream_t s) {
     return AC_OK;
 }
 
-__global__ void k_eval(const double* __restrict__ X, const double* __restrict__ R, const int8_t* __restrict__ sdim,
-                       const int64_t* __restrict__ sidx, int64_t m, const int4* const* __restrict__ G,
-                       double* __restrict__ out) {
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    const int d = sdim[j];
-    const int4 t = G[d][sidx[j]];
-    out[j] = orthosize_dd(X, R, t, d + 1);
+// The values at moved atoms, each source evaluated once: a row that is its own
+// source (unattached) by its double-double OrthoSize, then every attached row a
+// copy of its source's value. The FP64 pipe (2 lanes per clock and SM) bounds
+// it, and takes as long for a warp with one active lane as for a full one:
+// a block gathers the unattached rows of EVAL_TILE rows and evaluates those.
+constexpr int EVAL_THREADS = 128;
+constexpr int EVAL_TILE = 512;
+
+// indices (from first) of the rows of a tile with !skip(row), in no particular order
+template <class F>
+__device__ __forceinline__ int gather_rows(int64_t first, int64_t m, int* list, int* n_list, F&& skip) {
+    if (threadIdx.x == 0) *n_list = 0;
+    __syncthreads();
+    for (int u = threadIdx.x; u < EVAL_TILE; u += EVAL_THREADS) {
+        const bool take = first + u < m && !skip(first + u);
+        const unsigned b = __ballot_sync(0xffffffffu, take);
+        int base = 0;
+        if ((threadIdx.x & 31) == 0 && b) base = atomicAdd(n_list, __popc(b));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (take) list[base + __popc(b & ((1u << (threadIdx.x & 31)) - 1u))] = u;
+    }
+    __syncthreads();
+    return *n_list;
+}
+
+template <int K>
+__global__ void __launch_bounds__(EVAL_THREADS) k_eval_own(const double* __restrict__ X, const double* __restrict__ R,
+                                                           const int4* __restrict__ G,
+                                                           const uint8_t* __restrict__ attached, int64_t m,
+                                                           double* __restrict__ out) {
+    __shared__ int list[EVAL_TILE];
+    __shared__ int n_list;
+    const int64_t first = (int64_t)blockIdx.x * EVAL_TILE;
+    const int n = gather_rows(first, m, list, &n_list, [&](int64_t j) { return attached[j] != 0; });
+    for (int u = threadIdx.x; u < n; u += EVAL_THREADS) {
+        const int64_t j = first + list[u];
+        out[j] = orthosize_dd<K>(X, R, G[j]);
+    }
+}
+
+struct Vals4 {
+    const double* v[4];
+};
+
+__global__ void k_eval_attached(const uint8_t* __restrict__ attached, const int8_t* __restrict__ sdim,
+                                const int64_t* __restrict__ sidx, int64_t m, Vals4 vals, double* __restrict__ out) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < m && attached[j]) out[j] = vals.v[sdim[j]][sidx[j]];
+}
+
+template <int K>
+__device__ __forceinline__ void add_gradient(const double* __restrict__ X, const double* __restrict__ R, const int4& t,
+                                             double w, double* __restrict__ dX, double* __restrict__ dR) {
+    const Ortho o = ortho_fp64<K>(X, R, t);
+    const int v[4] = {t.x, t.y, t.z, t.w};
+    for (int k = 0; k < K; k++) {
+        const int a = v[k];
+        const double l2 = 2.0 * w * o.lam[k];
+        for (int c = 0; c < 3; c++) atomicAdd(&dX[3 * a + c], l2 * (X[3 * a + c] - o.c[c]));
+        atomicAdd(&dR[a], -l2 * R[a]);
+    }
 }
 
 __global__ void k_backward(const double* __restrict__ X, const double* __restrict__ R, const int8_t* __restrict__ sdim,
@@ -264,32 +332,45 @@ __global__ void k_backward(const double* __restrict__ X, const double* __restric
     if (wj == 0.0) return;
     const int d = sdim[j];
     const int4 t = G[d][sidx[j]];
-    const Ortho o = ortho_fp64(X, R, t, d + 1);
-    const int v[4] = {t.x, t.y, t.z, t.w};
-    for (int k = 0; k <= d; k++) {
-        const int a = v[k];
-        const double l2 = 2.0 * wj * o.lam[k];
-        for (int c = 0; c < 3; c++) atomicAdd(&dX[3 * a + c], l2 * (X[3 * a + c] - o.c[c]));
-        atomicAdd(&dR[a], -l2 * R[a]);
-    }
-}
-
-static int gtable(ac_ctx* c, DevBuf& tab, cudaStream_t s) {
-    const int4* h[4];
-    for (int d = 0; d < 4; d++) h[d] = c->Gbuf[d].as<int4>();
-    AC_TRY(tab.reserve(sizeof(h), s));
-    AC_CUDA(cudaMemcpyAsync(tab.p, h, sizeof(h), cudaMemcpyHostToDevice, s));
-    return AC_OK;
+    if (d == 0) add_gradient<1>(X, R, t, wj, dX, dR);
+    else if (d == 1) add_gradient<2>(X, R, t, wj, dX, dR);
+    else if (d == 2) add_gradient<3>(X, R, t, wj, dX, dR);
+    else add_gradient<4>(X, R, t, wj, dX, dR);
 }
 
 int eval_filtration(ac_ctx* c, const double* centres, const double* radii, double* const f_out[4], cudaStream_t s) {
-    AC_TRY(gtable(c, c->scratch[5], s));
-    for (int d = 0; d < 4; d++) {
+    // a dimension nobody asked for is evaluated into scratch where a lower one may take values from it
+    int lo = 4;
+    size_t extra = 0, off[4] = {0, 0, 0, 0};
+    for (int d = 3; d >= 0; d--)
+        if (f_out[d] && c->K[d].count > 0) lo = d;
+    for (int d = lo; d < 4; d++)
+        if (!f_out[d]) {
+            off[d] = extra;
+            extra += (size_t)c->K[d].count;
+        }
+    AC_TRY(c->scratch[5].reserve((extra > 0 ? extra : 1) * sizeof(double), s));
+    double* val[4] = {nullptr, nullptr, nullptr, nullptr};
+    Vals4 vals{};
+    for (int d = lo; d < 4; d++) {
+        val[d] = f_out[d] ? f_out[d] : c->scratch[5].as<double>() + off[d];
+        vals.v[d] = val[d];
+    }
+    for (int d = 3; d >= lo; d--) {
+        const int64_t m = c->K[d].count;
+        if (m == 0) continue;
+        void (*k)(const double*, const double*, const int4*, const uint8_t*, int64_t, double*) =
+            d == 3 ? k_eval_own<4> : d == 2 ? k_eval_own<3> : d == 1 ? k_eval_own<2> : k_eval_own<1>;
+        k<<<(unsigned)((m + EVAL_TILE - 1) / EVAL_TILE), EVAL_THREADS, 0, s>>>(
+            centres, radii, c->Gbuf[d].as<int4>(), c->K[d].attached.as<uint8_t>(), m, val[d]);
+        AC_LAUNCHED();
+    }
+    for (int d = lo; d < 3; d++) {  // a tetrahedron is never attached
         const int64_t m = c->K[d].count;
         if (!f_out[d] || m == 0) continue;
-        k_eval<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(centres, radii, c->K[d].src_dim.as<int8_t>(),
-                                                           c->K[d].src_idx.as<int64_t>(), m,
-                                                           c->scratch[5].as<const int4*>(), f_out[d]);
+        k_eval_attached<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(c->K[d].attached.as<uint8_t>(),
+                                                                    c->K[d].src_dim.as<int8_t>(),
+                                                                    c->K[d].src_idx.as<int64_t>(), m, vals, f_out[d]);
         AC_LAUNCHED();
     }
     AC_CUDA(cudaStreamSynchronize(s));
@@ -311,15 +392,21 @@ int eval_filtration(ac_ctx* c, const double* centres, const double* radii, doubl
 //      w(sigma) + the W' of the attached facets whose parent sigma is, in
 //      facet order. An unattached row's W' is its W_s; an attached row hands
 //      its W' up and is no source.
-//   2. k_contrib, one thread per unattached row with W_s != 0: the
-//      orthocentre and barycentric coordinates of s, and for each vertex k of
-//      s the contribution (2 W_s lambda_k (p_k - c), -2 W_s lambda_k r_k).
-//   3. k_gather_atoms, one warp per atom a: the contributions of the rows
-//      containing a, summed per lane and then over the lanes by a fixed tree.
-//      Every vertex of a simplex of the complex has a grown ball meeting a's,
-//      so the first (smallest) vertex of a row containing a is a or one of
-//      a's neighbours with a smaller input index: lane t takes neighbour t
-//      (and lane 0 a itself first), every list, every row of that first vertex.
+//   2. k_contrib, the unattached rows: the orthocentre and barycentric
+//      coordinates of s, and for each vertex k of s the contribution
+//      (2 W_s lambda_k (p_k - c), -2 W_s lambda_k r_k).
+//   3. k_edge_sums, eight lanes per atom b: of the rows with first vertex b, the
+//      contributions to b itself, and to each other vertex x. Such an x is the
+//      second vertex of a K^1 row with first vertex b, and its sum is written
+//      there (lane by lane in row order, so the order is fixed).
+//   4. k_gather_atoms, eight lanes per atom a: its own sum and those of the K^1
+//      rows (b, a), b the neighbours of a with a smaller input index (their grown
+//      balls meet), each found by a binary search among b's rows; summed per lane
+//      and then over the lanes by a fixed tree.
+// Without 3. every atom read all the rows of those neighbours (600 rows for the
+// 27 that hold it): 1.65 ms for the 100,000-atom probe globule. FP64 additions go
+// out at 16 clocks a warp however few lanes take part, so four atoms share a
+// warp and a lane of k_edge_sums steps through its own rows only.
 
 struct BackArgs {
     const double* X;         // centres (n x 3), input order
@@ -331,7 +418,9 @@ struct BackArgs {
     double* Wp[4];           // W' per row (pass 1)
     const int64_t* frows[3]; // frows[d]: rows of the attached facets (dim d) of each coface (dim d + 1), or -1
     const unsigned long long* parent[3];  // parent[d][r]: the coface (row of dim d + 1) of attached row r of dim d
-    double4* C[4];           // per row, per vertex: (dL/dp, dL/dr) contributions (pass 2)
+    double4* C[4];           // per unattached row, per vertex: (dL/dp, dL/dr) contributions (pass 2)
+    double4* E;              // per K^1 row: sum for its second vertex (pass 3)
+    double4* own;            // per atom: sum over the rows that start with it
     int64_t rows[4];
     const int32_t* rank;     // input index -> sorted position
     const int32_t* order;    // sorted position -> input index
@@ -355,65 +444,121 @@ __global__ void k_weights_up(BackArgs A, int d) {
     A.Wp[d][j] = W;
 }
 
-__global__ void k_contrib(BackArgs A, int d) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= A.rows[d]) return;
-    double4* out = A.C[d] + j * (d + 1);
-    const double W = A.att[d][j] ? 0.0 : A.Wp[d][j];
-    if (W == 0.0) {
-        for (int k = 0; k <= d; k++) out[k] = make_double4(0.0, 0.0, 0.0, 0.0);
-        return;
-    }
-    const int4 g = A.G[d][j];
-    const int v[4] = {g.x, g.y, g.z, g.w};
-    const Ortho o = ortho_fp64(A.X, A.R, g, d + 1);
-    for (int k = 0; k <= d; k++) {
-        const int64_t a = v[k];
-        const double l2 = 2.0 * W * o.lam[k];
-        out[k] = make_double4(l2 * (A.X[3 * a] - o.c[0]), l2 * (A.X[3 * a + 1] - o.c[1]), l2 * (A.X[3 * a + 2] - o.c[2]),
-                              -l2 * A.R[a]);
+template <int K>
+__global__ void __launch_bounds__(EVAL_THREADS) k_contrib(BackArgs A) {
+    __shared__ int list[EVAL_TILE];
+    __shared__ int n_list;
+    constexpr int d = K - 1;
+    const int64_t first = (int64_t)blockIdx.x * EVAL_TILE;
+    const int n = gather_rows(first, A.rows[d], list, &n_list, [&](int64_t j) { return A.att[d][j] != 0; });
+    for (int u = threadIdx.x; u < n; u += EVAL_THREADS) {
+        const int64_t j = first + list[u];
+        double4* out = A.C[d] + j * K;
+        const double W = A.Wp[d][j];
+        if (W == 0.0) {
+            for (int k = 0; k < K; k++) out[k] = make_double4(0.0, 0.0, 0.0, 0.0);
+            continue;
+        }
+        const int4 g = A.G[d][j];
+        const int v[4] = {g.x, g.y, g.z, g.w};
+        const Ortho o = ortho_fp64<K>(A.X, A.R, g);
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            const int64_t a = v[k];
+            const double l2 = 2.0 * W * o.lam[k];
+            out[k] = make_double4(l2 * (A.X[3 * a] - o.c[0]), l2 * (A.X[3 * a + 1] - o.c[1]),
+                                  l2 * (A.X[3 * a + 2] - o.c[2]), -l2 * A.R[a]);
+        }
     }
 }
 
-constexpr int GATHER_WARPS = 4;
+constexpr int SUM_LANES = 8;
+constexpr int SUM_THREADS = 128;
 
-__global__ void __launch_bounds__(GATHER_WARPS * 32) k_gather_atoms(BackArgs A, double* __restrict__ dX,
-                                                                     double* __restrict__ dR) {
-    const int lane = threadIdx.x & 31;
-    const int64_t a = (int64_t)blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
-    if (a >= A.n) return;
-    const int ia = A.rank[a];
-    const int64_t off = A.nb_stride ? (int64_t)ia * A.nb_stride : A.nb_off[ia];
-    const int m = A.nb_stride ? (int)A.nb_off[ia] : (int)(A.nb_off[ia + 1] - off);
-    double gx = 0.0, gy = 0.0, gz = 0.0, gr = 0.0;
-    for (int t = lane - 1; t < m; t += 32) {
-        const int64_t b = t < 0 ? a : (int64_t)A.order[A.nb[off + t]];
-        if (t >= 0 && b >= a) continue;
-        for (int d = 0; d < 4; d++) {
-            for (int64_t r = A.v0[d][b]; r < A.v0[d][b + 1]; r++) {
-                const int4 g = A.G[d][r];
-                const int k = g.x == a ? 0 : (d >= 1 && g.y == a) ? 1 : (d >= 2 && g.z == a) ? 2 : (d >= 3 && g.w == a) ? 3 : -1;
-                if (k < 0) continue;
-                const double4 q = A.C[d][r * (d + 1) + k];
-                gx += q.x;
-                gy += q.y;
-                gz += q.z;
-                gr += q.w;
+__device__ __forceinline__ void add4(double4& s, const double4& q) {
+    s.x += q.x;
+    s.y += q.y;
+    s.z += q.z;
+    s.w += q.w;
+}
+
+// sum over the SUM_LANES lanes of a group: a fixed tree, the same additions in the same order every call
+__device__ __forceinline__ double4 sum_lanes(double4 s) {
+#pragma unroll
+    for (int o = SUM_LANES / 2; o >= 1; o >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, o);
+        s.w += __shfl_xor_sync(0xffffffffu, s.w, o);
+    }
+    return s;
+}
+
+__global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
+    const int sub = threadIdx.x % SUM_LANES;
+    const int64_t b = ((int64_t)blockIdx.x * SUM_THREADS + threadIdx.x) / SUM_LANES;
+    double4 own = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (b < A.n) {
+        for (int d = 0; d < 4; d++)
+            for (int64_t r = A.v0[d][b] + sub; r < A.v0[d][b + 1]; r += SUM_LANES)
+                if (!A.att[d][r]) add4(own, A.C[d][r * (d + 1)]);
+    }
+    own = sum_lanes(own);
+    if (b >= A.n) return;
+    if (sub == 0) A.own[b] = own;
+    for (int64_t e = A.v0[1][b] + sub; e < A.v0[1][b + 1]; e += SUM_LANES) {
+        const int x = A.G[1][e].y;
+        double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
+        if (!A.att[1][e]) s = A.C[1][e * 2 + 1];  // the edge itself
+        for (int d = 2; d < 4; d++) {
+            const int64_t r1 = A.v0[d][b + 1];
+            for (int64_t r0 = A.v0[d][b]; r0 < r1; r0 += 32) {
+                const int cnt = (int)(r1 - r0 < 32 ? r1 - r0 : 32);
+                unsigned mask = 0u;  // of these rows, the unattached ones with vertex x
+                for (int t = 0; t < cnt; t++) {
+                    const int4 g = A.G[d][r0 + t];
+                    if ((g.y == x || g.z == x || g.w == x) && !A.att[d][r0 + t]) mask |= 1u << t;
+                }
+                for (; mask; mask &= mask - 1) {
+                    const int64_t r = r0 + __ffs(mask) - 1;
+                    const int4 g = A.G[d][r];
+                    add4(s, A.C[d][r * (d + 1) + (g.y == x ? 1 : g.z == x ? 2 : 3)]);
+                }
             }
         }
+        A.E[e] = s;
     }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {  // a fixed tree: the same additions in the same order every call
-        gx += __shfl_xor_sync(0xffffffffu, gx, o);
-        gy += __shfl_xor_sync(0xffffffffu, gy, o);
-        gz += __shfl_xor_sync(0xffffffffu, gz, o);
-        gr += __shfl_xor_sync(0xffffffffu, gr, o);
+}
+
+__global__ void __launch_bounds__(SUM_THREADS) k_gather_atoms(BackArgs A, double* __restrict__ dX,
+                                                               double* __restrict__ dR) {
+    const int sub = threadIdx.x % SUM_LANES;
+    const int64_t a = ((int64_t)blockIdx.x * SUM_THREADS + threadIdx.x) / SUM_LANES;
+    double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (a < A.n) {
+        if (sub == 0) s = A.own[a];
+        const int ia = A.rank[a];
+        const int64_t off = A.nb_stride ? (int64_t)ia * A.nb_stride : A.nb_off[ia];
+        const int m = A.nb_stride ? (int)A.nb_off[ia] : (int)(A.nb_off[ia + 1] - off);
+        for (int t = sub; t < m; t += SUM_LANES) {
+            const int64_t b = A.order[A.nb[off + t]];
+            if (b >= a) continue;
+            int64_t lo = A.v0[1][b], hi = A.v0[1][b + 1];
+            const int64_t end = hi;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (A.G[1][mid].y < a) lo = mid + 1;
+                else hi = mid;
+            }
+            if (lo < end && A.G[1][lo].y == a) add4(s, A.E[lo]);
+        }
     }
-    if (lane == 0) {
-        dX[3 * a] = gx;
-        dX[3 * a + 1] = gy;
-        dX[3 * a + 2] = gz;
-        dR[a] = gr;
+    s = sum_lanes(s);
+    if (sub == 0 && a < A.n) {
+        dX[3 * a] = s.x;
+        dX[3 * a + 1] = s.y;
+        dX[3 * a + 2] = s.z;
+        dR[a] = s.w;
     }
 }
 
@@ -430,9 +575,12 @@ int backward(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cud
         crows += (size_t)c->K[d].count * (d + 1);
     }
     const size_t wbytes = ((wrows > 0 ? wrows : 1) * sizeof(double) + 255) & ~(size_t)255;
-    AC_TRY(c->scratch[3].reserve(wbytes + (crows > 0 ? crows : 1) * sizeof(double4), s));
+    const size_t sums = (size_t)c->K[1].count + (size_t)n;  // E and own
+    AC_TRY(c->scratch[3].reserve(wbytes + (crows + sums) * sizeof(double4), s));
     double* Wbuf = c->scratch[3].as<double>();
     double4* Cbuf = reinterpret_cast<double4*>(static_cast<char*>(c->scratch[3].p) + wbytes);
+    A.E = Cbuf + crows;
+    A.own = A.E + c->K[1].count;
     for (int d = 0; d < 4; d++) {
         const int64_t m = c->K[d].count;
         A.G[d] = c->Gbuf[d].as<int4>();
@@ -465,10 +613,14 @@ int backward(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cud
     for (int d = 0; d < 4; d++) {
         const int64_t m = A.rows[d];
         if (m == 0) continue;
-        k_contrib<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(A, d);
+        void (*k)(BackArgs) = d == 3 ? k_contrib<4> : d == 2 ? k_contrib<3> : d == 1 ? k_contrib<2> : k_contrib<1>;
+        k<<<(unsigned)((m + EVAL_TILE - 1) / EVAL_TILE), EVAL_THREADS, 0, s>>>(A);
         AC_LAUNCHED();
     }
-    k_gather_atoms<<<(unsigned)((n + GATHER_WARPS - 1) / GATHER_WARPS), GATHER_WARPS * 32, 0, s>>>(A, dc, dr);
+    const unsigned nb = (unsigned)((n * SUM_LANES + SUM_THREADS - 1) / SUM_THREADS);
+    k_edge_sums<<<nb, SUM_THREADS, 0, s>>>(A);
+    AC_LAUNCHED();
+    k_gather_atoms<<<nb, SUM_THREADS, 0, s>>>(A, dc, dr);
     AC_LAUNCHED();
     AC_CUDA(cudaStreamSynchronize(s));
     return AC_OK;
