@@ -289,6 +289,33 @@ AC_API int ac_subcomplex(ac_ctx* ctx, int dim, int64_t mol, double alpha2, uint8
                          void* stream);
 
 /*
+ * The rows and values of a sub-complex (Section 2.4 at alpha2): of list dim of
+ * molecule mol, the rows whose entry of d_flags (as ac_subcomplex set it) is
+ * not 0, in list order, to d_rows (count_in x (dim + 1) int32), and their
+ * filtration values (as ac_filtration_values) to d_f (count_in doubles).
+ * count_in is ac_subcomplex's count; rows past it are not written. Caller-owned
+ * DEVICE arrays; either output may be NULL. Enqueued on stream, does not wait.
+ * Errors: AC_ERR_INVALID_ARG (bad dim/mol, NULL flags, count_in < 0),
+ * AC_ERR_STATE (no build yet), AC_ERR_OOM, AC_ERR_CUDA.
+ */
+AC_API int ac_subcomplex_lists(ac_ctx* ctx, int dim, int64_t mol, const uint8_t* d_flags, int64_t count_in,
+                               int32_t* d_rows, double* d_f, void* stream);
+
+/* which list ac_copy_list copies */
+#define AC_LIST_ROWS 0     /* ac_get_simplices: int32, dim + 1 per row */
+#define AC_LIST_VALUES 1   /* ac_filtration_values: double */
+#define AC_LIST_ATTACHED 2 /* ac_attached_flags: uint8 */
+
+/*
+ * Copy list `what` of (dim, mol) of the complex (Section 2.4), count rows, to dst (device or host
+ * memory), enqueued on stream; does not wait (a pageable dst may make the copy
+ * itself wait). count must be the list's length. Errors: AC_ERR_INVALID_ARG
+ * (bad what/dim/mol, another count, NULL dst with rows to copy), AC_ERR_STATE,
+ * AC_ERR_CUDA.
+ */
+AC_API int ac_copy_list(ac_ctx* ctx, int what, int dim, int64_t mol, void* dst, int64_t count, void* stream);
+
+/*
  * ---- Out-of-core build: host-resident inputs and results ----------------
  *
  * For a molecule whose lists do not fit in device memory at once (Section

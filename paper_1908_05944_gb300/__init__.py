@@ -33,11 +33,14 @@ AC_PRECISION_FILTERED = 0
 AC_PRECISION_PLAIN_FP64 = 1
 AC_FILTRATION_SIZE = 0
 AC_FILTRATION_ORTHOSIZE = 1
+AC_LIST_ROWS = 0
+AC_LIST_VALUES = 1
+AC_LIST_ATTACHED = 2
 
 # every symbol include/alphac.h declares
 EXPORTS = ["ac_create", "ac_create_batch", "ac_build", "ac_get_simplices", "ac_filtration_values", "ac_attached_flags",
            "ac_get_candidates", "ac_eval_filtration", "ac_eval_filtration_fp32", "ac_backward", "ac_backward_noalloc", "ac_autotune",
-           "ac_subcomplex", "ac_get_simplices_host", "ac_chunk_plan", "ac_build_chunked", "ac_part_plan", "ac_build_part",
+           "ac_subcomplex", "ac_subcomplex_lists", "ac_copy_list", "ac_get_simplices_host", "ac_chunk_plan", "ac_build_chunked", "ac_part_plan", "ac_build_part",
            "ac_merge_parts", "ac_chunked_simplices", "ac_chunked_info",
            "ac_chunked_free", "ac_get_stats", "ac_get_sizes", "ac_destroy", "ac_error_string", "ac_last_error_detail",
            "ac_fma_peak"]
@@ -102,6 +105,8 @@ def _declare(lib):
     lib.ac_backward_noalloc.argtypes = [vp, vp, vp, vp, vp]
     lib.ac_autotune.argtypes = [vp, vp, P(ac_options)]
     lib.ac_subcomplex.argtypes = [vp, i32, i64, dbl, vp, P(i64), vp]
+    lib.ac_subcomplex_lists.argtypes = [vp, i32, i64, vp, i64, vp, vp, vp]
+    lib.ac_copy_list.argtypes = [vp, i32, i32, i64, vp, i64, vp]
     lib.ac_get_simplices_host.argtypes = [vp, i32, i64, P(vp), P(vp), P(vp), P(i64)]
     lib.ac_chunk_plan.argtypes = [vp, vp, i64, dbl, i64, vp, i64, P(i64), P(i64)]
     lib.ac_build_chunked.argtypes = [vp, vp, i64, dbl, P(ac_options), i64, vp, P(vp)]
@@ -167,6 +172,8 @@ def _stream_ptr(stream):
     if stream is None:
         try:
             import torch
+            if torch.cuda.is_initialized():
+                return _current_stream(torch, torch.cuda.current_device())
             if torch.cuda.is_available():
                 return torch.cuda.current_stream().cuda_stream
         except Exception:
@@ -175,12 +182,42 @@ def _stream_ptr(stream):
     return getattr(stream, "cuda_stream", stream)
 
 
+def _current_stream(torch, index):
+    """The current stream of CUDA device `index` as an integer, without building a Stream object (3 us)."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(index) if raw is not None else torch.cuda.current_stream(index).cuda_stream
+
+
 class _DeviceArray:
     """Non-owning __cuda_array_interface__ view of device memory owned by a context."""
 
     def __init__(self, ptr, shape, typestr):
         self.__cuda_array_interface__ = {"shape": tuple(shape), "typestr": typestr, "data": (ptr or 0, False),
                                          "version": 3, "strides": None}
+
+
+_kinds_cache = None
+
+
+def _list_kinds():
+    """(torch, per AC_LIST_* the getter, tensor dtype and array type string, the CUDA devices): what every list
+    call needs, looked up once (a batch is read with thousands of calls of a few microseconds)."""
+    global _kinds_cache
+    if _kinds_cache is None:
+        import torch
+        L = lib()
+        _kinds_cache = (torch, ((L.ac_get_simplices, torch.int32, "<i4"), (L.ac_filtration_values, torch.float64, "<f8"),
+                                (L.ac_attached_flags, torch.uint8, "|u1")),
+                        [torch.device("cuda", k) for k in range(max(1, torch.cuda.device_count()))])
+    return _kinds_cache
+
+
+class _HostArray:
+    """Non-owning __array_interface__ view of host memory owned by a context (a ctypes array would need a new
+    ctypes type for every length)."""
+
+    def __init__(self, ptr, shape, typestr):
+        self.__array_interface__ = {"shape": shape, "typestr": typestr, "data": (ptr, False), "version": 3}
 
 
 def options(precision=AC_PRECISION_FILTERED, filtration=AC_FILTRATION_SIZE, cell_factor=0.0, block_warps=0,
@@ -232,26 +269,35 @@ class AlphaComplex:
         _check(lib().ac_build(self._h, _stream_ptr(stream)), "ac_build")
         return self
 
-    def _view(self, getter, dim, mol, width, typestr, copy):
-        import torch
+    def _list(self, what, dim, mol, copy):
+        """List `what` (AC_LIST_*): a tensor of its own, filled by one copy, or a view into the context."""
+        torch, kinds, devices = _list_kinds()
+        getter, dt, typestr = kinds[what]
         p = ctypes.c_void_p()
         cnt = ctypes.c_int64()
-        _check(getter(self._h, dim, mol, ctypes.byref(p), ctypes.byref(cnt)), getter.__name__)
-        shape = (cnt.value, width) if width else (cnt.value,)
-        if cnt.value == 0:
-            dt = {"<i4": torch.int32, "<f8": torch.float64, "|u1": torch.uint8}[typestr]
-            return torch.zeros(shape, dtype=dt, device="cuda")
-        t = torch.as_tensor(_DeviceArray(p.value, shape, typestr), device="cuda")
-        return t.clone() if copy else t
+        rc = getter(self._h, dim, mol, ctypes.byref(p), ctypes.byref(cnt))
+        if rc != AC_OK:
+            _check(rc, getter.__name__)
+        n = cnt.value
+        shape = (n, dim + 1) if what == AC_LIST_ROWS else (n,)
+        index = torch.cuda.current_device()
+        if n == 0:
+            return torch.zeros(shape, dtype=dt, device=devices[index])
+        if not copy:
+            return torch.as_tensor(_DeviceArray(p.value, shape, typestr), device=devices[index])
+        out = torch.empty(shape, dtype=dt, device=devices[index])
+        _check(lib().ac_copy_list(self._h, what, dim, mol, out.data_ptr(), n, _current_stream(torch, index)),
+               "ac_copy_list")
+        return out
 
     def simplices(self, dim: int, mol: int = -1, copy: bool = True):
-        return self._view(lib().ac_get_simplices, dim, mol, dim + 1, "<i4", copy)
+        return self._list(AC_LIST_ROWS, dim, mol, copy)
 
     def filtration_values(self, dim: int, mol: int = -1, copy: bool = True):
-        return self._view(lib().ac_filtration_values, dim, mol, 0, "<f8", copy)
+        return self._list(AC_LIST_VALUES, dim, mol, copy)
 
     def attached(self, dim: int, mol: int = -1, copy: bool = True):
-        return self._view(lib().ac_attached_flags, dim, mol, 0, "|u1", copy)
+        return self._list(AC_LIST_ATTACHED, dim, mol, copy)
 
     def host_lists(self, dim: int, mol: int = -1, copy: bool = True):
         """(rows, filtration values, attached flags) of list dim as numpy arrays, from the host copies the
@@ -264,9 +310,8 @@ class AlphaComplex:
         n = cnt.value
         if n == 0:
             return (np.zeros((0, dim + 1), np.int32), np.zeros(0, np.float64), np.zeros(0, np.uint8))
-        out = (np.ctypeslib.as_array((ctypes.c_int32 * (n * (dim + 1))).from_address(t.value)).reshape(n, dim + 1),
-               np.ctypeslib.as_array((ctypes.c_double * n).from_address(f.value)),
-               np.ctypeslib.as_array((ctypes.c_uint8 * n).from_address(a.value)))
+        out = (np.asarray(_HostArray(t.value, (n, dim + 1), "<i4")), np.asarray(_HostArray(f.value, (n,), "<f8")),
+               np.asarray(_HostArray(a.value, (n,), "|u1")))
         return tuple(x.copy() for x in out) if copy else out
 
     def candidates(self, dim: int, copy: bool = True):
@@ -297,11 +342,17 @@ class AlphaComplex:
 
     def subcomplex(self, alpha2: float, mol: int = -1, stream=None):
         """The alpha complex at alpha2 <= alpha from this build: per dimension (simplices, Size values)."""
+        import torch
+        index = torch.cuda.current_device()
         out = []
         for d in range(4):
-            mask, _ = self.subcomplex_mask(d, alpha2, mol, stream)
-            keep = mask.bool()
-            out.append((self.simplices(d, mol)[keep], self.filtration_values(d, mol)[keep]))
+            mask, n = self.subcomplex_mask(d, alpha2, mol, stream)
+            rows = torch.empty((n, d + 1), dtype=torch.int32, device=mask.device)
+            f = torch.empty((n,), dtype=torch.float64, device=mask.device)
+            if n:
+                _check(lib().ac_subcomplex_lists(self._h, d, mol, mask.data_ptr(), n, rows.data_ptr(), f.data_ptr(),
+                                                 _current_stream(torch, index)), "ac_subcomplex_lists")
+            out.append((rows, f))
         return out
 
     def stats(self) -> dict:

@@ -1205,6 +1205,32 @@ extern "C" int ac_subcomplex(ac_ctx* c, int dim, int64_t mol, double alpha2, uin
     return subcomplex_flags(c, dim, first, count, alpha2, d_flags, count_in, (cudaStream_t)stream);
 }
 
+extern "C" int ac_subcomplex_lists(ac_ctx* c, int dim, int64_t mol, const uint8_t* d_flags, int64_t count_in,
+                                   int32_t* d_rows, double* d_f, void* stream) {
+    int64_t first = 0, count = 0;
+    AC_TRY(get_list(c, c ? c->K : nullptr, dim, mol, &first, &count));
+    if (count_in < 0 || (count > 0 && !d_flags)) return fail(AC_ERR_INVALID_ARG, "bad argument");
+    StreamScope scope((cudaStream_t)stream);
+    return subcomplex_lists(c, dim, first, count, d_flags, count_in, d_rows, d_f, (cudaStream_t)stream);
+}
+
+extern "C" int ac_copy_list(ac_ctx* c, int what, int dim, int64_t mol, void* dst, int64_t count, void* stream) {
+    int64_t first = 0, n = 0;
+    AC_TRY(get_list(c, c ? c->K : nullptr, dim, mol, &first, &n));
+    if (what < AC_LIST_ROWS || what > AC_LIST_ATTACHED) return fail(AC_ERR_INVALID_ARG, "unknown list");
+    if (count != n || (n > 0 && !dst)) return fail(AC_ERR_INVALID_ARG, "bad count or NULL dst");
+    if (n == 0) return AC_OK;
+    const ac::SimplexList& L = c->K[dim];
+    const ac::DevBuf& b = what == AC_LIST_ROWS       ? L.tuples
+                          : what == AC_LIST_ATTACHED ? L.attached
+                          : c->opt.filtration == AC_FILTRATION_ORTHOSIZE ? L.orthosize
+                                                                         : L.f;
+    const size_t item = what == AC_LIST_ROWS ? (size_t)(dim + 1) * sizeof(int32_t) : what == AC_LIST_VALUES ? sizeof(double) : 1;
+    AC_CUDA(cudaMemcpyAsync(dst, static_cast<const char*>(b.p) + (size_t)first * item, (size_t)n * item, cudaMemcpyDefault,
+                            (cudaStream_t)stream));
+    return AC_OK;
+}
+
 extern "C" int ac_autotune(ac_ctx* c, void* stream, ac_options* chosen) {
     if (!c) return fail(AC_ERR_INVALID_ARG, "ctx is NULL");
     c->plan_fresh = false;  // every trial plans its own grid

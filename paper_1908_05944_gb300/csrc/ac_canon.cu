@@ -1213,14 +1213,18 @@ __global__ void k_coface_apply(int64_t m, const uint8_t* __restrict__ attached, 
 // K_alpha2 iff Size <= alpha2 (Section 2.4). Size is the OrthoSize of the
 // simplex's source (itself when unattached, else the coface its value came
 // from), compared exactly: num <= A2 den.
-__global__ void k_subcomplex(const int4* __restrict__ P, const int4* __restrict__ const* G, const int8_t* __restrict__ src_dim,
+struct RowLists {
+    const int4* G[4];
+};
+
+__global__ void k_subcomplex(const int4* __restrict__ P, RowLists rows, const int8_t* __restrict__ src_dim,
                              const int64_t* __restrict__ src_idx, int64_t first, int64_t m, long long A2,
                              uint8_t* __restrict__ flags, unsigned long long* __restrict__ n_in) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool in = false;
     if (j < m) {
         const int sd = src_dim[first + j];
-        const int4 t = G[sd][src_idx[first + j]];
+        const int4 t = rows.G[sd][src_idx[first + j]];
         i128 num, den;
         orthosize_rational(P, t, sd + 1, num, den);
         in = num <= (i128)A2 * den;
@@ -1233,23 +1237,109 @@ __global__ void k_subcomplex(const int4* __restrict__ P, const int4* __restrict_
 int subcomplex_flags(ac_ctx* c, int dim, int64_t first, int64_t m, double alpha2, uint8_t* flags, int64_t* count,
                      cudaStream_t s) {
     const long long A2 = (long long)nearbyint(alpha2 * 1048576.0);
-    AC_TRY(c->scratch[6].reserve(sizeof(unsigned long long) + 4 * sizeof(int4*), s));
+    AC_TRY(c->scratch[6].reserve(sizeof(unsigned long long), s));
     unsigned long long* n_in = c->scratch[6].as<unsigned long long>();
-    const int4** g = reinterpret_cast<const int4**>(n_in + 1);
-    const int4* gh[4];
-    for (int d = 0; d < 4; d++) gh[d] = c->Gbuf[d].as<int4>();
-    AC_CUDA(cudaMemcpyAsync(g, gh, sizeof(gh), cudaMemcpyHostToDevice, s));
     AC_CUDA(cudaMemsetAsync(n_in, 0, sizeof(unsigned long long), s));
     if (m > 0) {
         SimplexList& L = c->K[dim];
-        k_subcomplex<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(c->P.as<int4>(), g, L.src_dim.as<int8_t>(),
+        RowLists rows;
+        for (int d = 0; d < 4; d++) rows.G[d] = c->Gbuf[d].as<int4>();
+        k_subcomplex<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(c->P.as<int4>(), rows, L.src_dim.as<int8_t>(),
                                                                   L.src_idx.as<int64_t>(), first, m, A2, flags, n_in);
         AC_LAUNCHED();
     }
-    unsigned long long h = 0;
-    AC_CUDA(cudaMemcpyAsync(&h, n_in, sizeof(h), cudaMemcpyDeviceToHost, s));
+    AC_CUDA(cudaMemcpyAsync(c->h_stage, n_in, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     AC_CUDA(cudaStreamSynchronize(s));
-    *count = (int64_t)h;
+    *count = c->h_stage[0];
+    return AC_OK;
+}
+
+// The flagged rows of a list and their values, in list order: counts per tile
+// of SUB_TILE flags, their prefix by one block, then each tile writes its rows.
+// (Boolean indexing by the caller took two passes with a host wait each.)
+constexpr int SUB_THREADS = 256;
+constexpr int SUB_TILE = 4096;
+
+__global__ void __launch_bounds__(SUB_THREADS) k_sub_count(const uint8_t* __restrict__ flags, int64_t m,
+                                                           unsigned* __restrict__ tile) {
+    const int64_t j0 = (int64_t)blockIdx.x * SUB_TILE;
+    int c = 0;
+    for (int u = threadIdx.x; u < SUB_TILE; u += SUB_THREADS) c += __syncthreads_count(j0 + u < m && flags[j0 + u]);
+    if (threadIdx.x == 0) tile[blockIdx.x] = (unsigned)c;
+}
+
+__global__ void __launch_bounds__(1024) k_sub_prefix(unsigned* __restrict__ tile, int n) {
+    __shared__ unsigned sums[32];
+    __shared__ unsigned carry;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    for (int t0 = 0; t0 < n; t0 += 1024) {
+        const int t = t0 + threadIdx.x;
+        const unsigned v = t < n ? tile[t] : 0u;
+        unsigned inc = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += x;
+        }
+        if (lane == 31) sums[w] = inc;
+        __syncthreads();
+        unsigned before = carry;
+        for (int q = 0; q < w; q++) before += sums[q];
+        if (t < n) tile[t] = before + inc - v;
+        __syncthreads();
+        if (threadIdx.x == 1023) carry = before + inc;
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(SUB_THREADS) k_sub_write(const uint8_t* __restrict__ flags, int64_t m, int k,
+                                                           const unsigned* __restrict__ tile,
+                                                           const int32_t* __restrict__ rows,
+                                                           const double* __restrict__ f, int64_t count,
+                                                           int32_t* __restrict__ rows_out, double* __restrict__ f_out) {
+    __shared__ int sums[SUB_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t j0 = (int64_t)blockIdx.x * SUB_TILE;
+    int64_t at = tile[blockIdx.x];
+    for (int u = threadIdx.x; u < SUB_TILE; u += SUB_THREADS) {
+        const int64_t j = j0 + u;
+        const bool in = j < m && flags[j];
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) sums[w] = __popc(b);
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int q = 0; q < SUB_THREADS / 32; q++) {
+            before += q < w ? sums[q] : 0;
+            all += sums[q];
+        }
+        const int64_t r = at + before + __popc(b & ((1u << lane) - 1u));
+        if (in && r < count) {
+            if (rows_out)
+                for (int q = 0; q < k; q++) rows_out[r * k + q] = rows[j * k + q];
+            if (f_out) f_out[r] = f[j];
+        }
+        at += all;
+        __syncthreads();
+    }
+}
+
+int subcomplex_lists(ac_ctx* c, int dim, int64_t first, int64_t m, const uint8_t* flags, int64_t count, int32_t* rows,
+                     double* f, cudaStream_t s) {
+    if (m == 0 || count == 0 || (!rows && !f)) return AC_OK;
+    const SimplexList& L = c->K[dim];
+    const int k = dim + 1;
+    const DevBuf& v = c->opt.filtration == AC_FILTRATION_ORTHOSIZE ? L.orthosize : L.f;
+    const int64_t tiles = (m + SUB_TILE - 1) / SUB_TILE;
+    // this call's own, released in stream order: calls on other streams may overlap it
+    DevBuf tile;
+    AC_TRY(tile.reserve((size_t)tiles * sizeof(unsigned), s));
+    k_sub_count<<<(unsigned)tiles, SUB_THREADS, 0, s>>>(flags, m, tile.as<unsigned>());
+    AC_LAUNCHED();
+    k_sub_prefix<<<1, 1024, 0, s>>>(tile.as<unsigned>(), (int)tiles);
+    AC_LAUNCHED();
+    k_sub_write<<<(unsigned)tiles, SUB_THREADS, 0, s>>>(flags, m, k, tile.as<unsigned>(), L.tuples.as<int32_t>() + first * k,
+                                                        v.as<double>() + first, count, rows, f);
+    AC_LAUNCHED();
     return AC_OK;
 }
 

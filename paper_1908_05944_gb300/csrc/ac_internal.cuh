@@ -328,6 +328,8 @@ int backward(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cud
 int backward_noalloc(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cudaStream_t s);
 int subcomplex_flags(ac_ctx* c, int dim, int64_t first, int64_t m, double alpha2, uint8_t* flags, int64_t* count,
                      cudaStream_t s);
+int subcomplex_lists(ac_ctx* c, int dim, int64_t first, int64_t m, const uint8_t* flags, int64_t count, int32_t* rows,
+                     double* f, cudaStream_t s);
 
 int read_counters(ac_ctx* c, DevCounters* h, cudaStream_t s);
 // Replay checks: set DERR_REPLAY in the counters when a device value differs
