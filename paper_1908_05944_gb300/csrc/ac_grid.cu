@@ -241,7 +241,7 @@ static unsigned neighbour_blocks(int64_t n) { return (unsigned)((n + NB_THREADS 
 // kernel's tail is short; the atoms with more than 64 neighbours form its head.
 constexpr int DEG_BINS = 259;  // counts 0..256, 257 for 257..512, 258 for anything above
 
-__device__ __forceinline__ int deg_bin(int64_t m) { return m > 512 ? 258 : m > 256 ? 257 : (int)m; }
+__device__ __forceinline__ int deg_bin(int64_t m) { return m > 512 ? 258 : m > 256 ? 257 : m > 64 ? (int)m : ((int)m + 15) & ~15; }
 
 __global__ void k_deg_hist(const int64_t* __restrict__ cnt, int64_t n, unsigned* __restrict__ hist) {
     __shared__ unsigned h[DEG_BINS];
