@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "ac_internal.cuh"
+#include "ac_scan.cuh"
 
 namespace ac {
 
@@ -357,6 +358,11 @@ static int scan_entry(const T* in, T* out, int64_t n, DevBuf& tmp, DevCounters* 
         AC_CUDA(cudaMemsetAsync(out, 0, sizeof(T), s));
         return AC_OK;
     }
+    if (n <= SC_MAX) {
+        launch_small_scan(ScanArray<T>{in}, out, n, s);
+        AC_LAUNCHED();
+        return AC_OK;
+    }
     const int64_t tiles = n / SCAN_TILE + 1;  // n + 1 outputs
     if (tiles <= SCAN_SMALL_TILES) {
         AC_TRY(tmp.reserve((size_t)tiles * sizeof(T), s));
@@ -563,9 +569,17 @@ __global__ void k_fill_mol(const int64_t* __restrict__ mol_off, int64_t n_mol, i
     for (int64_t i = mol_off[m] + threadIdx.x; i < mol_off[m + 1]; i += blockDim.x) mol_of[i] = (int32_t)m;
 }
 
-__global__ void k_init_bbox(int32_t* bbox, int64_t n_mol, DevCounters* cnt) {
-    int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m == 0) cnt->bad_index = INT32_MAX;
+// What a build adds to, emptied in one launch: counters, bounding boxes, degree
+// histogram and cursors. One molecule: its offsets too.
+__global__ void k_init(int32_t* bbox, int64_t n_mol, DevCounters* cnt, unsigned* deg, int64_t* mol_off, int64_t n) {
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x == 0) {
+        unsigned* c = reinterpret_cast<unsigned*>(cnt);
+        for (int k = threadIdx.x; k < (int)(sizeof(DevCounters) / sizeof(unsigned)); k += blockDim.x)
+            c[k] = k == (int)(offsetof(DevCounters, bad_index) / sizeof(unsigned)) ? (unsigned)INT32_MAX : 0u;
+        for (int k = threadIdx.x; k < 2 * DEG_BINS; k += blockDim.x) deg[k] = 0u;
+        if (n_mol == 1 && threadIdx.x < 2) mol_off[threadIdx.x] = threadIdx.x ? n : 0;
+    }
     if (m >= n_mol) return;
     for (int k = 0; k < 3; k++) {
         bbox[6 * m + k] = INT32_MAX;
@@ -578,30 +592,26 @@ __global__ void k_init_bbox(int32_t* bbox, int64_t n_mol, DevCounters* cnt) {
 // side ~ h = sqrt(r_max^2 + alpha), dense cell table over each bounding box.
 int quantise_and_plan(ac_ctx* c, cudaStream_t s) {
     const int64_t n = c->n, n_mol = c->n_mol;
-    AC_TRY(c->scratch[0].reserve((size_t)n_mol * 6 * sizeof(int32_t), s));
-    AC_TRY(c->scratch[1].reserve(sizeof(int), s));
+    AC_TRY(c->deg.reserve(2 * DEG_BINS * sizeof(unsigned), s));
     DevCounters* dc = c->counters.as<DevCounters>();
-    AC_CUDA(cudaMemsetAsync(dc, 0, sizeof(DevCounters), s));
-    int32_t* bbox = c->scratch[0].as<int32_t>();
-    int* wmax = c->scratch[1].as<int>();
-    AC_CUDA(cudaMemsetAsync(wmax, 0, sizeof(int), s));
-    k_init_bbox<<<(unsigned)((n_mol + 255) / 256), 256, 0, s>>>(bbox, n_mol, dc);
+    int32_t* bbox = reinterpret_cast<int32_t*>(static_cast<char*>(c->counters.p) + BBOX_OFFSET);
+    k_init<<<(unsigned)((n_mol + 255) / 256), 256, 0, s>>>(bbox, n_mol, dc, c->deg.as<unsigned>(),
+                                                          c->d_moloff.as<int64_t>(), n);
     AC_LAUNCHED();
     if (n > 0) {
         k_quantise<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c->centres.as<double>(), c->radii.as<double>(), n,
-                                                              c->mol_of.as<int32_t>(), c->P.as<int4>(), bbox, wmax, dc);
+                                                              c->mol_of.as<int32_t>(), c->P.as<int4>(), bbox, &dc->wmax, dc);
         AC_LAUNCHED();
     }
     if (c->replaying) {
         // the recorded plan stands; check the bounds it rests on
         AC_TRY(expect_i32s(c, bbox, c->rec_bbox.as<int32_t>(), n_mol * 6));
-        AC_TRY(expect_i32s(c, wmax, c->rec_bbox.as<int32_t>() + n_mol * 6, 1));
+        AC_TRY(expect_i32s(c, &dc->wmax, c->rec_bbox.as<int32_t>() + n_mol * 6, 1));
         return AC_OK;
     }
-    // one readback: counters, largest weight, per-molecule boxes
-    AC_CUDA(cudaMemcpyAsync(c->h_cnt, c->counters.p, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
-    AC_CUDA(cudaMemcpyAsync(c->h_stage, wmax, sizeof(int), cudaMemcpyDeviceToHost, s));
-    AC_CUDA(cudaMemcpyAsync(c->h_bbox, bbox, (size_t)n_mol * 6 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    // one readback: counters (the largest weight among them), per-molecule boxes
+    AC_CUDA(cudaMemcpyAsync(c->h_cnt, c->counters.p, BBOX_OFFSET + (size_t)n_mol * 6 * sizeof(int32_t),
+                            cudaMemcpyDeviceToHost, s));
     AC_TRY(sync_host(c, s));
     const DevCounters hc = *c->h_cnt;
     if (hc.err & DERR_INVALID) {
@@ -615,7 +625,7 @@ int quantise_and_plan(ac_ctx* c, cudaStream_t s) {
                  hc.bad_index);
         return fail(AC_ERR_RANGE, b);
     }
-    const int wmax_h = *reinterpret_cast<const int*>(c->h_stage);
+    const int wmax_h = hc.wmax;
     const int32_t* hb = c->h_bbox;
 
     PredConst& pc = c->pc;
@@ -840,7 +850,7 @@ static int create_impl(const double* centres, const double* radii, const int64_t
         return code;
     };
     {
-        const size_t a0 = 64 * sizeof(int64_t), a1 = (sizeof(DevCounters) + 255) & ~(size_t)255;
+        const size_t a0 = 64 * sizeof(int64_t), a1 = BBOX_OFFSET;
         const size_t a2 = ((size_t)6 * n_mol * sizeof(int32_t) + 255) & ~(size_t)255;
         const size_t a3 = (size_t)7 * (n_mol + 1) * sizeof(int64_t);
         // small blocks share one size class, so cached sets fit most contexts
@@ -869,7 +879,7 @@ static int create_impl(const double* centres, const double* radii, const int64_t
     if ((rc = c->centres.reserve(nn * 3 * sizeof(double), s)) || (rc = c->radii.reserve(nn * sizeof(double), s)) ||
         (rc = c->P.reserve(nn * sizeof(int4), s)) || (rc = c->mol_of.reserve(nn * sizeof(int32_t), s)) ||
         (rc = c->d_moloff.reserve((size_t)(n_mol + 1) * sizeof(int64_t), s)) ||
-        (rc = c->counters.reserve(sizeof(DevCounters), s)))
+        (rc = c->counters.reserve(BBOX_OFFSET + (size_t)n_mol * 6 * sizeof(int32_t), s)))
         return bail(rc);
     // stream-ordered copies: the quantisation below waits for its bounds before ac_create
     // returns, so the caller's buffers are free again by then
@@ -878,12 +888,17 @@ static int create_impl(const double* centres, const double* radii, const int64_t
             cudaMemcpyAsync(c->radii.p, radii, (size_t)n * sizeof(double), cudaMemcpyDefault, s) != cudaSuccess)
             return bail(cuda_fail(cudaGetLastError(), "copy of centres/radii", __FILE__, __LINE__));
     }
-    if (cudaMemcpyAsync(c->d_moloff.p, offsets, (size_t)(n_mol + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) !=
-        cudaSuccess)
-        return bail(cuda_fail(cudaGetLastError(), "copy of offsets", __FILE__, __LINE__));
-
-    k_fill_mol<<<(unsigned)n_mol, 256, 0, s>>>(c->d_moloff.as<int64_t>(), n_mol, c->mol_of.as<int32_t>());
-    if (cudaGetLastError() != cudaSuccess) return bail(cuda_fail(cudaGetLastError(), "k_fill_mol", __FILE__, __LINE__));
+    if (n_mol == 1) {  // the offsets come with k_init
+        if (cudaMemsetAsync(c->mol_of.p, 0, nn * sizeof(int32_t), s) != cudaSuccess)
+            return bail(cuda_fail(cudaGetLastError(), "memset of the molecule index", __FILE__, __LINE__));
+    } else {
+        if (cudaMemcpyAsync(c->d_moloff.p, offsets, (size_t)(n_mol + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) !=
+            cudaSuccess)
+            return bail(cuda_fail(cudaGetLastError(), "copy of offsets", __FILE__, __LINE__));
+        k_fill_mol<<<(unsigned)n_mol, 256, 0, s>>>(c->d_moloff.as<int64_t>(), n_mol, c->mol_of.as<int32_t>());
+        if (cudaGetLastError() != cudaSuccess)
+            return bail(cuda_fail(cudaGetLastError(), "k_fill_mol", __FILE__, __LINE__));
+    }
     if ((rc = quantise_and_plan(c, s))) return bail(rc);
     c->plan_fresh = true;
     *out = c;
@@ -959,6 +974,12 @@ static int capture_replay(ac_ctx* c) {
     cudaStream_t s = c->cap_stream;
     c->expects.clear();
     AC_TRY(c->expect_table.reserve(MAX_EXPECTS * sizeof(ExpectEntry), s));
+    // the plan bounds the replays check against: those the synchronised build read back
+    const size_t nbox = (size_t)c->n_mol * 6 * sizeof(int32_t);
+    AC_TRY(c->rec_bbox.reserve(nbox + sizeof(int32_t), s));
+    AC_CUDA(cudaMemcpyAsync(c->rec_bbox.p, c->h_bbox, nbox, cudaMemcpyHostToDevice, s));
+    AC_CUDA(cudaMemcpyAsync(static_cast<char*>(c->rec_bbox.p) + nbox, &c->rec.wmax, sizeof(int32_t),
+                            cudaMemcpyHostToDevice, s));
     AC_CUDA(cudaStreamSynchronize(s));
     AC_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     const long long l0 = g_launch_count;
@@ -1015,17 +1036,6 @@ static int record_build(ac_ctx* c, const DevCounters& post, cudaStream_t s) {
     return AC_OK;
 }
 
-// The plan bounds a replay checks against, copied before the build's last host
-// wait (which then also completes them, before a replay on another stream reads them).
-static int record_copies(ac_ctx* c, cudaStream_t s) {
-    const size_t nb = (size_t)c->n_mol * 6;
-    AC_TRY(c->rec_bbox.reserve((nb + 1) * sizeof(int32_t), s));
-    AC_CUDA(cudaMemcpyAsync(c->rec_bbox.p, c->scratch[0].p, nb * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    AC_CUDA(cudaMemcpyAsync(c->rec_bbox.as<int32_t>() + nb, c->scratch[1].p, sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                            s));
-    return AC_OK;
-}
-
 extern "C" int ac_build(ac_ctx* c, void* stream) {
     if (!c) return fail(AC_ERR_INVALID_ARG, "ctx is NULL");
     cudaStream_t s = (cudaStream_t)stream;
@@ -1057,7 +1067,6 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
     if (!replayed) {
         drop_graph(c);
         AC_TRY(build_body(c, s));
-        if (!c->opt.no_graph) AC_TRY(record_copies(c, s));
         AC_TRY(read_counters(c, &h, s));
     }
     if (h.err & DERR_INTERNAL)

@@ -23,6 +23,7 @@
 #include "ac_internal.cuh"
 #include "ac_bucket.h"
 #include "ac_round.h"
+#include "ac_scan.cuh"
 
 namespace ac {
 
@@ -53,9 +54,8 @@ __device__ __forceinline__ void sort_asc(int4& t, int K) {
     }
 }
 
-// Unused tuple slots hold -1 so comparisons ignore them.
+// facet of a row of K + 1 ascending entries: the K-tuple without entry drop
 __device__ __forceinline__ int4 facet_of(const int4& t, int K, int drop) {
-    // t has K+1 valid ascending entries; return the K-tuple without entry drop
     int v[4] = {t.x, t.y, t.z, t.w};
     int o[4] = {-1, -1, -1, -1};
     int w = 0;
@@ -64,45 +64,30 @@ __device__ __forceinline__ int4 facet_of(const int4& t, int K, int drop) {
     return make_int4(o[0], o[1], o[2], o[3]);
 }
 
-// Items of one dimension: [0, nA) from a list in sorted positions (a4, or a2 for
-// edges), then nB * (K + 1) facets of a canonical list of width K + 1. An item
-// is an ascending K-tuple of input indices; its bucket is its first vertex. For
-// K <= 3 the unused last component carries the flag (1: the simplex passed AC2
-// at its orthocentre, 0: a facet); for K = 4 every item is a list item (flag 1).
+// The items of one list, K entries each, emitted once each by their owner:
+// nA tuples of sorted positions (a4, or a2 for edges), taken to ascending tuples
+// of input indices. An item's bucket is its first vertex.
 struct CanonArgs {
     const int4* a4;
     const int2* a2;
     int64_t nA;
-    const int4* cof;
-    int64_t nB;
     const int32_t* order;  // sorted position -> input index
-    int64_t total;
-    int64_t* bucket_cnt;   // count pass: items per bucket
+    int64_t* bucket_cnt;   // items per bucket; the scatter counts it down to 0
     const int64_t* off;    // scatter pass: bucket offsets
-    unsigned long long* cursor;
     int4* T;               // scattered items
 };
 
 template <int K>
 __device__ __forceinline__ int4 canon_item(const CanonArgs& a, int64_t j) {
     int4 t;
-    if (j < a.nA) {
-        if (K == 2) {
-            const int2 e = a.a2[j];
-            t = make_int4(a.order[e.x], a.order[e.y], -1, -1);
-        } else {
-            const int4 e = a.a4[j];
-            t = make_int4(a.order[e.x], a.order[e.y], a.order[e.z], K == 4 ? a.order[e.w] : -1);
-        }
-        sort_asc(t, K);
-        if (K < 4) t.w = 1;
+    if (K == 2) {
+        const int2 e = a.a2[j];
+        t = make_int4(a.order[e.x], a.order[e.y], -1, -1);
     } else {
-        const int64_t r = j - a.nA;
-        const int64_t row = r / (K + 1);
-        const int drop = (int)(r - row * (K + 1));
-        t = facet_of(a.cof[row], K, drop);
-        t.w = 0;  // K < 4 here: facets exist for K = 2, 3
+        const int4 e = a.a4[j];
+        t = make_int4(a.order[e.x], a.order[e.y], a.order[e.z], K == 4 ? a.order[e.w] : -1);
     }
+    sort_asc(t, K);
     return t;
 }
 
@@ -110,7 +95,7 @@ __device__ __forceinline__ int4 canon_item(const CanonArgs& a, int64_t j) {
 template <int K>
 __global__ void k_canon_count(CanonArgs a) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = j < a.total;
+    const bool valid = j < a.nA;
     const int lane = threadIdx.x & 31;
     const int x = valid ? canon_item<K>(a, j).x : -1 - lane;
     const unsigned peers = __match_any_sync(0xffffffffu, x);
@@ -121,27 +106,28 @@ __global__ void k_canon_count(CanonArgs a) {
 template <int K>
 __global__ void k_canon_scatter(CanonArgs a) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = j < a.total;
+    const bool valid = j < a.nA;
     const int lane = threadIdx.x & 31;
     int4 t = make_int4(-1 - lane, 0, 0, 0);
     if (valid) t = canon_item<K>(a, j);
     const unsigned peers = __match_any_sync(0xffffffffu, t.x);
     const int leader = __ffs(peers) - 1;
     unsigned long long base = 0;
-    if (valid && lane == leader) base = atomicAdd(&a.cursor[t.x], (unsigned long long)__popc(peers));
+    if (valid && lane == leader) {
+        const unsigned long long k = (unsigned long long)__popc(peers);
+        base = atomicAdd((unsigned long long*)&a.bucket_cnt[t.x], 0ull - k) - k;
+    }
     base = __shfl_sync(0xffffffffu, base, leader);
     if (valid) a.T[a.off[t.x] + (int64_t)base + __popc(peers & ((1u << lane) - 1u))] = t;
 }
 
-// In-bucket sort and de-duplication, one warp per bucket of up to CSORT_MAX
-// items. The rest of each tuple becomes a sort key: K = 2: (y << 1) | flag;
-// K = 3: (y << 33) | (z << 1) | flag (y, z < 2^31); K = 4: hi = (y << 32) | z,
-// lo = w (flag 1). Keys sit in registers, R = ceil(k/32) per lane (padded to a
-// power of two with the largest key), and a bitonic network sorts them:
-// exchanges across lanes by shuffles, across a lane's registers directly.
-// Equal tuples (the flag bit aside) are then adjacent; the first of each run
-// takes the OR of the run's flags and the run is compacted to the front of
-// the bucket.
+// In-bucket sort, one warp per bucket, which then writes its rows. Up to 32 items
+// every lane ranks its own among the others; up to CSORT_MAX a bitonic network
+// sorts them in registers, R = ceil(k/32) per lane (padded to a power of two
+// with the largest key), exchanges across lanes by shuffles, across a lane's
+// registers directly. The rest of each tuple is the sort key: K = 2: y; K = 3:
+// (y << 32) | z; K = 4: hi = (y << 32) | z, lo = w. The items are distinct; two
+// equal ones (a bug) raise DERR_INTERNAL.
 constexpr int CSORT_MAX = 256;
 constexpr int CSORT_WARPS = 4;
 
@@ -153,16 +139,8 @@ struct SortSmem {
 template <int K>
 __device__ __forceinline__ void make_key(const int4& t, unsigned long long& hi, unsigned& lo) {
     const unsigned long long y = (unsigned)t.y, z = (unsigned)t.z;
-    if (K == 2) {
-        hi = (y << 1) | (unsigned)t.w;
-        lo = 0u;
-    } else if (K == 3) {
-        hi = (y << 33) | (z << 1) | (unsigned)t.w;
-        lo = 0u;
-    } else {
-        hi = (y << 32) | z;
-        lo = (unsigned)t.w;
-    }
+    hi = K == 2 ? y : (y << 32) | z;
+    lo = K == 4 ? (unsigned)t.w : 0u;
 }
 
 template <int K, class H>
@@ -170,7 +148,7 @@ __device__ __forceinline__ bool key_less(H ah, unsigned al, H bh, unsigned bl) {
     return K == 4 ? (ah < bh || (ah == bh && al < bl)) : ah < bh;
 }
 
-// register type of the high key: edges' keys (y << 1 | flag, y < 2^31) fit 32 bits
+// register type of the high key: edges' keys fit 32 bits
 template <int K>
 using KeyHi = typename std::conditional<K == 2, unsigned, unsigned long long>::type;
 
@@ -240,15 +218,33 @@ __device__ __forceinline__ void bitonic_place(SortSmem& S, const int4* __restric
     }
 }
 
-// Buckets above CSORT_MAX items (rare): one lane, heap sort in place (O(k log k)) then de-duplication.
+struct CanonOut {
+    const int32_t* mol_of;   // input index -> molecule
+    const int64_t* mol_off;  // molecule -> first input index
+    int4* G;                 // canonical rows, global input indices
+    int32_t* out;            // packed rows, per-molecule local indices
+    uint8_t* attached;
+    unsigned* err;
+};
+
 template <int K>
-__device__ void sort_big_bucket(int4* __restrict__ T, int64_t a, int64_t b, int64_t* __restrict__ uniq_g) {
-    *uniq_g = sort_unique_bucket<K>(T, a, b);
+__device__ __forceinline__ void canon_row(const CanonOut& o, int64_t row, int4 t, int base) {
+    if (K < 4) t.w = -1;
+    if (K < 3) t.z = -1;
+    o.G[row] = t;
+    if (K == 4) {
+        reinterpret_cast<int4*>(o.out)[row] = make_int4(t.x - base, t.y - base, t.z - base, t.w - base);
+    } else {
+        o.out[row * K + 0] = t.x - base;
+        o.out[row * K + 1] = t.y - base;
+        if (K == 3) o.out[row * K + 2] = t.z - base;
+    }
+    o.attached[row] = 0;  // list items passed AC2 at their orthocentre
 }
 
 template <int K>
 __global__ void __launch_bounds__(CSORT_WARPS * 32) k_canon_sort(int4* __restrict__ T, const int64_t* __restrict__ off,
-                                                                  int64_t n, int64_t* __restrict__ uniq, bool unique) {
+                                                                  int64_t n, CanonOut o) {
     __shared__ SortSmem sm[CSORT_WARPS];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     SortSmem& S = sm[w];
@@ -256,9 +252,10 @@ __global__ void __launch_bounds__(CSORT_WARPS * 32) k_canon_sort(int4* __restric
     for (int64_t g = (int64_t)blockIdx.x * CSORT_WARPS + w; g < n; g += warps) {
         const int64_t a = off[g];
         const int64_t kb = off[g + 1] - a;
+        if (kb == 0) continue;
         const int k = kb > CSORT_MAX ? CSORT_MAX + 1 : (int)kb;
-        if (unique && k <= 32) {
-            // distinct items (nothing to merge), one per lane: each takes its rank among the others
+        const int base = (int)o.mol_off[o.mol_of[g]];
+        if (k <= 32) {
             int4 t = make_int4(0, 0, 0, 0);
             unsigned long long hi = ~0ull;
             unsigned lo = ~0u;
@@ -266,109 +263,41 @@ __global__ void __launch_bounds__(CSORT_WARPS * 32) k_canon_sort(int4* __restric
                 t = T[a + lane];
                 make_key<K>(t, hi, lo);
             }
-            int r = 0;
+            int r = 0, same = 0;
             for (int u = 0; u < k; u++) {
                 const unsigned long long hu = __shfl_sync(0xffffffffu, hi, u);
                 const unsigned lu = __shfl_sync(0xffffffffu, lo, u);
                 r += key_less<K, unsigned long long>(hu, lu, hi, lo) ? 1 : 0;
+                same += hu == hi && lu == lo ? 1 : 0;
             }
-            __syncwarp();
-            if (lane < k) T[a + r] = t;
-            if (lane == 0) uniq[g] = k;
-            __syncwarp();
+            if (lane < k) {
+                if (same != 1) atomicOr(o.err, DERR_INTERNAL);
+                canon_row<K>(o, a + r, t, base);
+            }
             continue;
         }
         if (k > CSORT_MAX) {
-            if (lane == 0) sort_big_bucket<K>(T, a, a + kb, &uniq[g]);
+            // rare: one lane, heap sort in place (O(k log k))
+            if (lane == 0 && sort_unique_bucket<K>(T, a, a + kb) != kb) atomicOr(o.err, DERR_INTERNAL);
             __syncwarp();
+            for (int64_t i = lane; i < kb; i += 32) canon_row<K>(o, a + i, T[a + i], base);
             continue;
         }
-        if (k <= 1) {
-            if (lane == 0) uniq[g] = k;
-            continue;
-        }
-        if (k <= 32) bitonic_place<K, 1>(S, T, a, k, lane);
-        else if (k <= 64) bitonic_place<K, 2>(S, T, a, k, lane);
+        if (k <= 64) bitonic_place<K, 2>(S, T, a, k, lane);
         else if (k <= 128) bitonic_place<K, 4>(S, T, a, k, lane);
         else bitonic_place<K, 8>(S, T, a, k, lane);
         __syncwarp();
-        // same tuple: equal keys without the flag bit (K <= 3), or equal (hi, lo)
-        auto same_at = [&](int x, int y) {
-            return K == 4 ? (S.ohi[x] == S.ohi[y] && S.olo[x] == S.olo[y]) : (S.ohi[x] >> 1) == (S.ohi[y] >> 1);
-        };
-        int base = 0;
-        for (int i0 = 0; i0 < k; i0 += 32) {
-            const int i = i0 + lane;
-            bool first = false;
-            int fl = 0;
-            if (i < k) {
-                first = i == 0 || !same_at(i, i - 1);
-                if (first) {
-                    fl = K == 4 ? 1 : (int)(S.ohi[i] & 1ull);
-                    for (int j = i + 1; j < k && same_at(j, i); j++) fl |= (int)(S.ohi[j] & 1ull);
-                }
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, first);
-            if (first) {
-                const int pos = base + __popc(bal & ((1u << lane) - 1u));
-                const unsigned long long hi = S.ohi[i];
-                int4 t;
-                t.x = (int)g;
-                if (K == 2) {
-                    t.y = (int)(hi >> 1);
-                    t.z = -1;
-                    t.w = fl;
-                } else if (K == 3) {
-                    t.y = (int)(hi >> 33);
-                    t.z = (int)((hi >> 1) & 0xffffffffull);
-                    t.w = fl;
-                } else {
-                    t.y = (int)(hi >> 32);
-                    t.z = (int)(unsigned)hi;
-                    t.w = (int)S.olo[i];
-                }
-                T[a + pos] = t;
-            }
-            base += __popc(bal);
+        for (int i = lane; i < k; i += 32) {
+            const unsigned long long hi = S.ohi[i];
+            if (i > 0 && S.ohi[i - 1] == hi && (K < 4 || S.olo[i - 1] == S.olo[i])) atomicOr(o.err, DERR_INTERNAL);
+            int4 t = make_int4((int)g, 0, 0, 0);
+            t.y = K == 2 ? (int)(unsigned)hi : (int)(hi >> 32);
+            if (K >= 3) t.z = (int)(unsigned)hi;
+            if (K == 4) t.w = (int)S.olo[i];
+            canon_row<K>(o, a + i, t, base);
         }
-        if (lane == 0) uniq[g] = base;
         __syncwarp();
     }
-}
-
-// Slot-parallel output: slot j of bucket g = T[j].x holds unique row j - off[g]
-// of the bucket when that is below uniq(g) = uoff[g+1] - uoff[g].
-struct CanonWriteArgs {
-    const int4* T;
-    int64_t total;
-    const int64_t* off;
-    const int64_t* uoff;
-    const int32_t* mol_of;   // input index -> molecule
-    const int64_t* mol_off;  // molecule -> first input index
-    int4* G;                 // canonical rows, global input indices
-    int32_t* out;            // packed rows, per-molecule local indices
-    uint8_t* attached;
-};
-
-template <int K>
-__global__ void k_canon_write(CanonWriteArgs a) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= a.total) return;
-    int4 t = a.T[j];
-    const int g = t.x;
-    const int64_t kk = j - a.off[g];
-    const int64_t u0 = a.uoff[g];
-    if (kk >= a.uoff[g + 1] - u0) return;
-    const int64_t row = u0 + kk;
-    const int flag = K == 4 ? 1 : t.w;
-    if (K < 4) t.w = -1;
-    a.G[row] = t;
-    const int base = (int)a.mol_off[a.mol_of[g]];
-    a.out[row * K + 0] = t.x - base;
-    a.out[row * K + 1] = t.y - base;
-    if (K >= 3) a.out[row * K + 2] = t.z - base;
-    if (K == 4) a.out[row * K + 3] = t.w - base;
-    a.attached[row] = flag ? 0 : 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -376,69 +305,27 @@ __global__ void k_canon_write(CanonWriteArgs a) {
 
 using Work = CanonWork;
 
-// the items were unique: the de-duplicated total must equal their number
-__global__ void k_check_total(const int64_t* __restrict__ total, int64_t want, unsigned* __restrict__ err) {
-    if (*total != want) atomicOr(err, DERR_INTERNAL);
-}
-
+// one list from items emitted once each: their number is the row count
 template <int K>
-static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, const int4* cof, int64_t nB,
-                       SimplexList& L, DevBuf& Gout, Work& w, cudaStream_t s, bool unique) {
+static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, SimplexList& L, DevBuf& Gout, Work& w,
+                       cudaStream_t s) {
     const int64_t n = c->n;
-    const int64_t total = nA + nB * (K + 1);
-    AC_TRY(w.T.reserve((size_t)(total + 1) * sizeof(int4), s));
+    AC_TRY(w.T.reserve((size_t)(nA + 1) * sizeof(int4), s));
     AC_TRY(w.cnt.reserve((size_t)(n + 1) * sizeof(int64_t), s));
-    AC_TRY(w.cursor.reserve((size_t)(n + 1) * sizeof(int64_t), s));
-    AC_TRY(w.uniq.reserve((size_t)(n + 1) * sizeof(int64_t), s));
-    AC_TRY(w.big.reserve((size_t)(n + 1), s));
     AC_TRY(L.v0_off.reserve((size_t)(n + 1) * sizeof(int64_t), s));
     int64_t* cnt = w.cnt.as<int64_t>();
+    int64_t* off = L.v0_off.as<int64_t>();  // the rows start where the buckets do
     AC_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(n + 1) * sizeof(int64_t), s));
-    AC_CUDA(cudaMemsetAsync(w.cursor.p, 0, (size_t)(n + 1) * sizeof(int64_t), s));
-    CanonArgs ca{a4, a2, nA, cof, nB, c->order.as<int32_t>(), total, cnt, cnt, w.cursor.as<unsigned long long>(),
-                 w.T.as<int4>()};
-    const unsigned gi = (unsigned)((total + 255) / 256);
-    if (total > 0) {
+    CanonArgs ca{a4, a2, nA, c->order.as<int32_t>(), cnt, off, w.T.as<int4>()};
+    const unsigned gi = (unsigned)((nA + 255) / 256);
+    if (nA > 0) {
         k_canon_count<K><<<gi, 256, 0, s>>>(ca);
         AC_LAUNCHED();
     }
-    AC_TRY(scan_exclusive_i64(c, cnt, cnt, n, s));  // bucket offsets, in place
-    int64_t* uniq = w.uniq.as<int64_t>();
-    if (total > 0) {
-        k_canon_scatter<K><<<gi, 256, 0, s>>>(ca);
-        AC_LAUNCHED();
-    }
-    if (n > 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        AC_CUDA(cudaGetDevice(&dev));
-        AC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        AC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_canon_sort<K>, CSORT_WARPS * 32, 0));
-        // one resident wave, buckets taken grid-stride
-        int64_t blocks = (n + CSORT_WARPS - 1) / CSORT_WARPS;
-        if (blocks > (int64_t)sms * (per_sm > 0 ? per_sm : 1)) blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-        k_canon_sort<K><<<(unsigned)blocks, CSORT_WARPS * 32, 0, s>>>(w.T.as<int4>(), cnt, n, uniq, unique);
-        AC_LAUNCHED();
-    }
-    int64_t* uoff = L.v0_off.as<int64_t>();
-    if (unique)  // every item is a row: the rows start where the buckets do
-        AC_CUDA(cudaMemcpyAsync(uoff, cnt, (size_t)(n + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    else
-        AC_TRY(scan_exclusive_i64(c, uniq, uoff, n, s));
-    int64_t count = L.count;  // a replay keeps the recorded build's count and checks it
-    if (c->replaying) {
-        AC_TRY(expect_i64(c, uoff + n, count, s));
-    } else if (unique) {
-        // items emitted once each (by their owner): their number is the count, checked on the device
-        count = total;
-        k_check_total<<<1, 1, 0, s>>>(uoff + n, total, &c->counters.as<DevCounters>()->err);
-        AC_LAUNCHED();
-    } else {
-        AC_CUDA(cudaMemcpyAsync(c->h_stage, uoff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        AC_TRY(sync_host(c, s));
-        count = c->h_stage[0];
-    }
-    L.count = count;
-    const size_t rows = (size_t)(count > 0 ? count : 1);
+    AC_TRY(scan_exclusive_i64(c, cnt, off, n, s));
+    if (c->replaying) AC_TRY(expect_i64(c, off + n, L.count, s));  // the recorded build's count
+    else L.count = nA;
+    const size_t rows = (size_t)(L.count > 0 ? L.count : 1);
     AC_TRY(L.tuples.reserve(rows * K * sizeof(int32_t), s));
     AC_TRY(L.attached.reserve(rows, s));
     AC_TRY(L.f.reserve(rows * sizeof(double), s));
@@ -446,21 +333,30 @@ static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, co
     AC_TRY(L.src_dim.reserve(rows, s));
     AC_TRY(L.src_idx.reserve(rows * sizeof(int64_t), s));
     AC_TRY(Gout.reserve(rows * sizeof(int4), s));
-    if (total > 0) {
-        CanonWriteArgs wa{w.T.as<int4>(), total, cnt, uoff, c->mol_of.as<int32_t>(), c->d_moloff.as<int64_t>(),
-                          Gout.as<int4>(), L.tuples.as<int32_t>(), L.attached.as<uint8_t>()};
-        k_canon_write<K><<<gi, 256, 0, s>>>(wa);
+    if (nA > 0) {
+        k_canon_scatter<K><<<gi, 256, 0, s>>>(ca);
+        AC_LAUNCHED();
+        int dev = 0, sms = 0, per_sm = 0;
+        AC_CUDA(cudaGetDevice(&dev));
+        AC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        AC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_canon_sort<K>, CSORT_WARPS * 32, 0));
+        // one resident wave, buckets taken grid-stride
+        int64_t blocks = (n + CSORT_WARPS - 1) / CSORT_WARPS;
+        if (blocks > (int64_t)sms * (per_sm > 0 ? per_sm : 1)) blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+        CanonOut o{c->mol_of.as<int32_t>(), c->d_moloff.as<int64_t>(), Gout.as<int4>(), L.tuples.as<int32_t>(),
+                   L.attached.as<uint8_t>(), &c->counters.as<DevCounters>()->err};
+        k_canon_sort<K><<<(unsigned)blocks, CSORT_WARPS * 32, 0, s>>>(w.T.as<int4>(), off, n, o);
         AC_LAUNCHED();
     }
     return AC_OK;
 }
 
-static int canon_dim(ac_ctx* c, int d, const int4* a4, const int2* a2, int64_t nA, const int4* cof, int64_t nB,
-                     SimplexList& L, DevBuf& Gout, Work& w, cudaStream_t s, bool unique = false) {
+static int canon_dim(ac_ctx* c, int d, const int4* a4, const int2* a2, int64_t nA, SimplexList& L, DevBuf& Gout, Work& w,
+                     cudaStream_t s) {
     switch (d) {
-        case 1: return canon_dim_k<2>(c, a4, a2, nA, cof, nB, L, Gout, w, s, unique);
-        case 2: return canon_dim_k<3>(c, a4, a2, nA, cof, nB, L, Gout, w, s, unique);
-        default: return canon_dim_k<4>(c, a4, a2, nA, cof, nB, L, Gout, w, s, unique);
+        case 1: return canon_dim_k<2>(c, a4, a2, nA, L, Gout, w, s);
+        case 2: return canon_dim_k<3>(c, a4, a2, nA, L, Gout, w, s);
+        default: return canon_dim_k<4>(c, a4, a2, nA, L, Gout, w, s);
     }
 }
 
@@ -627,20 +523,21 @@ static int canon_edges_by_marks(ac_ctx* c, cudaStream_t s) {
     const DevCounters& h = c->hc;
     const int64_t n = c->n;
     SimplexList& L = c->K[1];
-    Work& w = c->cw;
     const int words = (h.max_degree + 31) / 32 > 0 ? (h.max_degree + 31) / 32 : 1;
     const size_t nn = (size_t)(n > 0 ? n : 1);
+    // one buffer, emptied at once: row counts, the two masks, K^1's endpoint flags (for K^0)
     DevBuf& masks = c->scratch[2];
-    AC_TRY(masks.reserve(2 * nn * words * sizeof(unsigned), s));
-    AC_TRY(w.cnt.reserve((nn + 1) * sizeof(int64_t), s));
+    const size_t o_mask = nn * sizeof(int64_t), o_end = o_mask + 2 * nn * words * sizeof(unsigned);
+    AC_TRY(masks.reserve(o_end + nn, s));
     AC_TRY(L.v0_off.reserve((nn + 1) * sizeof(int64_t), s));
-    AC_CUDA(cudaMemsetAsync(masks.p, 0, 2 * nn * words * sizeof(unsigned), s));
-    int64_t* cnt = w.cnt.as<int64_t>();
-    AC_CUDA(cudaMemsetAsync(cnt, 0, nn * sizeof(int64_t), s));
+    AC_CUDA(cudaMemsetAsync(masks.p, 0, o_end + nn, s));
+    int64_t* cnt = masks.as<int64_t>();
+    unsigned* mask = reinterpret_cast<unsigned*>(masks.as<char>() + o_mask);
+    c->endpoint = masks.as<uint8_t>() + o_end;
     EdgeMarkArgs a{c->edge_pass.as<int2>(), (int64_t)h.n_edge_pass, c->Gbuf[2].as<int4>(), c->K[2].count,
                    c->order.as<int32_t>(), c->rank.as<int32_t>(), c->nb_cnt.as<int64_t>(), c->nb.as<int32_t>(),
-                   c->nb_stride, words, masks.as<unsigned>(), masks.as<unsigned>() + nn * words,
-                   reinterpret_cast<unsigned long long*>(cnt), &c->counters.as<DevCounters>()->err};
+                   c->nb_stride, words, mask, mask + nn * words, reinterpret_cast<unsigned long long*>(cnt),
+                   &c->counters.as<DevCounters>()->err};
     const int64_t items = a.nA + a.nB;
     if (items > 0) {
         k_edge_mark<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(a);
@@ -665,13 +562,11 @@ static int canon_edges_by_marks(ac_ctx* c, cudaStream_t s) {
     AC_TRY(L.src_dim.reserve(rows, s));
     AC_TRY(L.src_idx.reserve(rows * sizeof(int64_t), s));
     AC_TRY(c->Gbuf[1].reserve(rows * sizeof(int4), s));
-    AC_TRY(w.big.reserve(nn, s));  // endpoint flags of K^1, for K^0
-    AC_CUDA(cudaMemsetAsync(w.big.p, 0, nn, s));
     if (n > 0) {
         k_edge_write<<<(unsigned)((n + EW_WARPS - 1) / EW_WARPS), EW_WARPS * 32, 0, s>>>(a, n, uoff, c->mol_of.as<int32_t>(),
                                                                   c->d_moloff.as<int64_t>(), c->Gbuf[1].as<int4>(),
                                                                   L.tuples.as<int32_t>(), L.attached.as<uint8_t>(),
-                                                                  w.big.as<uint8_t>());
+                                                                  c->endpoint);
         AC_LAUNCHED();
     }
     return AC_OK;
@@ -887,23 +782,23 @@ static int canon_tris_by_marks(ac_ctx* c, cudaStream_t s) {
     const DevCounters& h = c->hc;
     const int64_t n = c->n;
     SimplexList& L = c->K[2];
-    Work& w = c->cw;
     const size_t nn = (size_t)(n > 0 ? n : 1);
     DevBuf& masks = c->scratch[2];
-    AC_TRY(w.cnt.reserve((nn + 1) * sizeof(int64_t), s));
     AC_TRY(L.v0_off.reserve((nn + 1) * sizeof(int64_t), s));
     // first mask word of each sorted position and their total: from the neighbour pass
     const int64_t* moff = c->pair_moff.as<int64_t>();
-    int64_t* cnt = w.cnt.as<int64_t>();
     const int64_t words = c->pair_words;
     const size_t mw = (size_t)(words > 0 ? words : 1);
-    AC_TRY(masks.reserve(2 * mw * sizeof(unsigned), s));
-    AC_CUDA(cudaMemsetAsync(masks.p, 0, 2 * mw * sizeof(unsigned), s));
-    AC_CUDA(cudaMemsetAsync(cnt, 0, nn * sizeof(int64_t), s));
+    // one buffer, emptied at once: row counts and the two masks
+    const size_t o_mask = nn * sizeof(int64_t), bytes = o_mask + 2 * mw * sizeof(unsigned);
+    AC_TRY(masks.reserve(bytes, s));
+    AC_CUDA(cudaMemsetAsync(masks.p, 0, bytes, s));
+    int64_t* cnt = masks.as<int64_t>();
+    unsigned* mask = reinterpret_cast<unsigned*>(masks.as<char>() + o_mask);
     TriMarkArgs a{c->tri_pass.as<int4>(), (int64_t)h.n_tri_pass, c->tet_out.as<int4>(), c->K[3].count,
                   c->order.as<int32_t>(), c->rank.as<int32_t>(), c->nb_cnt.as<int64_t>(), c->nb.as<int32_t>(),
-                  c->nb_stride, moff, masks.as<unsigned>(), masks.as<unsigned>() + mw,
-                  reinterpret_cast<unsigned long long*>(cnt), &c->counters.as<DevCounters>()->err};
+                  c->nb_stride, moff, mask, mask + mw, reinterpret_cast<unsigned long long*>(cnt),
+                  &c->counters.as<DevCounters>()->err};
     const int64_t items = a.nA + a.nB;
     if (items > 0) {
         k_tri_mark<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(a);
@@ -940,11 +835,18 @@ static int canon_tris_by_marks(ac_ctx* c, cudaStream_t s) {
 
 // Vertices (Step 5): K^0 = endpoints of K^1 (flagged by k_edge_write) + atoms
 // whose centre passes AC2.
-__global__ void k_vertex_flags(const uint8_t* __restrict__ endpoint, const uint8_t* __restrict__ vert_pass,
-                               const int32_t* __restrict__ rank, int64_t n, int64_t* __restrict__ inK) {
+struct VertexFlag {
+    const uint8_t* endpoint;
+    const uint8_t* vert_pass;
+    const int32_t* rank;
+    __device__ __forceinline__ long long operator()(int64_t g) const {
+        return endpoint[g] || vert_pass[rank[g]] ? 1 : 0;
+    }
+};
+
+__global__ void k_vertex_flags(VertexFlag f, int64_t n, int64_t* __restrict__ inK) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    inK[g] = (endpoint[g] || vert_pass[rank[g]]) ? 1 : 0;
+    if (g < n) inK[g] = f(g);
 }
 
 __global__ void k_vertex_write(const int64_t* __restrict__ voff, const uint8_t* __restrict__ vert_pass,
@@ -985,8 +887,7 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
     Work& w = c->cw;
     const int64_t n = c->n;
     // K^3
-    AC_TRY(canon_dim(c, 3, c->tet_out.as<int4>(), nullptr, (int64_t)h.n_tet_out, nullptr, 0, c->K[3], c->Gbuf[3], w, s,
-                     true));
+    AC_TRY(canon_dim(c, 3, c->tet_out.as<int4>(), nullptr, (int64_t)h.n_tet_out, c->K[3], c->Gbuf[3], w, s));
     AC_TRY(fork_orthosize(c, 3, s));
     AC_TRY(stage_mark(c, 4, s));
     // K^2 = unattached triangles + facets of K^3
@@ -1000,18 +901,21 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
     {
         SimplexList& L = c->K[0];
         size_t nn = (size_t)(n > 0 ? n : 1);
-        AC_TRY(w.big.reserve(nn, s));
-        AC_TRY(w.cnt.reserve((nn + 1) * sizeof(int64_t), s));
         AC_TRY(L.v0_off.reserve((nn + 1) * sizeof(int64_t), s));
-        uint8_t* endpoint = w.big.as<uint8_t>();  // set by k_edge_write
-        int64_t* inK = w.cnt.as<int64_t>();
-        if (n > 0) {
-            k_vertex_flags<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(endpoint, c->vert_pass.as<uint8_t>(),
-                                                                       c->rank.as<int32_t>(), n, inK);
-            AC_LAUNCHED();
-        }
         int64_t* voff = L.v0_off.as<int64_t>();
-        AC_TRY(scan_exclusive_i64(c, inK, voff, n, s));
+        const VertexFlag flag{c->endpoint, c->vert_pass.as<uint8_t>(), c->rank.as<int32_t>()};  // endpoint: k_edge_write
+        if (n > 0 && n <= SC_MAX) {
+            launch_small_scan(flag, reinterpret_cast<long long*>(voff), n, s);
+            AC_LAUNCHED();
+        } else {
+            AC_TRY(w.cnt.reserve((nn + 1) * sizeof(int64_t), s));
+            int64_t* inK = w.cnt.as<int64_t>();
+            if (n > 0) {
+                k_vertex_flags<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(flag, n, inK);
+                AC_LAUNCHED();
+            }
+            AC_TRY(scan_exclusive_i64(c, inK, voff, n, s));
+        }
         int64_t count = L.count;
         if (c->replaying) {
             AC_TRY(expect_i64(c, voff + n, count, s));
@@ -1044,9 +948,10 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
             int64_t m = (int64_t)h.n_cand_out[d];
             // each candidate is emitted once, by its owner
             AC_TRY(canon_dim(c, d, d >= 2 ? c->cand[d].as<int4>() : nullptr, d == 1 ? c->cand[1].as<int2>() : nullptr, m,
-                             nullptr, 0, c->C[d], c->CGbuf[d], w, s, true));
+                             c->C[d], c->CGbuf[d], w, s));
         }
     }
+    if (c->n_mol == 1) return AC_OK;  // its rows are the whole lists (finish_mol_rows)
     // per-molecule row ranges, copied to the host with the build's last transfer
     MolRowsArgs ma{};
     for (int d = 0; d < 4; d++) ma.v0_off[d] = c->K[d].v0_off.as<int64_t>();
@@ -1065,6 +970,12 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
 // Unpack the per-molecule row ranges once the stream has reached the end of the build.
 void finish_mol_rows(ac_ctx* c) {
     const size_t m1 = (size_t)c->n_mol + 1;
+    if (c->n_mol == 1) {
+        for (int d = 0; d < 4; d++) c->K[d].mol_off = {0, c->K[d].count};
+        if (c->pc.keep_candidates)
+            for (int d = 1; d <= 3; d++) c->C[d].mol_off = {0, c->C[d].count};
+        return;
+    }
     for (int d = 0; d < 4; d++) c->K[d].mol_off.assign(c->h_molrows + d * m1, c->h_molrows + (d + 1) * m1);
     if (c->pc.keep_candidates)
         for (int d = 1; d <= 3; d++)
@@ -1140,7 +1051,7 @@ __device__ void orthosize_rational(const int4* __restrict__ P, const int4& t, in
 __global__ void k_orthosize(const int4* __restrict__ P, const int4* __restrict__ G, int64_t m, int K,
                             const uint8_t* __restrict__ attached, double* __restrict__ os, double* __restrict__ f,
                             int8_t* __restrict__ src_dim, int64_t* __restrict__ src_idx,
-                            unsigned long long* __restrict__ fkey) {
+                            unsigned long long* __restrict__ fkey, unsigned long long* __restrict__ arg) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
     double v = orthosize_exact(P, G[j], K);
@@ -1148,7 +1059,8 @@ __global__ void k_orthosize(const int4* __restrict__ P, const int4* __restrict__
     src_dim[j] = (int8_t)(K - 1);
     src_idx[j] = j;
     f[j] = v;
-    if (fkey) fkey[j] = attached[j] ? ~0ull : 0ull;
+    fkey[j] = attached[j] ? ~0ull : 0ull;
+    if (arg) arg[j] = ~0ull;
 }
 
 __device__ __forceinline__ unsigned long long order_key(double x) {
@@ -1421,15 +1333,14 @@ static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
     cudaStream_t t = c->side;
     AC_CUDA(cudaStreamWaitEvent(t, c->ev_fork, 0));
     unsigned long long* keyb = c->fkey[d].as<unsigned long long>();
+    unsigned long long* argb = U ? c->fargs[d].as<unsigned long long>() : nullptr;
     k_orthosize<<<(unsigned)((m + 127) / 128), 128, 0, t>>>(c->P.as<int4>(), c->Gbuf[d].as<int4>(), m, d + 1,
                                                             L.attached.as<uint8_t>(), L.orthosize.as<double>(),
                                                             L.f.as<double>(), L.src_dim.as<int8_t>(),
-                                                            L.src_idx.as<int64_t>(), keyb);
+                                                            L.src_idx.as<int64_t>(), keyb, argb);
     AC_LAUNCHED();
     c->os_forked = true;
     if (!U) return copy_values_to_host(c, d, t);
-    unsigned long long* argb = c->fargs[d].as<unsigned long long>();
-    AC_CUDA(cudaMemsetAsync(argb, 0xff, (size_t)m * sizeof(unsigned long long), t));
     if (mu > 0) {
         const unsigned nbk = (unsigned)((mu + 127) / 128);
         int64_t* rows = c->frows[d].as<int64_t>();

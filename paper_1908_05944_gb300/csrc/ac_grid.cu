@@ -31,17 +31,21 @@ __global__ void k_cell_keys(const int4* __restrict__ P, const int32_t* __restric
     atomicAdd(&cell_cnt[c], 1u);
 }
 
+// cell_cnt counts down from the cells' sizes to 0
 __global__ void k_scatter(const uint32_t* __restrict__ cell_of, const uint32_t* __restrict__ cell_start, int64_t n,
-                          uint32_t* __restrict__ cursor, int32_t* __restrict__ order) {
+                          uint32_t* __restrict__ cell_cnt, int32_t* __restrict__ order) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     uint32_t c = cell_of[i];
-    uint32_t slot = cell_start[c] + atomicAdd(&cursor[c], 1u);
+    uint32_t slot = cell_start[c] + atomicSub(&cell_cnt[c], 1u) - 1u;
     order[slot] = (int32_t)i;
 }
 
-// Order each cell's run by input index (runs are short: a few atoms).
-__global__ void k_sort_cells(const uint32_t* __restrict__ cell_start, int64_t n_cells, int32_t* __restrict__ order) {
+// Order each cell's run by input index (runs are short: a few atoms) and gather
+// its atoms.
+__global__ void k_sort_gather(const uint32_t* __restrict__ cell_start, int64_t n_cells, int32_t* __restrict__ order,
+                              const int4* __restrict__ P, const int32_t* __restrict__ mol_of, int4* __restrict__ Ps,
+                              int32_t* __restrict__ mol_s, int32_t* __restrict__ rank) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n_cells) return;
     uint32_t a = cell_start[c], b = cell_start[c + 1];
@@ -54,17 +58,12 @@ __global__ void k_sort_cells(const uint32_t* __restrict__ cell_start, int64_t n_
         }
         order[j] = v;
     }
-}
-
-__global__ void k_gather(const int32_t* __restrict__ order, const int4* __restrict__ P,
-                         const int32_t* __restrict__ mol_of, int64_t n, int4* __restrict__ Ps,
-                         int32_t* __restrict__ mol_s, int32_t* __restrict__ rank) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    int32_t i = order[s];
-    Ps[s] = P[i];
-    mol_s[s] = mol_of[i];
-    rank[i] = (int32_t)s;
+    for (uint32_t s = a; s < b; s++) {
+        const int32_t i = order[s];
+        Ps[s] = P[i];
+        mol_s[s] = mol_of[i];
+        rank[i] = (int32_t)s;
+    }
 }
 
 int build_grid(ac_ctx* c, cudaStream_t s) {
@@ -89,13 +88,12 @@ int build_grid(ac_ctx* c, cudaStream_t s) {
                                    c->cell_of.as<uint32_t>(), cnt);
     AC_LAUNCHED();
     AC_TRY(scan_exclusive_u32_to_u32(c, cnt, start, c->n_cells, s));
-    AC_CUDA(cudaMemsetAsync(cnt, 0, (size_t)c->n_cells * sizeof(uint32_t), s));
     k_scatter<<<nb, 256, 0, s>>>(c->cell_of.as<uint32_t>(), start, n, cnt, c->order.as<int32_t>());
     AC_LAUNCHED();
-    k_sort_cells<<<(unsigned)((c->n_cells + 255) / 256), 256, 0, s>>>(start, c->n_cells, c->order.as<int32_t>());
-    AC_LAUNCHED();
-    k_gather<<<nb, 256, 0, s>>>(c->order.as<int32_t>(), c->P.as<int4>(), c->mol_of.as<int32_t>(), n, c->Ps.as<int4>(),
-                                c->mol_s.as<int32_t>(), c->rank.as<int32_t>());
+    k_sort_gather<<<(unsigned)((c->n_cells + 127) / 128), 128, 0, s>>>(start, c->n_cells, c->order.as<int32_t>(),
+                                                                       c->P.as<int4>(), c->mol_of.as<int32_t>(),
+                                                                       c->Ps.as<int4>(), c->mol_s.as<int32_t>(),
+                                                                       c->rank.as<int32_t>());
     AC_LAUNCHED();
     return AC_OK;
 }
@@ -164,14 +162,32 @@ __device__ __forceinline__ bool nb_meet(const int4& p, int64_t si, int32_t si32,
     }
 }
 
+// Work order of the per-atom pass: sorted positions by decreasing neighbour
+// count, so the costliest atoms start first and the kernel's tail is short; the
+// atoms with more than 64 neighbours form its head. Up to 64 neighbours the bins
+// are 16 wide: within a bin the order is nearly the grid's, and what the pass
+// emits together is near together (k_tri_mark); with one bin per count a 3.0 M
+// atom shell lost that, with a single bin the 100,000-atom pass had a longer
+// tail (768 -> 780 us).
+__device__ __forceinline__ int deg_bin(int64_t m) {
+    return m > 512 ? 258 : m > 256 ? 257 : m > 64 ? (int)m : ((int)m + 15) & ~15;
+}
+
+// MODE NB_COUNT and NB_PADDED also add up what the host sizes the next steps
+// by: pairs, largest count, words of the K^2 pair masks, degree histogram.
 template <int MODE, bool SMALL>
 __global__ void __launch_bounds__(NB_THREADS)
     k_neighbours(const int4* __restrict__ Ps, const int32_t* __restrict__ mol_s, const MolGrid* __restrict__ grids,
                  const uint32_t* __restrict__ cell_start, PredConst pc, int64_t n, int64_t* __restrict__ nb_cnt,
                  const int64_t* __restrict__ nb_off, int32_t* __restrict__ nb, DevCounters* __restrict__ cnt,
-                 int64_t* __restrict__ pw) {
+                 int64_t* __restrict__ pw, unsigned* __restrict__ hist) {
     const int64_t s = (int64_t)blockIdx.x * NB_THREADS + threadIdx.x;
-    int64_t count = 0;
+    int64_t count = 0, words = 0;
+    __shared__ unsigned b_hist[MODE != NB_CSR ? DEG_BINS : 1];
+    if (MODE != NB_CSR) {
+        for (int t = threadIdx.x; t < DEG_BINS; t += NB_THREADS) b_hist[t] = 0u;
+        __syncthreads();
+    }
     if (s < n) {
         const int4 p = Ps[s];
         const int64_t si = (int64_t)p.w + pc.A;
@@ -206,28 +222,38 @@ __global__ void __launch_bounds__(NB_THREADS)
         }
         if (MODE != NB_CSR) {
             nb_cnt[s] = count;
-            pw[s] = pair_mask_words((int)count);  // the K^2 pair mask of this atom
+            words = pair_mask_words((int)count);  // the K^2 pair mask of this atom
+            pw[s] = words;
+            atomicAdd(&b_hist[deg_bin(count)], 1u);
         }
     }
     if (MODE != NB_CSR) {
-        // one pair of atomics per block; every thread reaches here (no early exit above)
-        __shared__ unsigned long long b_tot[NB_THREADS / 32];
+        // one set of atomics per block; every thread reaches here (no early exit above)
+        __shared__ unsigned long long b_tot[NB_THREADS / 32], b_words[NB_THREADS / 32];
         __shared__ int b_max[NB_THREADS / 32];
         const unsigned wt = __reduce_add_sync(0xffffffffu, (unsigned)count);
         const unsigned wm = __reduce_max_sync(0xffffffffu, (unsigned)count);
+        unsigned long long ww = (unsigned long long)words;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, o);
         if ((threadIdx.x & 31) == 0) {
             b_tot[threadIdx.x >> 5] = wt;
             b_max[threadIdx.x >> 5] = (int)wm;
+            b_words[threadIdx.x >> 5] = ww;
         }
         __syncthreads();
+        for (int t = threadIdx.x; t < DEG_BINS; t += NB_THREADS)
+            if (b_hist[t]) atomicAdd(&hist[t], b_hist[t]);
         if (threadIdx.x == 0) {
-            unsigned long long tot = 0;
+            unsigned long long tot = 0, words_b = 0;
             int m = 0;
             for (int k = 0; k < NB_THREADS / 32; k++) {
                 tot += b_tot[k];
+                words_b += b_words[k];
                 m = max(m, b_max[k]);
             }
             if (tot) atomicAdd(&cnt->nb_sum, tot);
+            if (words_b) atomicAdd(&cnt->pair_words, words_b);
             atomicMax(&cnt->max_degree, m);
         }
     }
@@ -236,56 +262,32 @@ __global__ void __launch_bounds__(NB_THREADS)
 // Blocks of k_neighbours: one thread per atom.
 static unsigned neighbour_blocks(int64_t n) { return (unsigned)((n + NB_THREADS - 1) / NB_THREADS); }
 
-// Work order of the per-atom pass: sorted positions by decreasing neighbour
-// count (ties in any order), so the costliest atoms start first and the
-// kernel's tail is short; the atoms with more than 64 neighbours form its head.
-constexpr int DEG_BINS = 259;  // counts 0..256, 257 for 257..512, 258 for anything above
-
-__device__ __forceinline__ int deg_bin(int64_t m) { return m > 512 ? 258 : m > 256 ? 257 : m > 64 ? (int)m : ((int)m + 15) & ~15; }
-
-__global__ void k_deg_hist(const int64_t* __restrict__ cnt, int64_t n, unsigned* __restrict__ hist) {
-    __shared__ unsigned h[DEG_BINS];
-    for (int t = threadIdx.x; t < DEG_BINS; t += blockDim.x) h[t] = 0;
-    __syncthreads();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&h[deg_bin(cnt[i])], 1u);
-    __syncthreads();
-    for (int t = threadIdx.x; t < DEG_BINS; t += blockDim.x)
-        if (h[t]) atomicAdd(&hist[t], h[t]);
-}
-
-// start of each bin in decreasing order, and the head sizes (atoms with more
-// than 64, and more than 512, neighbours): one thread per bin
-__global__ void k_deg_starts(const unsigned* __restrict__ hist, unsigned* __restrict__ cursor,
-                             long long* __restrict__ n_wide) {
-    __shared__ unsigned h[DEG_BINS];
-    const int b = threadIdx.x;
-    if (b < DEG_BINS) h[b] = hist[b];
-    __syncthreads();
-    if (b >= DEG_BINS) return;
-    unsigned run = 0;
-    for (int q = DEG_BINS - 1; q > b; q--) run += h[q];
-    cursor[b] = run;
-    // atoms over 64, 512, 128 and 256 neighbours: the tiers of the per-atom pass
-    if (b == 65) n_wide[0] = run + h[65];
-    if (b == DEG_BINS - 1) n_wide[1] = h[DEG_BINS - 1];
-    if (b == 129) n_wide[2] = run + h[129];
-    if (b == DEG_BINS - 2) n_wide[3] = run + h[DEG_BINS - 2];
-}
-
-__global__ void k_deg_scatter(const int64_t* __restrict__ cnt, int64_t n, unsigned* __restrict__ cursor,
-                              int32_t* __restrict__ work) {
-    __shared__ unsigned h[DEG_BINS], base[DEG_BINS];
-    for (int t = threadIdx.x; t < DEG_BINS; t += blockDim.x) h[t] = 0;
+// Sorted positions by decreasing bin. A bin starts after the atoms of the bins
+// above it; the first block writes the sizes of the heads (the tiers of the
+// per-atom pass: more than 64, 512, 128 and 256 neighbours).
+__global__ void k_deg_scatter(const int64_t* __restrict__ cnt, int64_t n, const unsigned* __restrict__ hist,
+                              unsigned* __restrict__ cursor, int32_t* __restrict__ work, DevCounters* __restrict__ dc) {
+    __shared__ unsigned h[DEG_BINS], base[DEG_BINS], all[DEG_BINS];
+    for (int t = threadIdx.x; t < DEG_BINS; t += blockDim.x) {
+        h[t] = 0;
+        all[t] = hist[t];
+    }
     __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int b = i < n ? deg_bin(cnt[i]) : 0;
     const unsigned local = i < n ? atomicAdd(&h[b], 1u) : 0u;
     __syncthreads();
+    auto above = [&](int t) {
+        unsigned run = 0;
+        for (int q = t + 1; q < DEG_BINS; q++) run += all[q];
+        return run;
+    };
     for (int t = threadIdx.x; t < DEG_BINS; t += blockDim.x)
-        if (h[t]) base[t] = atomicAdd(&cursor[t], h[t]);
+        if (h[t]) base[t] = above(t) + atomicAdd(&cursor[t], h[t]);
     __syncthreads();
     if (i < n) work[base[b] + local] = (int32_t)i;
+    if (blockIdx.x == 0 && threadIdx.x < 4)
+        dc->n_over[threadIdx.x] = above(threadIdx.x == 0 ? 64 : threadIdx.x == 1 ? 257 : threadIdx.x == 2 ? 128 : 256);
 }
 
 // L(i) for every atom. With at most NB_STRIDE neighbours per atom (always so
@@ -314,31 +316,23 @@ int build_neighbours(ac_ctx* c, cudaStream_t s) {
     const GridView g{c->Ps.as<int4>(), c->mol_s.as<int32_t>(), c->grids.as<MolGrid>(), c->cell_start.as<uint32_t>()};
     AC_TRY(c->cw.cnt.reserve((size_t)(n + 1) * sizeof(int64_t), s));
     int64_t* pw = c->cw.cnt.as<int64_t>();
+    unsigned* hist = c->deg.as<unsigned>();  // emptied by k_init, with the cursors behind it
+    unsigned* cursor = hist + DEG_BINS;
     if (padded) {
         AC_TRY(c->nb.reserve((size_t)n * NB_STRIDE * sizeof(int32_t), s));
         auto k = small ? k_neighbours<NB_PADDED, true> : k_neighbours<NB_PADDED, false>;
-        k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, c->nb.as<int32_t>(), dc, pw);
+        k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, c->nb.as<int32_t>(), dc, pw,
+                                    hist);
     } else {
         auto k = small ? k_neighbours<NB_COUNT, true> : k_neighbours<NB_COUNT, false>;
-        k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, nullptr, dc, pw);
+        k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, nullptr, dc, pw, hist);
     }
     AC_LAUNCHED();
     // layout of the K^2 pair masks, from the words per atom
     AC_TRY(plan_pair_masks(c, pw, s));
     // work order from the counts (before a scan turns them into offsets)
     AC_TRY(c->work.reserve((size_t)n * sizeof(int32_t), s));
-    AC_TRY(c->deg.reserve(2 * DEG_BINS * sizeof(unsigned) + 64, s));
-    unsigned* hist = c->deg.as<unsigned>();
-    unsigned* cursor = hist + DEG_BINS;
-    static_assert((2 * DEG_BINS * sizeof(unsigned)) % 8 == 0, "head counts 8-aligned");
-    // atoms over 64 neighbours, over 512 (n_huge), over 128, over 256
-    long long* n_wide = reinterpret_cast<long long*>(hist + 2 * DEG_BINS);
-    AC_CUDA(cudaMemsetAsync(hist, 0, DEG_BINS * sizeof(unsigned), s));
-    k_deg_hist<<<nb, 128, 0, s>>>(cntp, n, hist);
-    AC_LAUNCHED();
-    k_deg_starts<<<1, (DEG_BINS + 31) / 32 * 32, 0, s>>>(hist, cursor, n_wide);
-    AC_LAUNCHED();
-    k_deg_scatter<<<nb, 128, 0, s>>>(cntp, n, cursor, c->work.as<int32_t>());
+    k_deg_scatter<<<nb, 128, 0, s>>>(cntp, n, hist, cursor, c->work.as<int32_t>(), dc);
     AC_LAUNCHED();
     int64_t total = 0;
     bool compact = !padded;
@@ -350,24 +344,20 @@ int build_neighbours(ac_ctx* c, cudaStream_t s) {
         c->n_w128 = c->rec.n_w128;
         c->n_w256 = c->rec.n_w256;
         AC_TRY(expect_u64(c, &dc->nb_sum, (unsigned long long)total, s));
-        AC_TRY(expect_i64(c, reinterpret_cast<const int64_t*>(n_wide), c->n_wide, s));
-        AC_TRY(expect_i64(c, reinterpret_cast<const int64_t*>(n_wide + 1), c->n_huge, s));
-        AC_TRY(expect_i64(c, reinterpret_cast<const int64_t*>(n_wide + 2), c->n_w128, s));
-        AC_TRY(expect_i64(c, reinterpret_cast<const int64_t*>(n_wide + 3), c->n_w256, s));
+        AC_TRY(expect_u64(c, &dc->n_over[0], (unsigned long long)c->n_wide, s));
+        AC_TRY(expect_u64(c, &dc->n_over[1], (unsigned long long)c->n_huge, s));
+        AC_TRY(expect_u64(c, &dc->n_over[2], (unsigned long long)c->n_w128, s));
+        AC_TRY(expect_u64(c, &dc->n_over[3], (unsigned long long)c->n_w256, s));
         AC_TRY(expect_i64(c, c->pair_moff.as<int64_t>() + n, c->pair_words, s));
     } else {
-        AC_CUDA(cudaMemcpyAsync(c->h_stage + 1, n_wide, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        AC_CUDA(cudaMemcpyAsync(c->h_stage + 3, n_wide + 1, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        AC_CUDA(cudaMemcpyAsync(c->h_stage + 2, c->pair_moff.as<int64_t>() + n, sizeof(int64_t),
-                                cudaMemcpyDeviceToHost, s));
         DevCounters h;
-        AC_TRY(read_counters(c, &h, s));  // also completes the copies above
+        AC_TRY(read_counters(c, &h, s));
         total = (int64_t)h.nb_sum;
-        c->n_wide = c->h_stage[1];
-        c->n_huge = c->h_stage[3];
-        c->n_w128 = c->h_stage[4];
-        c->n_w256 = c->h_stage[5];
-        c->pair_words = c->h_stage[2];
+        c->n_wide = (int64_t)h.n_over[0];
+        c->n_huge = (int64_t)h.n_over[1];
+        c->n_w128 = (int64_t)h.n_over[2];
+        c->n_w256 = (int64_t)h.n_over[3];
+        c->pair_words = (int64_t)h.pair_words;
         if (h.err & DERR_COINCIDENT)
             return fail(AC_ERR_DEGENERATE, "two centres coincide after quantisation to 1/1024 A");
         if (h.max_degree > NB_STRIDE) compact = true;  // rows too short: redo as compact lists
@@ -380,7 +370,7 @@ int build_neighbours(ac_ctx* c, cudaStream_t s) {
     AC_TRY(c->nb.reserve((size_t)(total > 0 ? total : 1) * sizeof(int32_t), s));
     auto k_fill = small ? k_neighbours<NB_CSR, true> : k_neighbours<NB_CSR, false>;
     k_fill<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, nullptr, cntp, c->nb.as<int32_t>(), dc,
-                              nullptr);
+                                     nullptr, nullptr);
     AC_LAUNCHED();
     return AC_OK;
 }

@@ -118,9 +118,18 @@ struct DevCounters {
     unsigned int err;
     int max_degree;
     int bad_index;
-    int pad;
+    int wmax;                         // largest quantised W
     unsigned long long nb_sum;        // neighbour pairs counted (sum of |L(i)|)
+    unsigned long long pair_words;    // words of the K^2 pair masks
+    unsigned long long n_over[4];     // atoms with more than 64, 512, 128, 256 neighbours
 };
+// The bounding boxes (6 int32 per molecule) follow the counters in one device
+// buffer, as in the page-locked readback block: one copy brings both.
+constexpr size_t BBOX_OFFSET = (sizeof(DevCounters) + 255) & ~(size_t)255;
+
+// Degree histogram and cursors of the work order (ac_grid.cu): counts 0..64 in
+// steps of 16, 65..256, 257 for 257..512, 258 for anything above.
+constexpr int DEG_BINS = 259;
 
 // Row length of the padded neighbour layout: L(i) at nb[i * NB_STRIDE ..]
 // when no atom has more neighbours, else a compact list at scanned offsets.
@@ -166,7 +175,7 @@ struct SimplexList {
 namespace ac {
 // Scratch of the canonicalisation, kept by the context so rebuilds allocate nothing.
 struct CanonWork {
-    DevBuf T, cnt, cursor, uniq, big;
+    DevBuf T, cnt, cursor;
 };
 
 // A size a replay checks on the device: *p (kind 0: int64, 1: uint64) equals
@@ -264,6 +273,7 @@ struct ac_ctx {
     ac::DevBuf frows[4];     // per-dimension facet rows of the cofaces (k_coface_min -> k_coface_arg)
     bool os_forked = false;  // k_orthosize launches on the side stream await their join
     int64_t pair_words = 0;  // words of the triangle pair masks (recorded for replays)
+    uint8_t* endpoint = nullptr;  // K^1's endpoint flags by input index (within scratch[2], this build's)
     ac::DevBuf pair_moff;    // first pair-mask word of each sorted position (n + 1)
     ac::DevBuf scan_tmp;
 

@@ -1598,10 +1598,9 @@ int run_local(ac_ctx* c, cudaStream_t s) {
             AC_TRY(c->cand[2].reserve((size_t)c->cap_cand[2] * sizeof(int4), s));
             AC_TRY(c->cand[3].reserve((size_t)c->cap_cand[3] * sizeof(int4), s));
         }
-        // zero the per-pass counters (keep max_degree and err)
+        // the per-pass counters start at zero (k_init); another attempt empties them again (max_degree and err stay)
         DevCounters* dc = c->counters.as<DevCounters>();
-        AC_CUDA(cudaMemsetAsync(dc, 0, offsetof(DevCounters, err), s));
-        AC_CUDA(cudaMemsetAsync(c->vert_pass.p, 0, nn, s));
+        if (attempt > 0) AC_CUDA(cudaMemsetAsync(dc, 0, offsetof(DevCounters, err), s));
         LocalArgs a;
         memset(&a, 0, sizeof(a));
         a.Ps = c->Ps.as<int4>();
