@@ -6,16 +6,12 @@
 // i. One warp handles one owner at a time and works entirely inside L(i), the
 // list of i's neighbours (atoms whose grown balls meet i's, ac_grid.cu), held
 // in shared memory as offsets q_x = P_x - P_i (exact integers, exact in FP32
-// because |q| <= 2h <= 2^13) and a_x = |q_x|^2 - W_x + W_i. Bitmasks over
-// positions in L(i) (WORDS 32-bit words, |L(i)| <= 32 * WORDS) carry:
-//   up       positions x > i with edge (i,x) in Sigma_ortho^1 (edge AC3 exact)
-//   M[p]     positions adjacent to p (grown balls meet), for p in up
-//   T[p]     positions k > p with triangle (i,p,k) in Sigma_ortho^2
-// Potential triangles are pairs (p,k), k in M[p] & up, k > p; potential
-// tetrahedra are (p,k,l) with l in T[p] & T[k]. Monotonicity of OrthoSize
-// (Section 4.3) makes this complete. Candidates are enumerated by random
-// access: per-row counts, a prefix sum, and candidate j -> row by binary
-// search -> vertex as the rank-th set bit, 32 candidates per warp step.
+// because |q| <= 2h <= 2^13) and a_x = |q_x|^2 - W_x + W_i. The n_up neighbours
+// x > i with edge (i,x) in Sigma_ortho^1 (edge AC3 exact) come first, positions
+// 0 .. n_up - 1; bitmasks over positions (WORDS 32-bit words, |L(i)| <= 32 *
+// WORDS) carry the rows M[p], p < n_up, of the positions adjacent to p (grown
+// balls meet). Potential triangles are pairs (p,k), p in M[k], p < k < n_up;
+// potential tetrahedra are (p,k,x) with x in M[p] & M[k], k < x < n_up.
 //
 // AC2 at the orthocentre c = P_i + y of sigma. Every ball x that violates it
 // (ties included) has pi(c, b_x) <= OrthoSize(sigma) <= alpha, so its grown
@@ -23,6 +19,29 @@
 // the candidates are M[p] & M[k] & M[l] (all of L(i) for the vertex i).
 //   Delta_x = pi(c, b_x) - pi(c, b_i) = a_x - 2 q_x . y;  AC2 fails iff some
 //   Delta_x < 0 (Delta_x = 0 is settled by the symbolic perturbation below).
+//
+// What is left of a simplex's witnesses. A simplex of the complex has a witness:
+// a point of equal power t <= alpha to its vertices with Delta_x >= 0 for every
+// ball x. It is one for each of its faces too. So:
+//   edge (i,p): the points of equal power within alpha are a disc, centre the
+//     edge's orthocentre c, radius rho, rho^2 = W_i + A - |y|^2. Over the disc
+//     Delta_x is largest at Delta_x(c) + 2 rho |q_x - (q_x.u) u|, u the edge's
+//     direction. If that is negative for one x, no simplex with this edge is in
+//     the complex (set kup holds the other edges).
+//   triangle (i,p,k): those points are the segment y + s n, n = q_p x q_k,
+//     |s| <= S, S^2 = (W_i + A - |y|^2) / |n|^2. Delta_x(y + s n) = Delta_x(y) -
+//     2 s g_x, g_x = q_x . n: each x cuts one end off. If nothing is left the
+//     triangle and everything over it is out.
+//   tetrahedron (i,p,k,x): its orthocentre is the point of the line with
+//     Delta_x = 0, s = Delta_x(y) / (2 g_x): AC3 holds iff |Delta_x(y)| <= 2 S
+//     |g_x|, and it is in K^3 only if that s is an end of what is left.
+// Every candidate of Sigma^2 and Sigma^3 is still decided (they are counted, and
+// listed on request), a tetrahedron by two dot products on its triangle's line;
+// but AC2 scans are left for free edges and triangles, and for the tetrahedra at
+// the ends of the segments: about one for every tetrahedron of K^3, where a scan
+// of every Sigma^3 tetrahedron at its own orthocentre made 470 tests per atom.
+// All of this prunes with bounds on the safe side; what survives is decided by
+// the tests below, so a wider bound costs time and nothing else.
 //
 // Bounded floating point. k_local evaluates y and every Delta_x in one
 // precision R (FP32 for AC_PRECISION_FILTERED, FP64 for
@@ -43,21 +62,35 @@
 //   edge: D = |q|^2 (|D~ - D| <= gamma_3 H^2), mu = a / (2D), y = mu q.
 // AC3 (|y|^2 <= W_i + A, since |y|^2 - W_i is OrthoSize): S~ = fl(|y~|^2),
 // |S~ - |y|^2| <= gamma_3 S~ (1 + gamma_3) + e_y (2|y~|_1 + 3 e_y); W_i + A <=
-// 2^24 is exact. AC2: |fl(Delta) - Delta| <= u|fl(Delta)|(1+u) + u A_m +
-// 2 gamma_3 H |y~| + 2 sqrt3 H e_y, and |y| <= h once AC3 holds, so a test is
-// decided when |fl(Delta)| > (K0 + K1 e_y)(1 + 1.01u), K0 = u A_m +
-// 2 gamma_3 H h, K1 = 2 sqrt3 H (1 + gamma_3).
+// 2^24 is exact. Delta by three FMAs from a_x with z = -2 y~ (exact): partial
+// sums stay below A_m + 2 H h (|y| <= h once AC3 holds), so |fl(Delta) - Delta|
+// <= u A_m + gamma_3 (A_m + 2 H h) + 2 sqrt3 H e_y, and a test is decided when
+// |fl(Delta)| > E = (K0 + K1 e_y)(1 + 1.01u), K0 = u A_m + gamma_3 (A_m + 2 H h),
+// K1 = 2 sqrt3 H (1 + gamma_3).
+//   On the line: |fl(g) - g| <= sqrt3 H e_C + gamma_3 H |n~|, and S |n| <= h, so
+//     Delta~ - 2 s g~ is within E_i = E + K2 (2S) + K3 of Delta(y + s n), K2 =
+//     sqrt3 H e_C, K3 = 12 u H h (2.4 gamma_3 H h for the second term, |n~| up to
+//     1.2 |n|, and the roundings of the comparisons). With det within rho of
+//     det~, 2S lies between s2lo and s2.
+//   In the disc: -Delta > 2 rho |q_perp| is compared squared, |q_perp|^2 = |q_x|^2
+//     - (q_x.u)^2 with an allowance of 64 u H^2 for every rounding in it.
 // A simplex whose AC3, or whose AC2 with no decided violator, stays open is
-// appended to a pending list (an undecided triangle still counts as potential
-// for the enumeration of tetrahedra: a superset is harmless there). Two kernels
-// settle the pending simplices: k_resolve_prep, one thread per simplex, takes
-// the exact AC3 in 128-bit integers and the FP64 orthocentre from the exact
-// integer minors (relative error <= 4.0001 u_64 per component of y); then
-// k_resolve_scan, a group of lanes per simplex whose AC3 holds, makes every AC2
-// test in FP32 and FP64 from that orthocentre and, where both are undecided,
-// in exact 128-bit integers. Keeping the exact arithmetic out of k_local keeps
-// its register budget small.
+// appended to a pending list (the tetrahedra over an undecided triangle are
+// tested all the same). Two kernels settle the pending simplices: k_resolve_prep,
+// one thread per simplex, takes the exact AC3 in 128-bit integers and the FP64
+// orthocentre from the exact integer minors (relative error <= 4.0001 u_64 per
+// component of y); then k_resolve_scan, a group of lanes per simplex whose AC3
+// holds, makes every AC2 test in FP32 and FP64 from that orthocentre and, where
+// both are undecided, in exact 128-bit integers. Keeping the exact arithmetic out
+// of k_local keeps its register budget small.
 // Edge AC3 and the vertex test are exact 64-bit integers in every mode.
+//
+// What bounds it: instruction issue (81 % of the issue slots, 18 of 32 lanes).
+// 100,000-atom probe globule, 64-bit rows: 727 us and 7,380 warp instructions per
+// atom, of which loading and ranking 670, adjacency rows 650, edges 1,020, lines
+// and enumeration 1,290, segments 1,580, AC3 on the lines 1,600, tetrahedra 560
+// (1,020 us and 10,500 when every Sigma^3 tetrahedron had its own orthocentre and
+// scan).
 //
 // Ties (Section 2, symbolic perturbation): squared radii W_k + eps_k with eps_k
 // falling steeply in the INPUT index k. Delta_x is affine in the weights; its
@@ -87,7 +120,7 @@ struct WarpSmem {
     static constexpr int SH = WORDS > 8 ? 10 : 8;
     static constexpr unsigned PM = (1u << SH) - 1u;
     float4 qf[M];   // (qx, qy, qz, a_x): coordinates exact, a_x rounded once
-    int ai[M];      // a_x exact
+    alignas(16) int ai[M];  // sort keys, then a_x exact
     float rs[M];    // sqrt(W_x + A) rounded up
     int idx[M];     // sorted position
     unsigned Mrow[M][WORDS];
@@ -634,28 +667,47 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
             }
             n_up += __popc(__ballot_sync(FULL, upper));
         }
+        if (WORDS <= 2 && lane < 4 && m + lane < MAXM) S.ai[m + lane] = -1;  // past the end: above every key
         __syncwarp();
         int xr[WORDS], rr[WORDS];
+        if constexpr (WORDS <= 2) {
+            // a lane's keys against all of them, four per load
+            unsigned De[WORDS];
 #pragma unroll
-        for (int w = 0; w < WORDS; w++) {
-            const int e = 32 * w + lane;
-            xr[w] = -1;
-            rr[w] = 0;
-            if (w < nw && e < m) {
-                const unsigned De = (unsigned)S.ai[e];
-                int rank = 0;
-                if constexpr (WORDS <= 2) {
-#pragma unroll 4
-                    for (int f = 0; f < m; f++) rank += (unsigned)S.ai[f] < De ? 1 : 0;
-                } else {
+            for (int w = 0; w < WORDS; w++) {
+                const int e = 32 * w + lane;
+                De[w] = e < m ? (unsigned)S.ai[e] : 0u;
+                xr[w] = e < m ? S.idx[e] : -1;
+                rr[w] = 0;
+            }
+#pragma unroll 2
+            for (int f = 0; f < m; f += 4) {
+                const int4 k = *reinterpret_cast<const int4*>(&S.ai[f]);
+#pragma unroll
+                for (int w = 0; w < WORDS; w++) {
+                    rr[w] += (unsigned)k.x < De[w] ? 1 : 0;
+                    rr[w] += (unsigned)k.y < De[w] ? 1 : 0;
+                    rr[w] += (unsigned)k.z < De[w] ? 1 : 0;
+                    rr[w] += (unsigned)k.w < De[w] ? 1 : 0;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int w = 0; w < WORDS; w++) {
+                const int e = 32 * w + lane;
+                xr[w] = -1;
+                rr[w] = 0;
+                if (w < nw && e < m) {
+                    const unsigned De = (unsigned)S.ai[e];
+                    int rank = 0;
 #pragma unroll 4
                     for (int f = 0; f < m; f++) {
                         const unsigned Df = (unsigned)S.ai[f];
                         rank += (Df < De || (Df == De && f < e)) ? 1 : 0;
                     }
+                    xr[w] = S.idx[e];
+                    rr[w] = rank;
                 }
-                xr[w] = S.idx[e];
-                rr[w] = rank;
             }
         }
         __syncwarp();
@@ -692,31 +744,34 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
         // relation: |q_e - q_p|^2 rounded down <= (sqrt s_p + sqrt s_e)^2 rounded up
         // keeps every pair whose grown balls meet (and a few more at the margin).
         if constexpr (WORDS <= 2) {
-            // each lane keeps its columns in registers across the rows
+            // Each lane keeps its columns in registers across the rows: lane L column
+            // 31 - L of every word, so that a ballot is the mask word as it stands. A
+            // column past the end lies out of every ball's reach.
             float cx[WORDS], cy[WORDS], cz[WORDS], cr[WORDS];
-            bool cv[WORDS];
 #pragma unroll
             for (int w = 0; w < WORDS; w++) {
-                const int e = 32 * w + lane;
-                cv[w] = w < nw && e < m;
-                const float4 qe = S.qf[cv[w] ? e : 0];
-                cx[w] = qe.x;
+                const int e = 32 * w + 31 - lane;
+                const float4 qe = S.qf[e < m ? e : 0];
+                cx[w] = e < m ? qe.x : 1e30f;
                 cy[w] = qe.y;
                 cz[w] = qe.z;
-                cr[w] = S.rs[cv[w] ? e : 0];
+                cr[w] = S.rs[e < m ? e : 0];
             }
 #pragma unroll 1
             for (int p = 0; p < n_up; p++) {
                 const float4 qp = S.qf[p];
                 const float rp = S.rs[p];
+                unsigned b[WORDS];
 #pragma unroll
                 for (int w = 0; w < WORDS; w++) {
                     const float dx = cx[w] - qp.x, dy = cy[w] - qp.y, dz = cz[w] - qp.z;  // exact: |.| <= 2^14
                     const float d2 = __fmaf_rd(dz, dz, __fmaf_rd(dy, dy, __fmul_rd(dx, dx)));
                     const float rr = __fadd_ru(rp, cr[w]);
-                    const bool adj = cv[w] && 32 * w + lane != p && d2 <= __fmul_ru(rr, rr);
-                    const unsigned b = __ballot_sync(FULL, adj);  // words past nw come out empty
-                    if (lane == 0) S.Mrow[p][w] = __brev(b);
+                    b[w] = __ballot_sync(FULL, d2 > 0.0f && d2 <= __fmul_ru(rr, rr));  // p is not its own neighbour
+                }
+                if (lane == 0) {
+#pragma unroll
+                    for (int w = 0; w < WORDS; w++) S.Mrow[p][w] = b[w];
                 }
             }
         } else {
@@ -1000,7 +1055,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                             }
                         }
                     }
-                    __syncwarp();
+                    if (!__any_sync(FULL, pass || pend || (keep && keep_it))) continue;  // nothing to append
                     const int4 item = make_int4(i, valid ? S.idx[pp] : 0, valid ? S.idx[kk] : 0, 0);
                     if (keep)
                         append_direct(keep_it, item, A.cand2, &cnt->n_cand_out[2], A.cap_cand[2], &cnt->err,
