@@ -85,12 +85,16 @@
 // of k_local keeps its register budget small.
 // Edge AC3 and the vertex test are exact 64-bit integers in every mode.
 //
-// What bounds it: instruction issue (81 % of the issue slots, 18 of 32 lanes).
+// What bounds it in FP32: instruction issue (81 % of the issue slots, 18 of 32 lanes).
 // 100,000-atom probe globule, 64-bit rows: 727 us and 7,380 warp instructions per
 // atom, of which loading and ranking 670, adjacency rows 650, edges 1,020, lines
 // and enumeration 1,290, segments 1,580, AC3 on the lines 1,600, tetrahedra 560
 // (1,020 us and 10,500 when every Sigma^3 tetrahedron had its own orthocentre and
 // scan).
+// In FP64: the FP64 pipe. Only the predicates use it (about 1,000 FP64 warp
+// instructions per atom): pruning runs in FP32, the error bounds of the lines in
+// FP32, the points come as FP64 from shared memory. 5.6 ms for the same globule
+// (18.1 ms with every Sigma^3 scan, bounds and conversions on the FP64 pipe).
 //
 // Ties (Section 2, symbolic perturbation): squared radii W_k + eps_k with eps_k
 // falling steeply in the INPUT index k. Delta_x is affine in the weights; its
@@ -113,14 +117,23 @@ constexpr int STAGE = 32;
 constexpr int CAND_CAP = 256;  // triangle candidates written out per batch
 constexpr unsigned TET_OPEN = 1u << 31;  // of a code in tl: AC3 not decided yet
 
-template <int WORDS>
-struct WarpSmem {
+// FP64 copies of the offsets and a_x, for the FP64 kernels only (four conversions
+// per candidate would run on the FP64 pipe they are bound by)
+template <int M, class R>
+struct PointsD {};
+template <int M>
+struct PointsD<M, double> {
+    double2 qd[M][2];  // (qx, qy), (qz, a_x)
+};
+
+template <int WORDS, class R>
+struct WarpSmem : PointsD<32 * WORDS, R> {
     static constexpr int M = 32 * WORDS;
     // row positions take 8 bits up to 256 neighbours, 10 bits beyond
     static constexpr int SH = WORDS > 8 ? 10 : 8;
     static constexpr unsigned PM = (1u << SH) - 1u;
     float4 qf[M];   // (qx, qy, qz, a_x): coordinates exact, a_x rounded once
-    alignas(16) int ai[M];  // sort keys, then a_x exact
+    alignas(16) int ai[M];  // sort keys
     float rs[M];    // sqrt(W_x + A) rounded up
     int idx[M];     // sorted position
     unsigned Mrow[M][WORDS];
@@ -136,7 +149,7 @@ struct WarpSmem {
 };
 
 // Eight warps of 64-bit rows must fit four blocks per SM (228 KB, 1 KB reserved per block).
-static_assert(sizeof(WarpSmem<2>) * 8 <= 56 * 1024, "narrow per-atom kernel: 4 blocks of 8 warps per SM");
+static_assert(sizeof(WarpSmem<2, float>) * 8 <= 56 * 1024, "narrow per-atom kernel: 4 blocks of 8 warps per SM");
 
 // Constants of the bounds for one precision (derivation in the header comment).
 template <class R>
@@ -173,6 +186,7 @@ struct LocalArgs {
     PredConst pc;
     Bounds<float> b32;
     Bounds<double> b64;
+    Bounds<float> b64f;  // the FP64 constants rounded up to FP32
     float perp_err;  // >= the rounding errors of |q_x|^2 - (q_x.u)^2 (edge discs)
     // FP64 thresholds of the resolve kernel (y from exact minors)
     double tet_eps64, tri_k0_64, tri_k1_64;
@@ -245,13 +259,16 @@ struct P4 {
     R x, y, z, w;  // offset from P_i and a_x
 };
 
-// Position e of L(i) in precision R: FP32 uses the rounded a_x; FP64 takes the
-// exact coordinates from FP32 and a_x exactly from the integer copy.
-template <class R, int WORDS>
-__device__ __forceinline__ P4<R> point(const WarpSmem<WORDS>& S, int e) {
-    const float4 v = S.qf[e];
-    if (sizeof(R) == 4) return {(R)v.x, (R)v.y, (R)v.z, (R)v.w};
-    return {(R)v.x, (R)v.y, (R)v.z, (R)S.ai[e]};
+// Position e of L(i) in precision R: exact but for FP32's a_x, which is rounded once.
+template <class R, class SM>
+__device__ __forceinline__ P4<R> point(const SM& S, int e) {
+    if constexpr (sizeof(R) == 4) {
+        const float4 v = S.qf[e];
+        return {v.x, v.y, v.z, v.w};
+    } else {
+        const double2 a = S.qd[e][0], b = S.qd[e][1];
+        return {a.x, a.y, b.x, b.y};
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -463,61 +480,142 @@ __device__ __forceinline__ float sqrt_dn(float x) {
 // The triangle's line of equal power, y + s n with n = q_1 x q_2, and the part
 // of it inside the grown balls of its vertices, |s| <= S (header comment).
 template <class R>
-struct TriLine {
-    R z0, z1, z2, n0, n1, n2;  // z = -2 y
-    R E;           // bound on |Delta~ - Delta| at y
-    R Ei;          // bound on |(Delta~ - 2 s g~) - Delta(y + s n)|, |s| <= S
-    R s2lo;        // <= 2 S
-    float s2;      // >= 2 S
+struct TriLine;
+
+template <>
+struct TriLine<float> {
+    float z0, z1, z2, n0, n1, n2;  // z = -2 y
+    float E;         // bound on |Delta~ - Delta| at y
+    float Ei;        // bound on |(Delta~ - 2 s g~) - Delta(y + s n)|, |s| <= S
+    float s2lo, s2;  // bounds of 2 S
     int ac3;
+    __device__ __forceinline__ void undecided() {  // every test on this line is
+        z0 = z1 = z2 = n0 = n1 = n2 = s2lo = s2 = 0.0f;
+        E = Ei = INFINITY;
+        ac3 = 0;
+    }
+    // AC3 of the tetrahedron with Delta~ = d, g~ = g: |Delta| <= 2 S |g|; sets bit in `in` or `out` if decided
+    __device__ __forceinline__ void tet_ac3(float d, float g, unsigned bit, unsigned& in, unsigned& out) const {
+        if (fabsf(d) < __fmaf_rd(fabsf(g), s2lo, -Ei)) in |= bit;
+        if (fabsf(d) > __fmaf_ru(fabsf(g), s2, Ei)) out |= bit;
+    }
 };
 
-template <class R>
-__device__ __forceinline__ TriLine<R> tri_line(const P4<R>& q1, const P4<R>& q2, R T, const Bounds<R>& B) {
-    using A = Ar<R>;
-    TriLine<R> L;
-    const R g11 = A::fma(q1.z, q1.z, A::fma(q1.y, q1.y, A::mul(q1.x, q1.x)));
-    const R g22 = A::fma(q2.z, q2.z, A::fma(q2.y, q2.y, A::mul(q2.x, q2.x)));
-    const R g12 = A::fma(q1.z, q2.z, A::fma(q1.y, q2.y, A::mul(q1.x, q2.x)));
-    const R det = A::fma(g11, g22, -A::mul(g12, g12));
-    const R r = A::rcp(R(2) * det);
-    const R inv = A::mul_up(A::abs(r), B.two_up);  // >= 1/|det~|
-    const R rho = A::mul_up(B.eDet, inv);
-    if (!(rho <= R(0.125))) {  // every test on this line is undecided
-        L.z0 = L.z1 = L.z2 = L.n0 = L.n1 = L.n2 = L.s2lo = R(0);
-        L.s2 = 0.0f;
-        L.E = L.Ei = R(INFINITY);
-        L.ac3 = 0;
+template <>
+struct TriLine<double> {
+    double z0, z1, z2, n0, n1, n2;
+    double E;
+    double s2mid, W;  // 2 S |g| is within W - E_i of s2mid |g|
+    int ac3;
+    __device__ __forceinline__ void undecided() {
+        z0 = z1 = z2 = n0 = n1 = n2 = s2mid = 0.0;
+        E = W = INFINITY;
+        ac3 = 0;
+    }
+    __device__ __forceinline__ void tet_ac3(double d, double g, unsigned bit, unsigned& in, unsigned& out) const {
+        const double v = __fma_rn(fabs(g), s2mid, -fabs(d));
+        if (fabs(v) > W) (__double2hiint(v) >= 0 ? in : out) |= bit;
+    }
+};
+
+__device__ __forceinline__ TriLine<float> tri_line(const P4<float>& q1, const P4<float>& q2, float T,
+                                                   const Bounds<float>& B) {
+    using A = Ar<float>;
+    TriLine<float> L;
+    const float g11 = A::fma(q1.z, q1.z, A::fma(q1.y, q1.y, A::mul(q1.x, q1.x)));
+    const float g22 = A::fma(q2.z, q2.z, A::fma(q2.y, q2.y, A::mul(q2.x, q2.x)));
+    const float g12 = A::fma(q1.z, q2.z, A::fma(q1.y, q2.y, A::mul(q1.x, q2.x)));
+    const float det = A::fma(g11, g22, -A::mul(g12, g12));
+    const float r = A::rcp(2.0f * det);
+    const float inv = A::mul_up(A::abs(r), B.two_up);  // >= 1/|det~|
+    const float rho = A::mul_up(B.eDet, inv);
+    if (!(rho <= 0.125f)) {
+        L.undecided();
         return L;
     }
-    Ortho<R> o;
-    const R n1 = A::fma(g22, q1.w, -A::mul(g12, q2.w));
-    const R n2 = A::fma(g11, q2.w, -A::mul(g12, q1.w));
-    const R m1 = A::mul(n1, r), m2 = A::mul(n2, r);
-    const R en = A::mul_up(B.cn, A::add_up(A::abs(q1.w), A::abs(q2.w)));
-    const R emu = quotient_bound(en, inv, A::max(A::abs(m1), A::abs(m2)), rho, B);
+    Ortho<float> o;
+    const float n1 = A::fma(g22, q1.w, -A::mul(g12, q2.w));
+    const float n2 = A::fma(g11, q2.w, -A::mul(g12, q1.w));
+    const float m1 = A::mul(n1, r), m2 = A::mul(n2, r);
+    const float en = A::mul_up(B.cn, A::add_up(A::abs(q1.w), A::abs(q2.w)));
+    const float emu = quotient_bound(en, inv, A::max(A::abs(m1), A::abs(m2)), rho, B);
     o.y0 = A::fma(m1, q1.x, A::mul(m2, q2.x));
     o.y1 = A::fma(m1, q1.y, A::mul(m2, q2.y));
     o.y2 = A::fma(m1, q1.z, A::mul(m2, q2.z));
-    o.ey = A::mul_up(B.H, A::fma_up(R(2), emu, A::mul_up(B.ky, A::add_up(A::abs(m1), A::abs(m2)))));
-    R S, eS;
+    o.ey = A::mul_up(B.H, A::fma_up(2.0f, emu, A::mul_up(B.ky, A::add_up(A::abs(m1), A::abs(m2)))));
+    float S, eS;
     norm2(o, B, S, eS);
     L.ac3 = ac3_of(S, eS, T);
-    L.z0 = R(-2) * o.y0;
-    L.z1 = R(-2) * o.y1;
-    L.z2 = R(-2) * o.y2;
+    L.z0 = -2.0f * o.y0;
+    L.z1 = -2.0f * o.y1;
+    L.z2 = -2.0f * o.y2;
     L.n0 = cross_c(q1.y, q2.z, q1.z, q2.y);
     L.n1 = cross_c(q1.z, q2.x, q1.x, q2.z);
     L.n2 = cross_c(q1.x, q2.y, q1.y, q2.x);
     // S^2 = (T - |y|^2) / det, 1 / det between inv (1 - 64 u) (1 - rho) and inv (1 + 1.2 rho)
-    const R t_up = A::max(A::add_up(A::add_up(T, -S), eS), R(0));
-    const R t_lo = A::max(A::sub_dn(A::sub_dn(T, S), eS), R(0));
-    const R s2_up = A::mul_up(A::mul_up(t_up, inv), A::fma_up(R(1.2), rho, R(1)));
-    const R s2_lo = A::mul_dn(A::mul_dn(t_lo, A::mul_dn(inv, B.inv_lo)), A::sub_dn(R(1), rho));
-    L.s2 = 2.0f * sqrt_up(A::to_f32_up(s2_up));
-    L.s2lo = R(2) * R(sqrt_dn(A::to_f32_dn(s2_lo)));
+    const float t_up = A::max(A::add_up(A::add_up(T, -S), eS), 0.0f);
+    const float t_lo = A::max(A::sub_dn(A::sub_dn(T, S), eS), 0.0f);
+    const float s2_up = A::mul_up(A::mul_up(t_up, inv), A::fma_up(1.2f, rho, 1.0f));
+    const float s2_lo = A::mul_dn(A::mul_dn(t_lo, A::mul_dn(inv, B.inv_lo)), A::sub_dn(1.0f, rho));
+    L.s2 = 2.0f * sqrt_up(s2_up);
+    L.s2lo = 2.0f * sqrt_dn(s2_lo);
     L.E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);
-    L.Ei = A::add_up(A::fma_up(B.K2, R(L.s2), B.K3), L.E);
+    L.Ei = A::add_up(A::fma_up(B.K2, L.s2, B.K3), L.E);
+    return L;
+}
+
+// The same in FP64. The FP64 pipe is 1/64 of the FP32 one and bounds the kernel,
+// so only what the predicates rest on runs there (about 45 operations); the error
+// bounds (B: the FP64 constants rounded up to FP32; their 1 + k comes out as 1
+// there, hence the factors 1 + 2^-18) run in FP32 beside it. f1, f2: FP32 copies
+// of q1, q2.
+__device__ __forceinline__ TriLine<double> tri_line(const P4<double>& q1, const P4<double>& q2, const float4& f1,
+                                                    const float4& f2, double T, float Tf, const Bounds<float>& B) {
+    using A = Ar<double>;
+    using F = Ar<float>;
+    constexpr float more = 1.0f + 0x1p-18f;
+    TriLine<double> L;
+    const double g11 = A::fma(q1.z, q1.z, A::fma(q1.y, q1.y, A::mul(q1.x, q1.x)));
+    const double g22 = A::fma(q2.z, q2.z, A::fma(q2.y, q2.y, A::mul(q2.x, q2.x)));
+    const double g12 = A::fma(q1.z, q2.z, A::fma(q1.y, q2.y, A::mul(q1.x, q2.x)));
+    const double det = A::fma(g11, g22, -A::mul(g12, g12));
+    const double r = A::rcp(-det);  // -2 / (2 det): M = -2 mu below
+    const float inv = F::mul_up(F::mul_up(A::to_f32_up(A::abs(r)), B.two_up), 0.5f * more);  // >= 1/|det~|
+    const float rho = F::mul_up(B.eDet, inv);
+    if (!(rho <= 0.125f)) {
+        L.undecided();
+        return L;
+    }
+    const double M1 = A::mul(A::fma(g22, q1.w, -A::mul(g12, q2.w)), r);
+    const double M2 = A::mul(A::fma(g11, q2.w, -A::mul(g12, q1.w)), r);
+    L.z0 = A::fma(M1, q1.x, A::mul(M2, q2.x));
+    L.z1 = A::fma(M1, q1.y, A::mul(M2, q2.y));
+    L.z2 = A::fma(M1, q1.z, A::mul(M2, q2.z));
+    const float m1 = 0.5f * A::to_f32_up(A::abs(M1)), m2 = 0.5f * A::to_f32_up(A::abs(M2));
+    const float en = F::mul_up(B.cn, F::mul_up(F::add_up(fabsf(f1.w), fabsf(f2.w)), more));
+    const float emu = F::mul_up(quotient_bound(en, inv, F::max(m1, m2), rho, B), more);
+    const float ey = F::mul_up(F::mul_up(B.H, F::fma_up(2.0f, emu, F::mul_up(B.ky, F::add_up(m1, m2)))), more);
+    // |y|^2 - T in one chain from -4 T: rounding below gamma_3 (T + |y|^2)
+    const float dif = 0.25f * (float)A::fma(L.z2, L.z2, A::fma(L.z1, L.z1, A::fma(L.z0, L.z0, -4.0 * T)));
+    const float ad = fabsf(dif), yy = F::mul_up(F::add_up(Tf, ad), more);  // yy >= |y~|^2
+    const float l1 = 1.7321f * sqrt_up(yy);
+    const float eS = F::mul_up(F::fma_up(0x1p-22f, ad,
+                                         F::fma_up(ey, F::fma_up(3.0f, ey, F::mul_up(2.0f, l1)),
+                                                   F::mul_up(B.g3s, F::add_up(Tf, yy)))), more);
+    L.ac3 = dif > eS ? -1 : dif < -eS ? 1 : 0;
+    L.n0 = cross_c(q1.y, q2.z, q1.z, q2.y);
+    L.n1 = cross_c(q1.z, q2.x, q1.x, q2.z);
+    L.n2 = cross_c(q1.x, q2.y, q1.y, q2.x);
+    const float t_up = F::max(F::add_up(-dif, eS), 0.0f), t_lo = F::max(F::sub_dn(-dif, eS), 0.0f);
+    const float s_hi = sqrt_up(F::mul_up(F::mul_up(t_up, inv), F::fma_up(1.2f, rho, 1.0f)));
+    const float s_lo = sqrt_dn(F::mul_dn(F::mul_dn(t_lo, F::mul_dn(inv, 1.0f - 0x1p-16f)), F::sub_dn(1.0f, rho)));
+    const float E = F::mul_up(F::fma_up(B.K1, ey, B.K0), more);
+    const float Ei = F::add_up(F::fma_up(B.K2, 2.0f * s_hi, B.K3), E);
+    // |g| <= H |n|, |n|^2 = det <= 1.14 / inv
+    const float gmax = F::mul_up(F::mul_up(B.H, 1.1f), rsqrt_f32(inv));
+    L.E = (double)E;
+    L.W = (double)F::mul_up(F::fma_up(F::add_up(s_hi, -s_lo), gmax, Ei), more);
+    L.s2mid = (double)s_hi + (double)s_lo;
     return L;
 }
 
@@ -550,15 +648,13 @@ __device__ __forceinline__ R dot3(const P4<R>& v, R n0, R n1, R n2) {
     return Ar<R>::fma(v.z, n2, Ar<R>::fma(v.y, n1, Ar<R>::mul(v.x, n0)));
 }
 
-// AC2 scan of a tetrahedron (i,p,k,l) over the candidates M[p] & M[k] & M[l].
-// Returns -1 if a candidate violates AC2, +1 if every test clears, 0 if none
-// violates but some test is undecided at this precision.
-template <class R, int WORDS>
-__device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const Ortho<R>& o, const Bounds<R>& B, int p,
-                                        int k, int l, unsigned& n_ok) {
-    using A = Ar<R>;
-    const R E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);  // inf when o.ey is
-    const R z0 = R(-2) * o.y0, z1 = R(-2) * o.y1, z2 = R(-2) * o.y2;
+// AC2 scan at the orthocentre of z = -2 y with threshold E over the candidates
+// M[p] & M[k] & M[l] (an edge: p three times; a triangle: k twice). Returns -1 if
+// a candidate violates AC2, +1 if every test clears, 0 if none violates but some
+// test is undecided at this precision.
+template <class R, class SM>
+__device__ __forceinline__ int ac2_scan(const SM& S, int nw, R z0, R z1, R z2, R E, int p, int k, int l,
+                                        unsigned& n_ok) {
     bool open = false;
 #pragma unroll 1
     for (int w = 0; w < nw; w++) {
@@ -568,11 +664,102 @@ __device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const 
             b ^= pos_bit(e);
             const R d = delta(point<R>(S, 32 * w + e), z0, z1, z2);
             n_ok++;
-            if (d < -E) return -1;
-            if (!(d > E)) open = true;
+            if constexpr (sizeof(R) == 4) {
+                if (d < -E) return -1;
+                if (!(d > E)) open = true;
+            } else if (fabs(d) > E) {  // one comparison on the FP64 pipe
+                if (__double2hiint(d) < 0) return -1;
+            } else {
+                open = true;
+            }
         }
     }
     return open ? 0 : 1;
+}
+
+// the FP32 line of a triangle: its own, or (FP64) one beside it
+__device__ __forceinline__ const TriLine<float>& line32(const TriLine<float>& L, const TriLine<float>&) { return L; }
+__device__ __forceinline__ const TriLine<float>& line32(const TriLine<double>&, const TriLine<float>& F) { return F; }
+
+// Edge (i,p) in FP32: true if one ball covers its whole disc (header comment);
+// otherwise dmin is the smallest Delta~ over the candidates, E its bound.
+template <class SM>
+__device__ __forceinline__ bool disc_covered(const SM& S, int nw, int p, float T, const Bounds<float>& B,
+                                             float perp_err, float& dmin, float& E, unsigned& n_ok) {
+    using A = Ar<float>;
+    const Ortho<float> o = ortho_edge<float>(point<float>(S, p), B);
+    float S2, eS;
+    norm2(o, B, S2, eS);
+    E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);
+    const float z0 = -2.0f * o.y0, z1 = -2.0f * o.y1, z2 = -2.0f * o.y2;
+    // 4 rho^2, rho the disc's radius; the last factor covers the products below
+    const float r4 = 4.0f * (1.0f + 0x1p-18f) * A::max(A::add_up(A::add_up(T, -S2), eS), 0.0f);
+    const float4 qp = S.qf[p];
+    const float ri = rsqrt_f32(__fmaf_rn(qp.z, qp.z, __fmaf_rn(qp.y, qp.y, __fmul_rn(qp.x, qp.x))));
+    const float u0 = qp.x * ri, u1 = qp.y * ri, u2 = qp.z * ri;  // unit vector along the edge
+    dmin = INFINITY;
+#pragma unroll 1
+    for (int w = 0; w < nw; w++) {
+        unsigned b = S.Mrow[p][w];
+        n_ok += __popc(b);
+        while (b) {
+            const int e = first_pos(b);
+            b ^= pos_bit(e);
+            const P4<float> q = point<float>(S, 32 * w + e);
+            const float d = delta(q, z0, z1, z2);
+            dmin = A::min(d, dmin);
+            if (d < -E) {
+                // Delta_x < 0 all over the disc iff -Delta_x > 2 rho |q_x - (q_x.u) u|
+                const float m = A::sub_dn(-d, E);
+                const float t = dot3(q, u0, u1, u2);
+                const float X2 = __fmaf_rn(q.z, q.z, __fmaf_rn(q.y, q.y, __fmaf_rn(q.x, q.x, perp_err)));
+                if (__fmul_rn(m, m) > __fmul_rn(r4, __fmaf_rn(-t, t, X2))) {
+                    n_ok -= __popc(b);
+                    return true;
+                }
+            }
+        }
+    }
+    return false;
+}
+
+// Triangle (i,p,k) in FP32: false if the balls leave nothing of its segment;
+// otherwise -nlo <= 2 s <= hi holds what they leave, dmin is the smallest Delta~.
+template <class SM>
+__device__ __forceinline__ bool segment_left(const SM& S, int nw, int p, int k, const TriLine<float>& L,
+                                             float& hi, float& nlo, float& dmin, unsigned& n_ok) {
+    hi = nlo = L.s2;
+    const float c = 0x1p-16f * L.s2;  // quotients are within 2^-19 relative, see below
+    dmin = INFINITY;
+#pragma unroll 1
+    for (int w = 0; w < nw; w++) {
+        unsigned b = S.Mrow[p][w] & S.Mrow[k][w];
+        bool alive = true;
+        n_ok += __popc(b);
+        while (b) {
+            const int e = first_pos(b);
+            b ^= pos_bit(e);
+            const P4<float> v = point<float>(S, 32 * w + e);
+            const float d = delta(v, L.z0, L.z1, L.z2);
+            const float g = dot3(v, L.n0, L.n1, L.n2);
+            dmin = fminf(d, dmin);
+            // 2 s g <= d + Ei
+            const float s1 = __fadd_ru(d, L.Ei) * Ar<float>::rcp(fabsf(g));
+            if (g > 0.0f) hi = fminf(hi, s1);
+            else nlo = fminf(nlo, s1);
+            // empty: hi and nlo are at most 2 S, and one below -4 S empties the interval
+            // whatever its rounding, so the two errors are below c / 2
+            if (hi + nlo < -c) {
+                n_ok -= __popc(b);
+                b = 0u;
+                alive = false;
+            }
+        }
+        if (!alive) return false;
+    }
+    hi += c;
+    nlo += c;
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -580,7 +767,7 @@ __device__ __forceinline__ int ac2_scan(const WarpSmem<WORDS>& S, int nw, const 
 template <int WORDS, class R, bool KEEP>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using SM = WarpSmem<WORDS>;
+    using SM = WarpSmem<WORDS, R>;
     constexpr int MAXM = SM::M;
     constexpr bool is32 = sizeof(R) == 4;
     const int lane = threadIdx.x & 31;
@@ -630,7 +817,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
             continue;
         }
         const int nw = (m + 31) >> 5;
-        const R T = (R)si;  // W_i + A <= 2^24: exact
+        const R T = (R)si;  // W_i + A <= 2^24: exact, in FP32 too
+        const float T32 = (float)si;
 
         // ---- phase A: load L(i), the n_up neighbours with an edge of Sigma^1 owned
         // by i first, each part in order of distance from p_i; vertex AC2 (Step
@@ -719,7 +907,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                 const int qx = o.x - Pi.x, qy = o.y - Pi.y, qz = o.z - Pi.z;
                 const int ax = qx * qx + qy * qy + qz * qz - o.w + Wi;
                 S.qf[e] = make_float4((float)qx, (float)qy, (float)qz, (float)ax);
-                S.ai[e] = ax;
+                if constexpr (!is32) {
+                    S.qd[e][0] = make_double2((double)qx, (double)qy);
+                    S.qd[e][1] = make_double2((double)qz, (double)ax);
+                }
                 S.rs[e] = __fsqrt_ru((float)((long long)o.w + Aq));  // W + A <= 2^24: exact in FP32
                 S.idx[e] = x;
             }
@@ -807,48 +998,22 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
             const bool ok = p < n_up;
             bool pass = false, pend = false;
             if (ok) {
-                const Ortho<R> o = ortho_edge<R>(point<R>(S, p), B);
-                R S2, eS;
-                norm2(o, B, S2, eS);
-                const R E = Ar<R>::mul_up(Ar<R>::fma_up(B.K1, o.ey, B.K0), B.up1);
-                const R z0 = R(-2) * o.y0, z1 = R(-2) * o.y1, z2 = R(-2) * o.y2;
-                // 4 rho^2, rho the disc's radius; the last factor covers the products below
-                const float r4 = 4.0f * (1.0f + 0x1p-18f) *
-                                 Ar<R>::to_f32_up(Ar<R>::max(Ar<R>::add_up(Ar<R>::add_up(T, -S2), eS), R(0)));
-                const float4 qp = S.qf[p];
-                const float ri = rsqrt_f32(__fmaf_rn(qp.z, qp.z, __fmaf_rn(qp.y, qp.y, __fmul_rn(qp.x, qp.x))));
-                const float u0 = qp.x * ri, u1 = qp.y * ri, u2 = qp.z * ri;  // unit vector along the edge
-                R dmin = R(INFINITY);
-                bool out = false;
-#pragma unroll 1
-                for (int w = 0; w < nw; w++) {
-                    unsigned b = S.Mrow[p][w];
-                    n_edge += __popc(b);
-                    while (b) {
-                        const int e = first_pos(b);
-                        b ^= pos_bit(e);
-                        const float4 q = S.qf[32 * w + e];
-                        const R d = delta(point<R>(S, 32 * w + e), z0, z1, z2);
-                        dmin = Ar<R>::min(d, dmin);
-                        if (d < -E) {
-                            // Delta_x < 0 all over the disc iff -Delta_x > 2 rho |q_x - (q_x.u) u|
-                            const float m = Ar<R>::to_f32_dn(Ar<R>::sub_dn(-d, E));
-                            const float t = __fmaf_rn(q.z, u2, __fmaf_rn(q.y, u1, __fmul_rn(q.x, u0)));
-                            const float X2 = __fmaf_rn(q.z, q.z, __fmaf_rn(q.y, q.y, __fmaf_rn(q.x, q.x, A.perp_err)));
-                            if (__fmul_rn(m, m) > __fmul_rn(r4, __fmaf_rn(-t, t, X2))) {
-                                out = true;
-                                n_edge -= __popc(b);
-                                break;
-                            }
-                        }
-                    }
-                    if (out) break;
-                }
-                if (!out) {
+                float dmin, E32;
+                unsigned tests = 0;
+                if (!disc_covered(S, nw, p, T32, A.b32, A.perp_err, dmin, E32, tests)) {
                     atomicOr(&S.kup[p >> 5], pos_bit(p));
-                    pass = dmin > E;
-                    pend = !pass && !(dmin < -E);
+                    if constexpr (is32) {
+                        pass = dmin > E32;
+                        pend = !pass && !(dmin < -E32);
+                    } else {  // the FP32 scan only prunes: AC2 in FP64
+                        const Ortho<R> o = ortho_edge<R>(point<R>(S, p), B);
+                        const R E = Ar<R>::mul_up(Ar<R>::fma_up(B.K1, o.ey, B.K0), B.up1);
+                        const int r = ac2_scan<R>(S, nw, R(-2) * o.y0, R(-2) * o.y1, R(-2) * o.y2, E, p, p, p, n_edge);
+                        pass = r > 0;
+                        pend = r == 0;
+                    }
                 }
+                if (is32) n_edge += tests;
             }
             const int idp = ok ? S.idx[p] : 0;
             append_direct(pend, make_int4(i, idp, -1, -1), A.pending, &cnt->n_pending, A.cap_pending, &cnt->err,
@@ -880,7 +1045,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                     if (!open || o.ac3 > 0) {
                         counted = open;
                         n_s3 += open ? 1 : 0;
-                        const int r3 = ac2_scan<R>(S, nw, o, B, p3, k3, ll, n_tet);
+                        const R E = Ar<R>::mul_up(Ar<R>::fma_up(B.K1, o.ey, B.K0), B.up1);  // inf when o.ey is
+                        const int r3 = ac2_scan<R>(S, nw, R(-2) * o.y0, R(-2) * o.y1, R(-2) * o.y2, E, p3, k3, ll, n_tet);
                         pass = r3 > 0;
                         pend = r3 == 0;
                     } else if (o.ac3 == 0) {
@@ -962,48 +1128,33 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                         const unsigned code = S.cand[j];
                         pp = code & SM::PM;
                         kk = code >> SM::SH;
-                        L = tri_line<R>(point<R>(S, pp), point<R>(S, kk), T, B);
+                        if constexpr (is32) L = tri_line(point<R>(S, pp), point<R>(S, kk), T, B);
+                        else L = tri_line(point<R>(S, pp), point<R>(S, kk), S.qf[pp], S.qf[kk], T, T32, A.b64f);
                     }
                     const bool keep_it = L.ac3 > 0;
                     n_ac3t += valid ? 1u : 0u;
                     n_s2 += keep_it ? 1u : 0u;
-                    // the part of the line nearer to the triangle than to any ball: -nlo <= 2 s <= hi
-                    float hi = L.s2, nlo = L.s2;
-                    const float c = 0x1p-16f * L.s2;  // quotients are within 2^-19 relative, see below
+                    // what the balls leave of the segment, in FP32: -nlo <= 2 s <= hi
+                    TriLine<float> own;
+                    const TriLine<float>& F = line32(L, own);
+                    float hi = INFINITY, nlo = INFINITY;
                     bool alive = keep_it && done + j < tot0;
                     if (alive) {
-                        R dmin = R(INFINITY);
-#pragma unroll 1
-                        for (int w = 0; w < nw; w++) {
-                            unsigned b = S.Mrow[pp][w] & S.Mrow[kk][w];
-                            n_tri += __popc(b);
-                            while (b) {
-                                const int e = first_pos(b);
-                                b ^= pos_bit(e);
-                                const P4<R> v = point<R>(S, 32 * w + e);
-                                const R d = delta(v, L.z0, L.z1, L.z2);
-                                const R g = dot3(v, L.n0, L.n1, L.n2);
-                                dmin = Ar<R>::min(d, dmin);
-                                // 2 s g <= d + Ei
-                                const float gf = (float)g;
-                                const float s1 = Ar<R>::to_f32_up(Ar<R>::add_up(d, L.Ei)) * Ar<float>::rcp(fabsf(gf));
-                                if (gf > 0.0f) hi = fminf(hi, s1);
-                                else nlo = fminf(nlo, s1);
-                                // empty: hi and nlo are at most 2 S, and one below -4 S empties the interval
-                                // whatever its rounding, so the two errors are below c / 2
-                                if (hi + nlo < -c) {
-                                    n_tri -= __popc(b);
-                                    b = 0u;
-                                    alive = false;
-                                }
+                        float dmin;
+                        unsigned tests = 0;
+                        if constexpr (is32) {
+                            alive = segment_left(S, nw, pp, kk, F, hi, nlo, dmin, tests);
+                            n_tri += tests;
+                            pass = alive && dmin > F.E;
+                            pend = alive && !pass && !(dmin < -F.E);
+                        } else {
+                            own = tri_line(point<float>(S, pp), point<float>(S, kk), T32, A.b32);
+                            if (F.ac3 > 0) alive = segment_left(S, nw, pp, kk, F, hi, nlo, dmin, tests);
+                            if (alive) {
+                                const int r = ac2_scan<R>(S, nw, L.z0, L.z1, L.z2, L.E, pp, kk, kk, n_tri);
+                                pass = r > 0;
+                                pend = r == 0;
                             }
-                            if (!alive) break;
-                        }
-                        if (alive) {
-                            pass = dmin > L.E;
-                            pend = !pass && !(dmin < -L.E);
-                            hi += c;
-                            nlo += c;
                         }
                     }
                     pend = pend || (valid && L.ac3 == 0);
@@ -1020,10 +1171,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                             const unsigned bit = pos_bit(e);
                             b ^= bit;
                             const P4<R> v = point<R>(S, 32 * w + e);
-                            const R ad = Ar<R>::abs(delta(v, L.z0, L.z1, L.z2));
-                            const R ag = Ar<R>::abs(dot3(v, L.n0, L.n1, L.n2));
-                            if (ad < Ar<R>::fma_dn(ag, L.s2lo, -L.Ei)) in3 |= bit;
-                            if (ad > Ar<R>::fma_up(ag, R(L.s2), L.Ei)) out3 |= bit;
+                            L.tet_ac3(delta(v, L.z0, L.z1, L.z2), dot3(v, L.n0, L.n1, L.n2), bit, in3, out3);
                         }
                         n_s3 += __popc(in3);
                         for (unsigned o = ~(in3 | out3); o;) {
@@ -1034,11 +1182,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                         for (unsigned o = alive ? in3 & S.kup[w] : 0u; o;) {
                             const int e = first_pos(o), x = 32 * w + e;
                             o ^= pos_bit(e);
-                            const P4<R> v = point<R>(S, x);
-                            const R d = delta(v, L.z0, L.z1, L.z2);
-                            const R g = dot3(v, L.n0, L.n1, L.n2);
-                            const R far = Ar<R>::max(Ar<R>::mul(R(hi), g), -Ar<R>::mul(R(nlo), g));
-                            if (!(Ar<R>::add_up(d, -far) > R(1.5) * L.Ei)) push_tet(pp, kk, x, false);
+                            const P4<float> v = point<float>(S, x);
+                            const float d = delta(v, F.z0, F.z1, F.z2), g = dot3(v, F.n0, F.n1, F.n2);
+                            const float far = fmaxf(hi * g, -(nlo * g));
+                            if (!(d - far > 1.5f * F.Ei)) push_tet(pp, kk, x, false);
                         }
                         if (keep) {
                             int tot3;
@@ -1445,8 +1592,8 @@ template <int WORDS, class R>
 static int launch_local(ac_ctx* c, const LocalArgs& a, int64_t max_items, int warps_req, cudaStream_t s) {
     int warps = warps_req > 0 ? warps_req : c->opt.block_warps > 0 ? c->opt.block_warps : 8;
     if (warps > 8) warps = 8;  // __launch_bounds__(256)
-    while (warps > 1 && (size_t)warps * sizeof(WarpSmem<WORDS>) > 200 * 1024) warps--;
-    const size_t smem = (size_t)warps * sizeof(WarpSmem<WORDS>);
+    while (warps > 1 && (size_t)warps * sizeof(WarpSmem<WORDS, R>) > 200 * 1024) warps--;
+    const size_t smem = (size_t)warps * sizeof(WarpSmem<WORDS, R>);
     void (*kern)(LocalArgs) = a.pc.keep_candidates ? k_local<WORDS, R, true> : k_local<WORDS, R, false>;
     AC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0, dev = 0, sms = 0;
@@ -1479,10 +1626,10 @@ static int launch_global(ac_ctx* c, LocalArgs a, cudaStream_t s) {
     int dev = 0, sms = 0;
     AC_CUDA(cudaGetDevice(&dev));
     AC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t cap = ((int64_t)4 << 30) / (int64_t)sizeof(WarpSmem<WORDS>);
+    const int64_t cap = ((int64_t)4 << 30) / (int64_t)sizeof(WarpSmem<WORDS, R>);
     const int64_t warps = std::min<int64_t>(std::min<int64_t>(a.n, 32 * (int64_t)sms), cap);
     const int64_t blocks = (warps + 1) / 2;
-    AC_TRY(c->huge_ws.reserve((size_t)blocks * 2 * sizeof(WarpSmem<WORDS>), s));
+    AC_TRY(c->huge_ws.reserve((size_t)blocks * 2 * sizeof(WarpSmem<WORDS, R>), s));
     a.gws = c->huge_ws.p;
     void (*kern)(LocalArgs) = a.pc.keep_candidates ? k_local<WORDS, R, true> : k_local<WORDS, R, false>;
     kern<<<(unsigned)blocks, 64, 0, s>>>(a);
@@ -1593,6 +1740,7 @@ static void set_constants(const PredConst& pc, int64_t wmax, LocalArgs& a) {
     set_bounds<float>(ldexp(1.0, -24), h, wmax, a.b32);
     a.perp_err = (float)(64.0 * ldexp(1.0, -24) * H * H);
     set_bounds<double>(ldexp(1.0, -53), h, wmax, a.b64);
+    set_bounds<float>(ldexp(1.0, -53), h, wmax, a.b64f);
     // resolve kernel: y from exact minors with relative error <= 4.0001 u64 per component
     const double v = ldexp(1.0, -53), g3d = 3 * v / (1 - 3 * v), dy = 4.0001 * v, sf = 1.0 + 16 * v;
     const double s3 = sqrt(3.0) * (1 + 1e-7), Am = 4 * h * h + (double)wmax;
