@@ -1078,6 +1078,8 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
         c->rec.valid = false;
         return fail(AC_ERR_TIMEOUT, "a bounded device wait (scan look-back) ran out");
     }
+    if (!replayed && c->deferred)
+        for (int d = 0; d < 3; d++) c->K[d].count = (int64_t)h.n_rows[d];
     if (!replayed && !c->opt.no_graph) AC_TRY(record_build(c, h, s));
     finish_mol_rows(c);
     const DevCounters& hl = h;  // the per-atom pass wrote them; later stages add only error bits

@@ -18,6 +18,7 @@
 // below 4 * 2^-53).
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "ac_internal.cuh"
@@ -325,6 +326,8 @@ static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, Si
     AC_TRY(scan_exclusive_i64(c, cnt, off, n, s));
     if (c->replaying) AC_TRY(expect_i64(c, off + n, L.count, s));  // the recorded build's count
     else L.count = nA;
+    L.cap = L.count;
+    L.d_count = nullptr;
     const size_t rows = (size_t)(L.count > 0 ? L.count : 1);
     AC_TRY(L.tuples.reserve(rows * K * sizeof(int32_t), s));
     AC_TRY(L.attached.reserve(rows, s));
@@ -374,7 +377,7 @@ struct EdgeMarkArgs {
     const int2* free_e;  // free edges (sorted positions), nA of them
     int64_t nA;
     const int4* tri;     // K^2 rows (global input indices), nB of them
-    int64_t nB;
+    RowCount nB;
     const int32_t* order;  // sorted position -> input index
     const int32_t* rank;   // input index -> sorted position
     const int64_t* nb_off; // offsets (stride 0) or counts (stride > 0)
@@ -428,7 +431,7 @@ __device__ __forceinline__ void mark_bit(const EdgeMarkArgs& a, int su, int gu, 
 // (a, b) and (a, c) in a's row, (b, c) in b's row
 __global__ void k_edge_mark(EdgeMarkArgs a) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= a.nA + a.nB) return;
+    if (j >= a.nA + a.nB.get()) return;
     int64_t off;
     int m;
     if (j < a.nA) {
@@ -519,6 +522,30 @@ __global__ void __launch_bounds__(EW_WARPS * 32) k_edge_write(EdgeMarkArgs a, in
     }
 }
 
+// Up to this many atoms a build does not wait for the row counts of K^2, K^1 and
+// K^0 one after another (about 13 us each, GPU idle): their buffers and launches
+// cover an upper bound known after the per-atom pass (about 2.5 times the rows,
+// 5 KB per atom in all) and the kernels read the counts on the device. Above,
+// the memory costs more than three waits (2 % of a 100,000-atom build).
+constexpr int64_t DEFER_MAX_ATOMS = 65536;
+
+// The row count of a list whose total the scan left at d_total (at most bound).
+static int list_rows(ac_ctx* c, SimplexList& L, const int64_t* d_total, int64_t bound, cudaStream_t s) {
+    L.d_count = nullptr;
+    if (c->replaying) {
+        AC_TRY(expect_i64(c, d_total, L.count, s));  // the recorded build's count
+    } else if (c->deferred) {
+        L.count = bound;  // until the build's last wait
+        L.d_count = d_total;
+    } else {
+        AC_CUDA(cudaMemcpyAsync(c->h_stage, d_total, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        AC_TRY(sync_host(c, s));
+        L.count = c->h_stage[0];
+    }
+    L.cap = L.count;
+    return AC_OK;
+}
+
 static int canon_edges_by_marks(ac_ctx* c, cudaStream_t s) {
     const DevCounters& h = c->hc;
     const int64_t n = c->n;
@@ -534,26 +561,21 @@ static int canon_edges_by_marks(ac_ctx* c, cudaStream_t s) {
     int64_t* cnt = masks.as<int64_t>();
     unsigned* mask = reinterpret_cast<unsigned*>(masks.as<char>() + o_mask);
     c->endpoint = masks.as<uint8_t>() + o_end;
-    EdgeMarkArgs a{c->edge_pass.as<int2>(), (int64_t)h.n_edge_pass, c->Gbuf[2].as<int4>(), c->K[2].count,
+    EdgeMarkArgs a{c->edge_pass.as<int2>(), (int64_t)h.n_edge_pass, c->Gbuf[2].as<int4>(),
+                   RowCount{c->K[2].cap, c->K[2].d_count},
                    c->order.as<int32_t>(), c->rank.as<int32_t>(), c->nb_cnt.as<int64_t>(), c->nb.as<int32_t>(),
                    c->nb_stride, words, mask, mask + nn * words, reinterpret_cast<unsigned long long*>(cnt),
                    &c->counters.as<DevCounters>()->err};
-    const int64_t items = a.nA + a.nB;
+    const int64_t items = a.nA + c->K[2].cap;
     if (items > 0) {
         k_edge_mark<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(a);
         AC_LAUNCHED();
     }
     int64_t* uoff = L.v0_off.as<int64_t>();
     AC_TRY(scan_exclusive_i64(c, cnt, uoff, n, s));
-    int64_t count = L.count;
-    if (c->replaying) {
-        AC_TRY(expect_i64(c, uoff + n, count, s));
-    } else {
-        AC_CUDA(cudaMemcpyAsync(c->h_stage, uoff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        AC_TRY(sync_host(c, s));
-        count = c->h_stage[0];
-    }
-    L.count = count;
+    // an edge of K^1 joins neighbours, and is free or an edge of a K^2 row
+    AC_TRY(list_rows(c, L, uoff + n, std::min((c->nb_total + 1) / 2, (int64_t)h.n_edge_pass + 3 * c->K[2].cap), s));
+    const int64_t count = L.cap;
     const size_t rows = (size_t)(count > 0 ? count : 1);
     AC_TRY(L.tuples.reserve(rows * 2 * sizeof(int32_t), s));
     AC_TRY(L.attached.reserve(rows, s));
@@ -807,15 +829,9 @@ static int canon_tris_by_marks(ac_ctx* c, cudaStream_t s) {
     const unsigned wb = (unsigned)((n + TW_WARPS - 1) / TW_WARPS);
     int64_t* uoff = L.v0_off.as<int64_t>();
     AC_TRY(scan_exclusive_i64(c, cnt, uoff, n, s));
-    int64_t count = L.count;
-    if (c->replaying) {
-        AC_TRY(expect_i64(c, uoff + n, count, s));
-    } else {
-        AC_CUDA(cudaMemcpyAsync(c->h_stage, uoff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        AC_TRY(sync_host(c, s));
-        count = c->h_stage[0];
-    }
-    L.count = count;
+    // a row of K^2 is a free triangle or a facet of a K^3 row
+    AC_TRY(list_rows(c, L, uoff + n, (int64_t)h.n_tri_pass + 4 * c->K[3].count, s));
+    const int64_t count = L.cap;
     const size_t rows = (size_t)(count > 0 ? count : 1);
     AC_TRY(L.tuples.reserve(rows * 3 * sizeof(int32_t), s));
     AC_TRY(L.attached.reserve(rows, s));
@@ -880,12 +896,19 @@ __global__ void k_mol_rows(MolRowsArgs a) {
 
 static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s);
 
+// the row counts, beside the counters the host reads last
+__global__ void k_row_counts(const int64_t* n0, const int64_t* n1, const int64_t* n2, DevCounters* cnt) {
+    const int64_t* p[3] = {n0, n1, n2};
+    if (threadIdx.x < 3) cnt->n_rows[threadIdx.x] = *p[threadIdx.x];
+}
+
 int canonicalise(ac_ctx* c, cudaStream_t s) {
     const DevCounters& h = c->hc;  // counters read at the end of the per-atom pass
     if (h.err & (DERR_OVF_TET | DERR_OVF_TRI | DERR_OVF_EDGE | DERR_OVF_CAND))
         return fail(AC_ERR_CAPACITY, "per-atom output overflow");
     Work& w = c->cw;
     const int64_t n = c->n;
+    c->deferred = !c->replaying && !c->opt.host_results && n <= DEFER_MAX_ATOMS;
     // K^3
     AC_TRY(canon_dim(c, 3, c->tet_out.as<int4>(), nullptr, (int64_t)h.n_tet_out, c->K[3], c->Gbuf[3], w, s));
     AC_TRY(fork_orthosize(c, 3, s));
@@ -916,15 +939,8 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
             }
             AC_TRY(scan_exclusive_i64(c, inK, voff, n, s));
         }
-        int64_t count = L.count;
-        if (c->replaying) {
-            AC_TRY(expect_i64(c, voff + n, count, s));
-        } else {
-            AC_CUDA(cudaMemcpyAsync(c->h_stage, voff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-            AC_TRY(sync_host(c, s));
-            count = c->h_stage[0];
-        }
-        L.count = count;
+        AC_TRY(list_rows(c, L, voff + n, n, s));
+        const int64_t count = L.cap;
         size_t rows = (size_t)(count > 0 ? count : 1);
         AC_TRY(L.tuples.reserve(rows * sizeof(int32_t), s));
         AC_TRY(L.attached.reserve(rows, s));
@@ -950,6 +966,10 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
             AC_TRY(canon_dim(c, d, d >= 2 ? c->cand[d].as<int4>() : nullptr, d == 1 ? c->cand[1].as<int2>() : nullptr, m,
                              c->C[d], c->CGbuf[d], w, s));
         }
+    }
+    if (c->deferred) {
+        k_row_counts<<<1, 32, 0, s>>>(c->K[0].d_count, c->K[1].d_count, c->K[2].d_count, c->counters.as<DevCounters>());
+        AC_LAUNCHED();
     }
     if (c->n_mol == 1) return AC_OK;  // its rows are the whole lists (finish_mol_rows)
     // per-molecule row ranges, copied to the host with the build's last transfer
@@ -1048,12 +1068,12 @@ __device__ void orthosize_rational(const int4* __restrict__ P, const int4& t, in
     }
 }
 
-__global__ void k_orthosize(const int4* __restrict__ P, const int4* __restrict__ G, int64_t m, int K,
+__global__ void k_orthosize(const int4* __restrict__ P, const int4* __restrict__ G, RowCount m, int K,
                             const uint8_t* __restrict__ attached, double* __restrict__ os, double* __restrict__ f,
                             int8_t* __restrict__ src_dim, int64_t* __restrict__ src_idx,
                             unsigned long long* __restrict__ fkey, unsigned long long* __restrict__ arg) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
+    if (j >= m.get()) return;
     double v = orthosize_exact(P, G[j], K);
     os[j] = v;
     src_dim[j] = (int8_t)(K - 1);
@@ -1092,12 +1112,12 @@ __device__ __forceinline__ int64_t find_row(const int4* __restrict__ L, const in
 
 // pass 1: smallest coface value of every attached face; the row of each
 // (coface, facet) that is an attached face is kept for pass 2 (-1 otherwise)
-__global__ void k_coface_min(const int4* __restrict__ Cof, const double* __restrict__ fc, int64_t mc, int Kc,
+__global__ void k_coface_min(const int4* __restrict__ Cof, const double* __restrict__ fc, RowCount mc, int Kc,
                              const int4* __restrict__ L, const int64_t* __restrict__ v0_off,
                              const uint8_t* __restrict__ attached, unsigned long long* __restrict__ fkey,
                              int64_t* __restrict__ rows) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= mc) return;
+    if (j >= mc.get()) return;
     int4 t = Cof[j];
     unsigned long long key = order_key(fc[j]);
     for (int drop = 0; drop < Kc; drop++) {
@@ -1110,10 +1130,10 @@ __global__ void k_coface_min(const int4* __restrict__ Cof, const double* __restr
 }
 
 // pass 2: among cofaces attaining the minimum, the first in lexicographic order
-__global__ void k_coface_arg(const double* __restrict__ fc, int64_t mc, int Kc, const int64_t* __restrict__ rows,
+__global__ void k_coface_arg(const double* __restrict__ fc, RowCount mc, int Kc, const int64_t* __restrict__ rows,
                              const unsigned long long* __restrict__ fkey, unsigned long long* __restrict__ arg) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= mc) return;
+    if (j >= mc.get()) return;
     unsigned long long key = order_key(fc[j]);
     for (int drop = 0; drop < Kc; drop++) {
         const int64_t r = rows[j * Kc + drop];
@@ -1121,12 +1141,12 @@ __global__ void k_coface_arg(const double* __restrict__ fc, int64_t mc, int Kc, 
     }
 }
 
-__global__ void k_coface_apply(int64_t m, const uint8_t* __restrict__ attached, const unsigned long long* __restrict__ fkey,
+__global__ void k_coface_apply(RowCount m, const uint8_t* __restrict__ attached, const unsigned long long* __restrict__ fkey,
                                const unsigned long long* __restrict__ arg, const int8_t* __restrict__ csrc_dim,
                                const int64_t* __restrict__ csrc_idx, double* __restrict__ f, int8_t* __restrict__ src_dim,
                                int64_t* __restrict__ src_idx, unsigned* __restrict__ err) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m || !attached[j]) return;
+    if (j >= m.get() || !attached[j]) return;
     unsigned long long a = arg[j];
     if (a == ~0ull) {
         // an attached simplex with no coface in the complex cannot occur
@@ -1319,10 +1339,11 @@ static int copy_values_to_host(ac_ctx* c, int d, cudaStream_t from) {
 // has its own buffers, reserved here on the build's stream before the fork.
 static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
     SimplexList& L = c->K[d];
-    const int64_t m = L.count;
+    const int64_t m = L.cap;
     if (m == 0) return AC_OK;
     SimplexList* U = d < 3 ? &c->K[d + 1] : nullptr;
-    const int64_t mu = U ? U->count : 0;
+    const int64_t mu = U ? U->cap : 0;
+    const RowCount rm{m, L.d_count}, ru{mu, U ? U->d_count : nullptr};
     AC_TRY(c->fkey[d].reserve((size_t)m * sizeof(unsigned long long), s));
     if (U) {
         AC_TRY(c->fargs[d].reserve((size_t)m * sizeof(unsigned long long), s));
@@ -1334,7 +1355,7 @@ static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
     AC_CUDA(cudaStreamWaitEvent(t, c->ev_fork, 0));
     unsigned long long* keyb = c->fkey[d].as<unsigned long long>();
     unsigned long long* argb = U ? c->fargs[d].as<unsigned long long>() : nullptr;
-    k_orthosize<<<(unsigned)((m + 127) / 128), 128, 0, t>>>(c->P.as<int4>(), c->Gbuf[d].as<int4>(), m, d + 1,
+    k_orthosize<<<(unsigned)((m + 127) / 128), 128, 0, t>>>(c->P.as<int4>(), c->Gbuf[d].as<int4>(), rm, d + 1,
                                                             L.attached.as<uint8_t>(), L.orthosize.as<double>(),
                                                             L.f.as<double>(), L.src_dim.as<int8_t>(),
                                                             L.src_idx.as<int64_t>(), keyb, argb);
@@ -1344,14 +1365,14 @@ static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
     if (mu > 0) {
         const unsigned nbk = (unsigned)((mu + 127) / 128);
         int64_t* rows = c->frows[d].as<int64_t>();
-        k_coface_min<<<nbk, 128, 0, t>>>(c->Gbuf[d + 1].as<int4>(), U->f.as<double>(), mu, d + 2, c->Gbuf[d].as<int4>(),
+        k_coface_min<<<nbk, 128, 0, t>>>(c->Gbuf[d + 1].as<int4>(), U->f.as<double>(), ru, d + 2, c->Gbuf[d].as<int4>(),
                                          L.v0_off.as<int64_t>(), L.attached.as<uint8_t>(), keyb, rows);
         AC_LAUNCHED();
-        k_coface_arg<<<nbk, 128, 0, t>>>(U->f.as<double>(), mu, d + 2, rows, keyb, argb);
+        k_coface_arg<<<nbk, 128, 0, t>>>(U->f.as<double>(), ru, d + 2, rows, keyb, argb);
         AC_LAUNCHED();
     }
     k_coface_apply<<<(unsigned)((m + 127) / 128), 128, 0, t>>>(
-        m, L.attached.as<uint8_t>(), keyb, argb, U->src_dim.as<int8_t>(), U->src_idx.as<int64_t>(), L.f.as<double>(),
+        rm, L.attached.as<uint8_t>(), keyb, argb, U->src_dim.as<int8_t>(), U->src_idx.as<int64_t>(), L.f.as<double>(),
         L.src_dim.as<int8_t>(), L.src_idx.as<int64_t>(), &c->counters.as<DevCounters>()->err);
     AC_LAUNCHED();
     return copy_values_to_host(c, d, t);

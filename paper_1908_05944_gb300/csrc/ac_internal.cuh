@@ -122,6 +122,7 @@ struct DevCounters {
     unsigned long long nb_sum;        // neighbour pairs counted (sum of |L(i)|)
     unsigned long long pair_words;    // words of the K^2 pair masks
     unsigned long long n_over[4];     // atoms with more than 64, 512, 128, 256 neighbours
+    long long n_rows[3];              // rows of K^0..K^2 (a build that does not wait for them in between)
 };
 // The bounding boxes (6 int32 per molecule) follow the counters in one device
 // buffer, as in the page-locked readback block: one copy brings both.
@@ -143,6 +144,13 @@ struct MolGrid {
     int32_t org[3];
     int32_t dims[3];
     int64_t cell_base;
+};
+
+// Number of rows of a list inside a build: m, or what *dm holds.
+struct RowCount {
+    int64_t m;
+    const int64_t* dm;
+    __device__ __forceinline__ int64_t get() const { return dm ? *dm : m; }
 };
 
 // Build-wide constants for the predicates.
@@ -167,6 +175,10 @@ struct SimplexList {
     DevBuf src_idx;  // int64: index of the source simplex in its list
     DevBuf v0_off;   // int64 (n+1): rows with first vertex (global input index) g start at v0_off[g]
     int64_t count = 0;
+    // while a build runs: its buffers and launches cover `cap` rows; d_count is where the device holds their
+    // number, or null when it is cap
+    int64_t cap = 0;
+    const int64_t* d_count = nullptr;
     std::vector<int64_t> mol_off;  // host: first row of each molecule, n_mol + 1
 };
 
@@ -273,6 +285,7 @@ struct ac_ctx {
     ac::DevBuf frows[4];     // per-dimension facet rows of the cofaces (k_coface_min -> k_coface_arg)
     bool os_forked = false;  // k_orthosize launches on the side stream await their join
     int64_t pair_words = 0;  // words of the triangle pair masks (recorded for replays)
+    bool deferred = false;        // this build reads the rows of K^0..K^2 with its last wait
     uint8_t* endpoint = nullptr;  // K^1's endpoint flags by input index (within scratch[2], this build's)
     ac::DevBuf pair_moff;    // first pair-mask word of each sorted position (n + 1)
     ac::DevBuf scan_tmp;
