@@ -55,16 +55,6 @@ __device__ __forceinline__ void sort_asc(int4& t, int K) {
     }
 }
 
-// facet of a row of K + 1 ascending entries: the K-tuple without entry drop
-__device__ __forceinline__ int4 facet_of(const int4& t, int K, int drop) {
-    int v[4] = {t.x, t.y, t.z, t.w};
-    int o[4] = {-1, -1, -1, -1};
-    int w = 0;
-    for (int k = 0; k <= K; k++)
-        if (k != drop) o[w++] = v[k];
-    return make_int4(o[0], o[1], o[2], o[3]);
-}
-
 // The items of one list, K entries each, emitted once each by their owner:
 // nA tuples of sorted positions (a4, or a2 for edges), taken to ascending tuples
 // of input indices. An item's bucket is its first vertex.
@@ -400,15 +390,39 @@ __device__ __forceinline__ void edge_row(const EdgeMarkArgs& a, int s, int64_t& 
     }
 }
 
-// position of sorted position x in the ascending row [off, off + m), or -1
-__device__ __forceinline__ int row_find(const int32_t* __restrict__ nb, int64_t off, int m, int x) {
-    int lo = 0, hi = m;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (nb[off + mid] < x) lo = mid + 1;
-        else hi = mid;
+// Positions e[k] of x[k] in the ascending rows [off[k], off[k] + m[k]), or -1. The
+// searches are chains of dependent loads: they step together, one load of each
+// in flight. That is what small builds wait for (k_edge_mark of 2,000 atoms 9.2
+// -> 8.0 us, the facet searches below 26 -> 17); large ones are bound by the
+// number of lines touched and see no difference.
+template <int N>
+__device__ __forceinline__ void row_find(const int32_t* __restrict__ nb, const int64_t (&off)[N], const int (&m)[N],
+                                         const int (&x)[N], int (&e)[N]) {
+    int lo[N], n[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        lo[k] = 0;
+        n[k] = m[k];
     }
-    return lo < m && nb[off + lo] == x ? lo : -1;
+    for (bool more = true; more;) {
+        int v[N];
+#pragma unroll
+        for (int k = 0; k < N; k++) v[k] = n[k] > 0 ? nb[off[k] + lo[k] + (n[k] >> 1)] : 0;
+        more = false;
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            const int half = n[k] >> 1;
+            if (n[k] > 0 && v[k] < x[k]) {
+                lo[k] += half + 1;
+                n[k] -= half + 1;
+            } else {
+                n[k] = half;
+            }
+            more = more || n[k] > 0;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) e[k] = lo[k] < m[k] && nb[off[k] + lo[k]] == x[k] ? lo[k] : -1;
 }
 
 // bit e of sorted position su's row mask; the first setting of a bit counts a
@@ -444,20 +458,26 @@ __global__ void k_edge_mark(EdgeMarkArgs a) {
             gu = gv;
         }
         edge_row(a, su, off, m);
-        mark_bit(a, su, gu, row_find(a.nb, off, m, sv), true);
+        const int64_t offs[1] = {off};
+        const int ms[1] = {m}, xs[1] = {sv};
+        int es[1];
+        row_find<1>(a.nb, offs, ms, xs, es);
+        mark_bit(a, su, gu, es[0], true);
         return;
     }
     const int4 t = a.tri[j - a.nA];
     const int sa = a.rank[t.x], sb = a.rank[t.y], sc = a.rank[t.z];
     edge_row(a, sa, off, m);
-    const int eb = row_find(a.nb, off, m, sb), ec = row_find(a.nb, off, m, sc);
     int64_t offb;
     int mb;
     edge_row(a, sb, offb, mb);
-    const int ebc = row_find(a.nb, offb, mb, sc);
-    mark_bit(a, sa, t.x, eb, false);
-    mark_bit(a, sa, t.x, ec, false);
-    mark_bit(a, sb, t.y, ebc, false);
+    const int64_t offs[3] = {off, off, offb};
+    const int ms[3] = {m, m, mb}, xs[3] = {sb, sc, sc};
+    int es[3];
+    row_find<3>(a.nb, offs, ms, xs, es);
+    mark_bit(a, sa, t.x, es[0], false);
+    mark_bit(a, sa, t.x, es[1], false);
+    mark_bit(a, sb, t.y, es[2], false);
 }
 
 // the marked entries of g's row, ranked by input index: one warp per atom;
@@ -674,7 +694,11 @@ __global__ void k_tri_mark(TriMarkArgs a) {
         if (gv[2] < gv[f]) f = 2;
         const int sa = sv[f], s1 = sv[f == 0 ? 1 : 0], s2 = sv[f == 2 ? 1 : 2];
         nb_row_of(a.nb_off, a.stride, sa, off, m);
-        mark_pair(a, sa, gv[f], row_find(a.nb, off, m, s1), row_find(a.nb, off, m, s2), true);
+        const int64_t offs[2] = {off, off};
+        const int ms[2] = {m, m}, xs[2] = {s1, s2};
+        int es[2];
+        row_find<2>(a.nb, offs, ms, xs, es);
+        mark_pair(a, sa, gv[f], es[0], es[1], true);
         return;
     }
     int4 q = a.tet[j - a.nA];  // sorted positions, put in order of input index below
@@ -694,12 +718,17 @@ __global__ void k_tri_mark(TriMarkArgs a) {
     cs(t.y, q.y, t.w, q.w);
     cs(t.y, q.y, t.z, q.z);
     nb_row_of(a.nb_off, a.stride, q.x, off, m);
-    const int pb = row_find(a.nb, off, m, q.y), pc = row_find(a.nb, off, m, q.z), pd = row_find(a.nb, off, m, q.w);
-    mark_pair(a, q.x, t.x, pb, pc, false);
-    mark_pair(a, q.x, t.x, pb, pd, false);
-    mark_pair(a, q.x, t.x, pc, pd, false);
-    nb_row_of(a.nb_off, a.stride, q.y, off, m);
-    mark_pair(a, q.y, t.y, row_find(a.nb, off, m, q.z), row_find(a.nb, off, m, q.w), false);
+    int64_t offb;
+    int mb;
+    nb_row_of(a.nb_off, a.stride, q.y, offb, mb);
+    const int64_t offs[5] = {off, off, off, offb, offb};
+    const int ms[5] = {m, m, m, mb, mb}, xs[5] = {q.y, q.z, q.w, q.z, q.w};
+    int es[5];
+    row_find<5>(a.nb, offs, ms, xs, es);
+    mark_pair(a, q.x, t.x, es[0], es[1], false);
+    mark_pair(a, q.x, t.x, es[0], es[2], false);
+    mark_pair(a, q.x, t.x, es[1], es[2], false);
+    mark_pair(a, q.y, t.y, es[3], es[4], false);
 }
 
 constexpr int TW_WARPS = 4;
@@ -1093,39 +1122,72 @@ __device__ __forceinline__ double key_value(unsigned long long k) {
     return __longlong_as_double((long long)b);
 }
 
-// row index of tuple t (global indices, K entries) in the canonical list L, or -1
-// (a row's components past its K entries are not looked at)
-__device__ __forceinline__ int64_t find_row(const int4* __restrict__ L, const int64_t* __restrict__ v0_off, int K,
-                                            const int4& t) {
-    int64_t lo = v0_off[t.x], hi = v0_off[t.x + 1];
-    if (K == 1) return lo < hi ? lo : -1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        const int4 r = L[mid];
-        const int dy = r.y - t.y, d = dy != 0 || K == 2 ? dy : r.z - t.z;  // indices: no overflow
-        if (d == 0) return mid;
-        if (d < 0) lo = mid + 1;
-        else hi = mid;
+// Rows of the K facets of coface t (K entries, facets of K - 1) in the canonical
+// list L, or -1: facet `drop` leaves out entry drop. The searches in the facets'
+// first-vertex buckets step together, as in row_find; a row's components past its
+// K - 1 entries are not looked at.
+template <int K>
+__device__ __forceinline__ void find_facets(const int4* __restrict__ L, const int64_t* __restrict__ v0_off, const int4& t,
+                                            int64_t (&r)[K]) {
+    const int64_t a0 = v0_off[t.x], a1 = v0_off[t.x + 1], b0 = v0_off[t.y], b1 = v0_off[t.y + 1];
+    if constexpr (K == 2) {  // vertices: one row per atom, if it has one
+        r[0] = b0 < b1 ? b0 : -1;
+        r[1] = a0 < a1 ? a0 : -1;
+    } else {
+        int64_t lo[K], hi[K];
+        int y[K], z[K];
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            lo[k] = k == 0 ? b0 : a0;
+            hi[k] = k == 0 ? b1 : a1;
+            y[k] = k <= 1 ? t.z : t.y;
+            z[k] = K == 4 ? (k <= 2 ? t.w : t.z) : 0;
+            r[k] = -1;
+        }
+        for (bool more = true; more;) {
+            int4 v[K];
+#pragma unroll
+            for (int k = 0; k < K; k++) v[k] = L[lo[k] < hi[k] ? (lo[k] + hi[k]) >> 1 : a0];
+            more = false;
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                if (lo[k] >= hi[k]) continue;
+                const int64_t mid = (lo[k] + hi[k]) >> 1;
+                const int dy = v[k].y - y[k], d = dy != 0 || K == 3 ? dy : v[k].z - z[k];  // indices: no overflow
+                if (d == 0) {
+                    r[k] = mid;
+                    lo[k] = hi[k];
+                } else if (d < 0) {
+                    lo[k] = mid + 1;
+                } else {
+                    hi[k] = mid;
+                }
+                more = more || lo[k] < hi[k];
+            }
+        }
     }
-    return -1;
 }
 
 // pass 1: smallest coface value of every attached face; the row of each
 // (coface, facet) that is an attached face is kept for pass 2 (-1 otherwise)
-__global__ void k_coface_min(const int4* __restrict__ Cof, const double* __restrict__ fc, RowCount mc, int Kc,
+template <int K>
+__global__ void k_coface_min(const int4* __restrict__ Cof, const double* __restrict__ fc, RowCount mc,
                              const int4* __restrict__ L, const int64_t* __restrict__ v0_off,
                              const uint8_t* __restrict__ attached, unsigned long long* __restrict__ fkey,
                              int64_t* __restrict__ rows) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= mc.get()) return;
-    int4 t = Cof[j];
-    unsigned long long key = order_key(fc[j]);
-    for (int drop = 0; drop < Kc; drop++) {
-        int4 face = facet_of(t, Kc - 1, drop);
-        int64_t r = find_row(L, v0_off, Kc - 1, face);
-        const bool hit = r >= 0 && attached[r];
-        rows[j * Kc + drop] = hit ? r : -1;
-        if (hit) atomicMin(&fkey[r], key);
+    const int4 t = Cof[j];
+    const unsigned long long key = order_key(fc[j]);
+    int64_t r[K];
+    find_facets<K>(L, v0_off, t, r);
+    bool hit[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) hit[k] = r[k] >= 0 && attached[r[k]];
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        rows[j * K + k] = hit[k] ? r[k] : -1;
+        if (hit[k]) atomicMin(&fkey[r[k]], key);
     }
 }
 
@@ -1365,8 +1427,9 @@ static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
     if (mu > 0) {
         const unsigned nbk = (unsigned)((mu + 127) / 128);
         int64_t* rows = c->frows[d].as<int64_t>();
-        k_coface_min<<<nbk, 128, 0, t>>>(c->Gbuf[d + 1].as<int4>(), U->f.as<double>(), ru, d + 2, c->Gbuf[d].as<int4>(),
-                                         L.v0_off.as<int64_t>(), L.attached.as<uint8_t>(), keyb, rows);
+        auto kmin = d == 2 ? k_coface_min<4> : d == 1 ? k_coface_min<3> : k_coface_min<2>;
+        kmin<<<nbk, 128, 0, t>>>(c->Gbuf[d + 1].as<int4>(), U->f.as<double>(), ru, c->Gbuf[d].as<int4>(),
+                                 L.v0_off.as<int64_t>(), L.attached.as<uint8_t>(), keyb, rows);
         AC_LAUNCHED();
         k_coface_arg<<<nbk, 128, 0, t>>>(U->f.as<double>(), ru, d + 2, rows, keyb, argb);
         AC_LAUNCHED();
