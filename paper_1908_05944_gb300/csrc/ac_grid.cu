@@ -173,6 +173,39 @@ __device__ __forceinline__ int deg_bin(int64_t m) {
     return m > 512 ? 258 : m > 256 ? 257 : m > 64 ? (int)m : ((int)m + 15) & ~15;
 }
 
+// What a block adds to the build's totals: one set of atomics per block. Every
+// thread of the block calls it (count and words 0 where it holds no atom).
+__device__ __forceinline__ void block_sums(int64_t count, int64_t words, unsigned* b_hist, unsigned* __restrict__ hist,
+                                           DevCounters* __restrict__ cnt) {
+    __shared__ unsigned long long b_tot[NB_THREADS / 32], b_words[NB_THREADS / 32];
+    __shared__ int b_max[NB_THREADS / 32];
+    const unsigned wt = __reduce_add_sync(0xffffffffu, (unsigned)count);
+    const unsigned wm = __reduce_max_sync(0xffffffffu, (unsigned)count);
+    unsigned long long ww = (unsigned long long)words;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, o);
+    if ((threadIdx.x & 31) == 0) {
+        b_tot[threadIdx.x >> 5] = wt;
+        b_max[threadIdx.x >> 5] = (int)wm;
+        b_words[threadIdx.x >> 5] = ww;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < DEG_BINS; t += NB_THREADS)
+        if (b_hist[t]) atomicAdd(&hist[t], b_hist[t]);
+    if (threadIdx.x == 0) {
+        unsigned long long tot = 0, words_b = 0;
+        int m = 0;
+        for (int k = 0; k < NB_THREADS / 32; k++) {
+            tot += b_tot[k];
+            words_b += b_words[k];
+            m = max(m, b_max[k]);
+        }
+        if (tot) atomicAdd(&cnt->nb_sum, tot);
+        if (words_b) atomicAdd(&cnt->pair_words, words_b);
+        atomicMax(&cnt->max_degree, m);
+    }
+}
+
 // MODE NB_COUNT and NB_PADDED also add up what the host sizes the next steps
 // by: pairs, largest count, words of the K^2 pair masks, degree histogram.
 template <int MODE, bool SMALL>
@@ -227,36 +260,93 @@ __global__ void __launch_bounds__(NB_THREADS)
             atomicAdd(&b_hist[deg_bin(count)], 1u);
         }
     }
-    if (MODE != NB_CSR) {
-        // one set of atomics per block; every thread reaches here (no early exit above)
-        __shared__ unsigned long long b_tot[NB_THREADS / 32], b_words[NB_THREADS / 32];
-        __shared__ int b_max[NB_THREADS / 32];
-        const unsigned wt = __reduce_add_sync(0xffffffffu, (unsigned)count);
-        const unsigned wm = __reduce_max_sync(0xffffffffu, (unsigned)count);
-        unsigned long long ww = (unsigned long long)words;
+    if (MODE != NB_CSR) block_sums(count, words, b_hist, hist, cnt);
+}
+
+// The padded search of a small molecule, NB_LANES lanes per atom: with a thread per
+// atom 20,000 atoms fill half the SMs' warps and each walks its 25 stencil rows
+// one after another, a chain of dependent loads. Here the lanes take a row each,
+// count its neighbours, place them by a prefix over the lanes (rows in (z, y)
+// order, so L(i) ascends as above) and go over the row again to write them. The
+// second walk and the idle lanes cost more than the chain once the GPU is full.
+// Neighbour stage of a rebuild in us, thread per atom / lanes: van der Waals radii
+// 2,000 atoms 33 / 20, 20,000 39 / 33, 35,000 38 / 38, 100,000 49 / 77; probe radii
+// 2,000 57 / 28, 20,000 65 / 47, 35,000 65 / 63, 100,000 86 / 139; particles 2,000
+// 116 / 47, 35,000 133 / 120, 50,000 151 / 157.
+constexpr int NB_LANES = 8;
+constexpr int64_t NB_LANES_MAX_ATOMS = 32768;
+
+template <bool SMALL>
+__global__ void __launch_bounds__(NB_THREADS)
+    k_neighbours_lanes(const int4* __restrict__ Ps, const int32_t* __restrict__ mol_s, const MolGrid* __restrict__ grids,
+                       const uint32_t* __restrict__ cell_start, PredConst pc, int64_t n, int64_t* __restrict__ nb_cnt,
+                       int32_t* __restrict__ nb, DevCounters* __restrict__ cnt, int64_t* __restrict__ pw,
+                       unsigned* __restrict__ hist) {
+    const int sub = threadIdx.x % NB_LANES;
+    const unsigned gmask = ((1u << NB_LANES) - 1u) << (threadIdx.x & 31 & ~(NB_LANES - 1));
+    const int64_t s = ((int64_t)blockIdx.x * NB_THREADS + threadIdx.x) / NB_LANES;
+    int count = 0;
+    __shared__ unsigned b_hist[DEG_BINS];
+    for (int t = threadIdx.x; t < DEG_BINS; t += NB_THREADS) b_hist[t] = 0u;
+    __syncthreads();
+    int64_t words = 0;
+    if (s < n) {
+        const int4 p = Ps[s];
+        const int64_t si = (int64_t)p.w + pc.A;
+        if (si >= 0) {
+            const MolGrid g = grids[mol_s[s]];
+            const int cell = pc.cell, R = pc.reach;
+            const int cx = (p.x - g.org[0]) / cell, cy = (p.y - g.org[1]) / cell, cz = (p.z - g.org[2]) / cell;
+            const int z0 = max(cz - R, 0), z1 = min(cz + R, g.dims[2] - 1);
+            const int y0 = max(cy - R, 0), y1 = min(cy + R, g.dims[1] - 1);
+            const int x0 = max(cx - R, 0), x1 = min(cx + R, g.dims[0] - 1);
+            const int32_t si32 = (int32_t)si;
+            const int A32 = (int)max(pc.A, -(int64_t)(1 << 30));
+            const int ny = y1 - y0 + 1, rows = (z1 - z0 + 1) * ny;
+            for (int r0 = 0; r0 < rows; r0 += NB_LANES) {  // the same for all lanes of the atom
+                const int r = r0 + sub;
+                uint32_t a = 0, b = 0;
+                if (r < rows) {
+                    const int z = z0 + r / ny, y = y0 + r % ny;
+                    const int64_t row = g.cell_base + ((int64_t)z * g.dims[1] + y) * g.dims[0];
+                    a = cell_start[row + x0];
+                    b = cell_start[row + x1 + 1];
+                }
+                int c = 0;
+                for (uint32_t t0 = a; t0 < b; t0 += NB_UNROLL) {
+                    int4 ov[NB_UNROLL];
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, o);
-        if ((threadIdx.x & 31) == 0) {
-            b_tot[threadIdx.x >> 5] = wt;
-            b_max[threadIdx.x >> 5] = (int)wm;
-            b_words[threadIdx.x >> 5] = ww;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < DEG_BINS; t += NB_THREADS)
-            if (b_hist[t]) atomicAdd(&hist[t], b_hist[t]);
-        if (threadIdx.x == 0) {
-            unsigned long long tot = 0, words_b = 0;
-            int m = 0;
-            for (int k = 0; k < NB_THREADS / 32; k++) {
-                tot += b_tot[k];
-                words_b += b_words[k];
-                m = max(m, b_max[k]);
+                    for (int u = 0; u < NB_UNROLL; u++) ov[u] = __ldg(&Ps[t0 + u < b ? t0 + u : a]);
+#pragma unroll
+                    for (int u = 0; u < NB_UNROLL; u++)
+                        if (t0 + u < b && t0 + u != (uint32_t)s && nb_meet<SMALL>(p, si, si32, A32, pc, ov[u], cnt)) c++;
+                }
+                int inc = c;
+#pragma unroll
+                for (int o = 1; o < NB_LANES; o <<= 1) {
+                    const int t = __shfl_up_sync(gmask, inc, o, NB_LANES);
+                    if (sub >= o) inc += t;
+                }
+                int at = count + inc - c;
+                count += __shfl_sync(gmask, inc, NB_LANES - 1, NB_LANES);
+                if (c == 0) continue;
+                for (uint32_t t = a; t < b; t++)
+                    if (t != (uint32_t)s && nb_meet<SMALL>(p, si, si32, A32, pc, __ldg(&Ps[t]), cnt)) {
+                        if (at < NB_STRIDE) nb[s * NB_STRIDE + at] = (int32_t)t;
+                        at++;
+                    }
             }
-            if (tot) atomicAdd(&cnt->nb_sum, tot);
-            if (words_b) atomicAdd(&cnt->pair_words, words_b);
-            atomicMax(&cnt->max_degree, m);
+        }
+        if (sub == 0) {
+            nb_cnt[s] = count;
+            words = pair_mask_words(count);
+            pw[s] = words;
+            atomicAdd(&b_hist[deg_bin(count)], 1u);
+        } else {
+            count = 0;  // counted once
         }
     }
+    block_sums(count, words, b_hist, hist, cnt);
 }
 
 // Blocks of k_neighbours: one thread per atom.
@@ -320,9 +410,15 @@ int build_neighbours(ac_ctx* c, cudaStream_t s) {
     unsigned* cursor = hist + DEG_BINS;
     if (padded) {
         AC_TRY(c->nb.reserve((size_t)n * NB_STRIDE * sizeof(int32_t), s));
-        auto k = small ? k_neighbours<NB_PADDED, true> : k_neighbours<NB_PADDED, false>;
-        k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, c->nb.as<int32_t>(), dc, pw,
-                                    hist);
+        if (n <= NB_LANES_MAX_ATOMS) {
+            auto k = small ? k_neighbours_lanes<true> : k_neighbours_lanes<false>;
+            k<<<neighbour_blocks(n * NB_LANES), NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp,
+                                                                    c->nb.as<int32_t>(), dc, pw, hist);
+        } else {
+            auto k = small ? k_neighbours<NB_PADDED, true> : k_neighbours<NB_PADDED, false>;
+            k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, c->nb.as<int32_t>(),
+                                        dc, pw, hist);
+        }
     } else {
         auto k = small ? k_neighbours<NB_COUNT, true> : k_neighbours<NB_COUNT, false>;
         k<<<kb, NB_THREADS, 0, s>>>(g.Ps, g.mol_s, g.grids, g.cell_start, c->pc, n, cntp, nullptr, nullptr, dc, pw, hist);
