@@ -262,18 +262,23 @@ int eval_filtration_f32(ac_ctx* c, float* const f_out[4], cudaStream_t s) {
 
 // The values at moved atoms, each source evaluated once: a row that is its own
 // source (unattached) by its double-double OrthoSize, then every attached row a
-// copy of its source's value. The FP64 pipe (2 lanes per clock and SM) bounds
+// copy of its source's value (100,000-atom probe globule: 2.4 ms; 9.9 ms when
+// every row evaluated its source, the four sizes mixed in a warp). The FP64 pipe (2 lanes per clock and SM) bounds
 // it, and takes as long for a warp with one active lane as for a full one:
-// a block gathers the unattached rows of EVAL_TILE rows and evaluates those.
+// a block gathers the unattached rows of a tile and evaluates those. A tile of 512
+// rows fills its last warp best; short lists take tiles of 128, one evaluation per
+// thread, or their few blocks run four long FP64 chains one after another (values
+// at moved atoms of a 2,000-atom globule: 330 us, now 157).
 constexpr int EVAL_THREADS = 128;
-constexpr int EVAL_TILE = 512;
+constexpr int EVAL_TILE = 512, EVAL_TILE_SHORT = 128;
+constexpr int64_t EVAL_SHORT_ROWS = 2 * 152 * EVAL_TILE;  // two blocks of EVAL_TILE rows per SM
 
 // indices (from first) of the rows of a tile with !skip(row), in no particular order
-template <class F>
+template <int TILE, class F>
 __device__ __forceinline__ int gather_rows(int64_t first, int64_t m, int* list, int* n_list, F&& skip) {
     if (threadIdx.x == 0) *n_list = 0;
     __syncthreads();
-    for (int u = threadIdx.x; u < EVAL_TILE; u += EVAL_THREADS) {
+    for (int u = threadIdx.x; u < TILE; u += EVAL_THREADS) {
         const bool take = first + u < m && !skip(first + u);
         const unsigned b = __ballot_sync(0xffffffffu, take);
         int base = 0;
@@ -285,15 +290,15 @@ __device__ __forceinline__ int gather_rows(int64_t first, int64_t m, int* list, 
     return *n_list;
 }
 
-template <int K>
+template <int K, int TILE>
 __global__ void __launch_bounds__(EVAL_THREADS) k_eval_own(const double* __restrict__ X, const double* __restrict__ R,
                                                            const int4* __restrict__ G,
                                                            const uint8_t* __restrict__ attached, int64_t m,
                                                            double* __restrict__ out) {
-    __shared__ int list[EVAL_TILE];
+    __shared__ int list[TILE];
     __shared__ int n_list;
-    const int64_t first = (int64_t)blockIdx.x * EVAL_TILE;
-    const int n = gather_rows(first, m, list, &n_list, [&](int64_t j) { return attached[j] != 0; });
+    const int64_t first = (int64_t)blockIdx.x * TILE;
+    const int n = gather_rows<TILE>(first, m, list, &n_list, [&](int64_t j) { return attached[j] != 0; });
     for (int u = threadIdx.x; u < n; u += EVAL_THREADS) {
         const int64_t j = first + list[u];
         out[j] = orthosize_dd<K>(X, R, G[j]);
@@ -359,9 +364,15 @@ int eval_filtration(ac_ctx* c, const double* centres, const double* radii, doubl
     for (int d = 3; d >= lo; d--) {
         const int64_t m = c->K[d].count;
         if (m == 0) continue;
+        constexpr int T = EVAL_TILE, TS = EVAL_TILE_SHORT;
+        const bool shrt = m < EVAL_SHORT_ROWS;
         void (*k)(const double*, const double*, const int4*, const uint8_t*, int64_t, double*) =
-            d == 3 ? k_eval_own<4> : d == 2 ? k_eval_own<3> : d == 1 ? k_eval_own<2> : k_eval_own<1>;
-        k<<<(unsigned)((m + EVAL_TILE - 1) / EVAL_TILE), EVAL_THREADS, 0, s>>>(
+            d == 3   ? (shrt ? k_eval_own<4, TS> : k_eval_own<4, T>)
+            : d == 2 ? (shrt ? k_eval_own<3, TS> : k_eval_own<3, T>)
+            : d == 1 ? (shrt ? k_eval_own<2, TS> : k_eval_own<2, T>)
+                     : (shrt ? k_eval_own<1, TS> : k_eval_own<1, T>);
+        const int tile = shrt ? TS : T;
+        k<<<(unsigned)((m + tile - 1) / tile), EVAL_THREADS, 0, s>>>(
             centres, radii, c->Gbuf[d].as<int4>(), c->K[d].attached.as<uint8_t>(), m, val[d]);
         AC_LAUNCHED();
     }
@@ -404,7 +415,8 @@ int eval_filtration(ac_ctx* c, const double* centres, const double* radii, doubl
 //      balls meet), each found by a binary search among b's rows; summed per lane
 //      and then over the lanes by a fixed tree.
 // Without 3. every atom read all the rows of those neighbours (600 rows for the
-// 27 that hold it): 1.65 ms for the 100,000-atom probe globule. FP64 additions go
+// 27 that hold it): 1.65 ms for the 100,000-atom probe globule; 3. and 4. take
+// 0.19 and 0.07. FP64 additions go
 // out at 16 clocks a warp however few lanes take part, so four atoms share a
 // warp and a lane of k_edge_sums steps through its own rows only.
 
@@ -444,13 +456,13 @@ __global__ void k_weights_up(BackArgs A, int d) {
     A.Wp[d][j] = W;
 }
 
-template <int K>
+template <int K, int TILE>
 __global__ void __launch_bounds__(EVAL_THREADS) k_contrib(BackArgs A) {
-    __shared__ int list[EVAL_TILE];
+    __shared__ int list[TILE];
     __shared__ int n_list;
     constexpr int d = K - 1;
-    const int64_t first = (int64_t)blockIdx.x * EVAL_TILE;
-    const int n = gather_rows(first, A.rows[d], list, &n_list, [&](int64_t j) { return A.att[d][j] != 0; });
+    const int64_t first = (int64_t)blockIdx.x * TILE;
+    const int n = gather_rows<TILE>(first, A.rows[d], list, &n_list, [&](int64_t j) { return A.att[d][j] != 0; });
     for (int u = threadIdx.x; u < n; u += EVAL_THREADS) {
         const int64_t j = first + list[u];
         double4* out = A.C[d] + j * K;
@@ -613,8 +625,14 @@ int backward(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cud
     for (int d = 0; d < 4; d++) {
         const int64_t m = A.rows[d];
         if (m == 0) continue;
-        void (*k)(BackArgs) = d == 3 ? k_contrib<4> : d == 2 ? k_contrib<3> : d == 1 ? k_contrib<2> : k_contrib<1>;
-        k<<<(unsigned)((m + EVAL_TILE - 1) / EVAL_TILE), EVAL_THREADS, 0, s>>>(A);
+        constexpr int T = EVAL_TILE, TS = EVAL_TILE_SHORT;
+        const bool shrt = m < EVAL_SHORT_ROWS;
+        void (*k)(BackArgs) = d == 3   ? (shrt ? k_contrib<4, TS> : k_contrib<4, T>)
+                              : d == 2 ? (shrt ? k_contrib<3, TS> : k_contrib<3, T>)
+                              : d == 1 ? (shrt ? k_contrib<2, TS> : k_contrib<2, T>)
+                                       : (shrt ? k_contrib<1, TS> : k_contrib<1, T>);
+        const int tile = shrt ? TS : T;
+        k<<<(unsigned)((m + tile - 1) / tile), EVAL_THREADS, 0, s>>>(A);
         AC_LAUNCHED();
     }
     const unsigned nb = (unsigned)((n * SUM_LANES + SUM_THREADS - 1) / SUM_THREADS);
