@@ -430,9 +430,10 @@ struct BackArgs {
     double* Wp[4];           // W' per row (pass 1)
     const int64_t* frows[3]; // frows[d]: rows of the attached facets (dim d) of each coface (dim d + 1), or -1
     const unsigned long long* parent[3];  // parent[d][r]: the coface (row of dim d + 1) of attached row r of dim d
-    double4* C[4];           // per unattached row, per vertex: (dL/dp, dL/dr) contributions (pass 2)
-    double4* E;              // per K^1 row: sum for its second vertex (pass 3)
-    double4* own;            // per atom: sum over the rows that start with it
+    // per row, per vertex: (dL/dp, dL/dr) contributions of the unattached rows (pass 2). Pass 3 keeps its sums in
+    // them: for the second vertex of K^1 row e in C[1][2e + 1], for the rows that start with an atom in C[0] at the
+    // atom's row (an atom without a row is in no simplex); only the lane that writes such a place has read it.
+    double4* C[4];
     int64_t rows[4];
     const int32_t* rank;     // input index -> sorted position
     const int32_t* order;    // sorted position -> input index
@@ -517,7 +518,7 @@ __global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
     }
     own = sum_lanes(own);
     if (b >= A.n) return;
-    if (sub == 0) A.own[b] = own;
+    if (sub == 0 && A.v0[0][b] < A.v0[0][b + 1]) A.C[0][A.v0[0][b]] = own;
     for (int64_t e = A.v0[1][b] + sub; e < A.v0[1][b + 1]; e += SUM_LANES) {
         const int x = A.G[1][e].y;
         double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
@@ -538,7 +539,7 @@ __global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
                 }
             }
         }
-        A.E[e] = s;
+        A.C[1][e * 2 + 1] = s;
     }
 }
 
@@ -548,7 +549,7 @@ __global__ void __launch_bounds__(SUM_THREADS) k_gather_atoms(BackArgs A, double
     const int64_t a = ((int64_t)blockIdx.x * SUM_THREADS + threadIdx.x) / SUM_LANES;
     double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
     if (a < A.n) {
-        if (sub == 0) s = A.own[a];
+        if (sub == 0 && A.v0[0][a] < A.v0[0][a + 1]) s = A.C[0][A.v0[0][a]];
         const int ia = A.rank[a];
         const int64_t off = A.nb_stride ? (int64_t)ia * A.nb_stride : A.nb_off[ia];
         const int m = A.nb_stride ? (int)A.nb_off[ia] : (int)(A.nb_off[ia + 1] - off);
@@ -562,7 +563,7 @@ __global__ void __launch_bounds__(SUM_THREADS) k_gather_atoms(BackArgs A, double
                 if (A.G[1][mid].y < a) lo = mid + 1;
                 else hi = mid;
             }
-            if (lo < end && A.G[1][lo].y == a) add4(s, A.E[lo]);
+            if (lo < end && A.G[1][lo].y == a) add4(s, A.C[1][lo * 2 + 1]);
         }
     }
     s = sum_lanes(s);
@@ -587,12 +588,9 @@ int backward(ac_ctx* c, const double* const dldf[4], double* dc, double* dr, cud
         crows += (size_t)c->K[d].count * (d + 1);
     }
     const size_t wbytes = ((wrows > 0 ? wrows : 1) * sizeof(double) + 255) & ~(size_t)255;
-    const size_t sums = (size_t)c->K[1].count + (size_t)n;  // E and own
-    AC_TRY(c->scratch[3].reserve(wbytes + (crows + sums) * sizeof(double4), s));
+    AC_TRY(c->scratch[3].reserve(wbytes + (crows > 0 ? crows : 1) * sizeof(double4), s));
     double* Wbuf = c->scratch[3].as<double>();
     double4* Cbuf = reinterpret_cast<double4*>(static_cast<char*>(c->scratch[3].p) + wbytes);
-    A.E = Cbuf + crows;
-    A.own = A.E + c->K[1].count;
     for (int d = 0; d < 4; d++) {
         const int64_t m = c->K[d].count;
         A.G[d] = c->Gbuf[d].as<int4>();

@@ -2,11 +2,13 @@
 //
 // Steps 3-5 of Section 3.1 (arXiv 1908.05944): K^d is the set of facets of
 // K^(d+1) together with the simplices of Sigma_ortho^d that pass AC2 at their
-// orthocentre. The per-atom pass emitted the latter; here both sources are
-// mapped to input indices, each tuple sorted ascending, bucketed by its first
-// vertex (counting sort over input indices), sorted and de-duplicated inside
-// each bucket. A simplex that arrives only as a facet fails AC2 at its own
-// orthocentre: it is "attached".
+// orthocentre. The per-atom pass emitted the latter. K^3 and the potential
+// simplices, each emitted once, are mapped to input indices, sorted ascending,
+// bucketed by their first vertex (counting sort over input indices) and sorted
+// inside each bucket. K^2 and K^1 are marked bits over the neighbour rows, where
+// a simplex that comes from both sources sets the same bit, and are written in
+// order from the marks. A simplex that arrives only as a facet fails AC2 at its
+// own orthocentre: it is "attached".
 //
 // Filtration value Size (Section 2.3): an unattached simplex's closest witness
 // is its orthocentre, so Size = OrthoSize; an attached simplex's closest
