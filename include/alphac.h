@@ -99,8 +99,8 @@ typedef struct {
     int64_t ac3_tests[4];   /* AC3 tests per dimension (edges: exact 64-bit integers) */
     int64_t ac3_exact;      /* triangle/tetrahedron AC3 tests the filter left to exact integers */
     double ms_total;        /* device time of the last ac_build (CUDA events) */
-    double ms_stage[8];     /* grid, neighbours, per-atom pass, canonical K3, K2, K1+K0+lists, filtration,
-                               and the per-atom kernel's own launch */
+    double ms_stage[8];     /* grid, neighbours, per-atom pass, canonical K3 (its launches: it runs beside K2), K2,
+                               K1+K0+lists, filtration, and the per-atom kernel's own launch */
     int64_t kernel_launches; /* kernels the last ac_build launched (graph nodes when replayed) */
     int32_t replayed;        /* 1: the last ac_build ran as a CUDA graph replay */
     int32_t host_syncs;      /* host waits for the device during the last ac_build */

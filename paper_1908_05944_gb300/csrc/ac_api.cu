@@ -390,7 +390,7 @@ static int scan_entry(const T* in, T* out, int64_t n, DevBuf& tmp, DevCounters* 
 
 int scan_exclusive_i64(ac_ctx* c, const int64_t* in, int64_t* out, int64_t n, cudaStream_t s) {
     return scan_entry<long long>(reinterpret_cast<const long long*>(in), reinterpret_cast<long long*>(out), n,
-                                 c->scan_tmp, c->counters.as<DevCounters>(), s);
+                                 s == c->side ? c->scan_tmp_side : c->scan_tmp, c->counters.as<DevCounters>(), s);
 }
 
 int scan_exclusive_u32_to_u32(ac_ctx* c, const uint32_t* in, uint32_t* out, int64_t n, cudaStream_t s) {
@@ -693,7 +693,7 @@ using namespace ac;
 struct CtxRes {
     int device = -1;
     cudaEvent_t ev[10] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_copy = nullptr, ev_cjoin = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_copy = nullptr, ev_cjoin = nullptr, ev_k3 = nullptr;
     cudaStream_t side = nullptr, cap_stream = nullptr, copy = nullptr;
     void* pinned = nullptr;
     size_t pinned_bytes = 0;
@@ -710,6 +710,7 @@ static void res_free(CtxRes& r) {
     if (r.ev_join) cudaEventDestroy(r.ev_join);
     if (r.ev_copy) cudaEventDestroy(r.ev_copy);
     if (r.ev_cjoin) cudaEventDestroy(r.ev_cjoin);
+    if (r.ev_k3) cudaEventDestroy(r.ev_k3);
     if (r.side) cudaStreamDestroy(r.side);
     if (r.copy) cudaStreamDestroy(r.copy);
     if (r.cap_stream) cudaStreamDestroy(r.cap_stream);
@@ -738,6 +739,7 @@ static int res_take(size_t pinned_bytes, CtxRes& out) {
          cudaEventCreateWithFlags(&r.ev_join, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&r.ev_copy, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&r.ev_cjoin, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventCreateWithFlags(&r.ev_k3, cudaEventDisableTiming) == cudaSuccess &&
          cudaStreamCreateWithFlags(&r.side, cudaStreamNonBlocking) == cudaSuccess &&
          cudaStreamCreateWithFlags(&r.copy, cudaStreamNonBlocking) == cudaSuccess &&
          cudaStreamCreateWithFlags(&r.cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -862,6 +864,7 @@ static int create_impl(const double* centres, const double* radii, const int64_t
         c->ev_join = r.ev_join;
         c->ev_copy = r.ev_copy;
         c->ev_cjoin = r.ev_cjoin;
+        c->ev_k3 = r.ev_k3;
         c->side = r.side;
         c->copy = r.copy;
         c->cap_stream = r.cap_stream;
@@ -1066,7 +1069,12 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
     }
     if (!replayed) {
         drop_graph(c);
-        AC_TRY(build_body(c, s));
+        const int rc = build_body(c, s);
+        if (rc != AC_OK && c->os_forked) {  // nothing of a failed build runs on beside the next one
+            cudaStreamSynchronize(c->side);
+            c->os_forked = false;
+        }
+        AC_TRY(rc);
         AC_TRY(read_counters(c, &h, s));
     }
     if (h.err & DERR_INTERNAL)
@@ -1305,6 +1313,7 @@ extern "C" void ac_destroy(ac_ctx* c) {
     r.ev_join = c->ev_join;
     r.ev_copy = c->ev_copy;
     r.ev_cjoin = c->ev_cjoin;
+    r.ev_k3 = c->ev_k3;
     r.side = c->side;
     r.copy = c->copy;
     r.cap_stream = c->cap_stream;
@@ -1312,7 +1321,7 @@ extern "C" void ac_destroy(ac_ctx* c) {
     r.pinned_bytes = c->h_pinned_bytes;
     // a set from a failed creation is incomplete: free it rather than cache it
     bool whole = r.device >= 0 && r.pinned && r.side && r.cap_stream && r.copy && r.ev_fork && r.ev_join &&
-                 r.ev_copy && r.ev_cjoin;
+                 r.ev_copy && r.ev_cjoin && r.ev_k3;
     for (int k = 0; k < 10; k++) whole = whole && r.ev[k];
     if (whole && cudaGetLastError() == cudaSuccess) res_give(r);
     else res_free(r);

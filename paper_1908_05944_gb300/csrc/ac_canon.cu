@@ -298,24 +298,18 @@ __global__ void __launch_bounds__(CSORT_WARPS * 32) k_canon_sort(int4* __restric
 
 using Work = CanonWork;
 
-// one list from items emitted once each: their number is the row count
+// One list from items emitted once each: their number is the row count. Its
+// buffers are reserved on stream s; its kernels run on stream t (s, or a stream
+// that waits here for s).
 template <int K>
 static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, SimplexList& L, DevBuf& Gout, Work& w,
-                       cudaStream_t s) {
+                       cudaStream_t s, cudaStream_t t) {
     const int64_t n = c->n;
     AC_TRY(w.T.reserve((size_t)(nA + 1) * sizeof(int4), s));
     AC_TRY(w.cnt.reserve((size_t)(n + 1) * sizeof(int64_t), s));
     AC_TRY(L.v0_off.reserve((size_t)(n + 1) * sizeof(int64_t), s));
     int64_t* cnt = w.cnt.as<int64_t>();
     int64_t* off = L.v0_off.as<int64_t>();  // the rows start where the buckets do
-    AC_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(n + 1) * sizeof(int64_t), s));
-    CanonArgs ca{a4, a2, nA, c->order.as<int32_t>(), cnt, off, w.T.as<int4>()};
-    const unsigned gi = (unsigned)((nA + 255) / 256);
-    if (nA > 0) {
-        k_canon_count<K><<<gi, 256, 0, s>>>(ca);
-        AC_LAUNCHED();
-    }
-    AC_TRY(scan_exclusive_i64(c, cnt, off, n, s));
     if (c->replaying) AC_TRY(expect_i64(c, off + n, L.count, s));  // the recorded build's count
     else L.count = nA;
     L.cap = L.count;
@@ -328,8 +322,20 @@ static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, Si
     AC_TRY(L.src_dim.reserve(rows, s));
     AC_TRY(L.src_idx.reserve(rows * sizeof(int64_t), s));
     AC_TRY(Gout.reserve(rows * sizeof(int4), s));
+    if (t != s) {
+        AC_CUDA(cudaEventRecord(c->ev_fork, s));
+        AC_CUDA(cudaStreamWaitEvent(t, c->ev_fork, 0));
+    }
+    AC_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(n + 1) * sizeof(int64_t), t));
+    CanonArgs ca{a4, a2, nA, c->order.as<int32_t>(), cnt, off, w.T.as<int4>()};
+    const unsigned gi = (unsigned)((nA + 255) / 256);
     if (nA > 0) {
-        k_canon_scatter<K><<<gi, 256, 0, s>>>(ca);
+        k_canon_count<K><<<gi, 256, 0, t>>>(ca);
+        AC_LAUNCHED();
+    }
+    AC_TRY(scan_exclusive_i64(c, cnt, off, n, t));
+    if (nA > 0) {
+        k_canon_scatter<K><<<gi, 256, 0, t>>>(ca);
         AC_LAUNCHED();
         int dev = 0, sms = 0, per_sm = 0;
         AC_CUDA(cudaGetDevice(&dev));
@@ -340,18 +346,18 @@ static int canon_dim_k(ac_ctx* c, const int4* a4, const int2* a2, int64_t nA, Si
         if (blocks > (int64_t)sms * (per_sm > 0 ? per_sm : 1)) blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
         CanonOut o{c->mol_of.as<int32_t>(), c->d_moloff.as<int64_t>(), Gout.as<int4>(), L.tuples.as<int32_t>(),
                    L.attached.as<uint8_t>(), &c->counters.as<DevCounters>()->err};
-        k_canon_sort<K><<<(unsigned)blocks, CSORT_WARPS * 32, 0, s>>>(w.T.as<int4>(), off, n, o);
+        k_canon_sort<K><<<(unsigned)blocks, CSORT_WARPS * 32, 0, t>>>(w.T.as<int4>(), off, n, o);
         AC_LAUNCHED();
     }
     return AC_OK;
 }
 
 static int canon_dim(ac_ctx* c, int d, const int4* a4, const int2* a2, int64_t nA, SimplexList& L, DevBuf& Gout, Work& w,
-                     cudaStream_t s) {
+                     cudaStream_t s, cudaStream_t t) {
     switch (d) {
-        case 1: return canon_dim_k<2>(c, a4, a2, nA, L, Gout, w, s);
-        case 2: return canon_dim_k<3>(c, a4, a2, nA, L, Gout, w, s);
-        default: return canon_dim_k<4>(c, a4, a2, nA, L, Gout, w, s);
+        case 1: return canon_dim_k<2>(c, a4, a2, nA, L, Gout, w, s, t);
+        case 2: return canon_dim_k<3>(c, a4, a2, nA, L, Gout, w, s, t);
+        default: return canon_dim_k<4>(c, a4, a2, nA, L, Gout, w, s, t);
     }
 }
 
@@ -925,13 +931,21 @@ __global__ void k_mol_rows(MolRowsArgs a) {
     for (int l = 0; l < 7; l++) a.out[l * (a.n_mol + 1) + m] = a.v0_off[l] ? a.v0_off[l][at] : 0;
 }
 
-static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s);
+static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s, cudaStream_t from);
 
 // the row counts, beside the counters the host reads last
 __global__ void k_row_counts(const int64_t* n0, const int64_t* n1, const int64_t* n2, DevCounters* cnt) {
     const int64_t* p[3] = {n0, n1, n2};
     if (threadIdx.x < 3) cnt->n_rows[threadIdx.x] = *p[threadIdx.x];
 }
+
+// Up to this many atoms K^3 is canonicalised beside K^2: four launches, each of them
+// too short or too unevenly filled to use the whole chip, leave the critical path
+// (replay of a 100,000-atom build 1,384 -> 1,352 us, first build 1,470 -> 1,436;
+// 250,000 atoms 3,205 -> 3,181; even from 500,000 on). For 3.0 M atoms both are
+// bound by the traffic of their scattered rows and masks, and side by side they
+// took 0.5 ms longer (37.9 -> 38.4 ms).
+constexpr int64_t K3_BESIDE_MAX_ATOMS = 1 << 20;
 
 int canonicalise(ac_ctx* c, cudaStream_t s) {
     const DevCounters& h = c->hc;  // counters read at the end of the per-atom pass
@@ -940,17 +954,24 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
     Work& w = c->cw;
     const int64_t n = c->n;
     c->deferred = !c->replaying && !c->opt.host_results && n <= DEFER_MAX_ATOMS;
-    // K^3
-    AC_TRY(canon_dim(c, 3, c->tet_out.as<int4>(), nullptr, (int64_t)h.n_tet_out, c->K[3], c->Gbuf[3], w, s));
-    AC_TRY(fork_orthosize(c, 3, s));
+    // K^3: its facets are marked from the tetrahedra as emitted, so K^2 does not wait for its rows, only the
+    // filtration does, which runs on the side stream too
+    const bool beside = n <= K3_BESIDE_MAX_ATOMS;
+    const cudaStream_t t3 = beside ? c->side : s;
+    AC_TRY(canon_dim(c, 3, c->tet_out.as<int4>(), nullptr, (int64_t)h.n_tet_out, c->K[3], c->Gbuf[3], c->cw_k3, s, t3));
+    if (beside) {
+        c->os_forked = true;
+        AC_CUDA(cudaEventRecord(c->ev_k3, t3));
+    }
+    AC_TRY(fork_orthosize(c, 3, s, t3));
     AC_TRY(stage_mark(c, 4, s));
     // K^2 = unattached triangles + facets of K^3
     AC_TRY(canon_tris_by_marks(c, s));
-    AC_TRY(fork_orthosize(c, 2, s));
+    AC_TRY(fork_orthosize(c, 2, s, s));
     AC_TRY(stage_mark(c, 5, s));
     // K^1 = unattached edges + edges of K^2, by marks over the neighbour rows
     AC_TRY(canon_edges_by_marks(c, s));
-    AC_TRY(fork_orthosize(c, 1, s));
+    AC_TRY(fork_orthosize(c, 1, s, s));
     // K^0
     {
         SimplexList& L = c->K[0];
@@ -988,14 +1009,14 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
             AC_LAUNCHED();
         }
     }
-    AC_TRY(fork_orthosize(c, 0, s));
+    AC_TRY(fork_orthosize(c, 0, s, s));
     // estimation-pass lists, when kept (single molecule)
     if (c->pc.keep_candidates) {
         for (int d = 1; d <= 3; d++) {
             int64_t m = (int64_t)h.n_cand_out[d];
             // each candidate is emitted once, by its owner
             AC_TRY(canon_dim(c, d, d >= 2 ? c->cand[d].as<int4>() : nullptr, d == 1 ? c->cand[1].as<int2>() : nullptr, m,
-                             c->C[d], c->CGbuf[d], w, s));
+                             c->C[d], c->CGbuf[d], w, s, s));
         }
     }
     if (c->deferred) {
@@ -1003,6 +1024,7 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
         AC_LAUNCHED();
     }
     if (c->n_mol == 1) return AC_OK;  // its rows are the whole lists (finish_mol_rows)
+    if (beside) AC_CUDA(cudaStreamWaitEvent(s, c->ev_k3, 0));  // K^3's offsets
     // per-molecule row ranges, copied to the host with the build's last transfer
     MolRowsArgs ma{};
     for (int d = 0; d < 4; d++) ma.v0_off[d] = c->K[d].v0_off.as<int64_t>();
@@ -1396,12 +1418,12 @@ static int copy_values_to_host(ac_ctx* c, int d, cudaStream_t from) {
 }
 
 // The filtration of list d on the side stream, as soon as the list's rows are
-// final, overlapping the canonicalisation of the lower dimensions: OrthoSize
+// final (written on stream `from`: s or the side stream), overlapping the canonicalisation of the lower dimensions: OrthoSize
 // (with the initial Size, source and coface key), then for d < 3 the two
 // coface passes over K^(d+1), whose values are final by then (the side stream
 // ran its passes first). compute_filtration joins the side stream. Each pass
 // has its own buffers, reserved here on the build's stream before the fork.
-static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
+static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s, cudaStream_t from) {
     SimplexList& L = c->K[d];
     const int64_t m = L.cap;
     if (m == 0) return AC_OK;
@@ -1413,7 +1435,7 @@ static int fork_orthosize(ac_ctx* c, int d, cudaStream_t s) {
         AC_TRY(c->fargs[d].reserve((size_t)m * sizeof(unsigned long long), s));
         if (mu > 0) AC_TRY(c->frows[d].reserve((size_t)mu * (d + 2) * sizeof(int64_t), s));
     }
-    AC_TRY(copy_rows_to_host(c, d, s));
+    AC_TRY(copy_rows_to_host(c, d, from));
     AC_CUDA(cudaEventRecord(c->ev_fork, s));
     cudaStream_t t = c->side;
     AC_CUDA(cudaStreamWaitEvent(t, c->ev_fork, 0));

@@ -288,7 +288,7 @@ struct ac_ctx {
     bool deferred = false;        // this build reads the rows of K^0..K^2 with its last wait
     uint8_t* endpoint = nullptr;  // K^1's endpoint flags by input index (within scratch[2], this build's)
     ac::DevBuf pair_moff;    // first pair-mask word of each sorted position (n + 1)
-    ac::DevBuf scan_tmp;
+    ac::DevBuf scan_tmp, scan_tmp_side;  // scans on the build's stream and on the side stream
 
     ac::DevCounters hc{};             // host copy of the counters from the last readback
     void* h_pinned = nullptr;         // one page-locked block holding the four readback areas below
@@ -308,7 +308,7 @@ struct ac_ctx {
     cudaGraphExec_t graph_exec = nullptr;
     long long graph_launches = 0; // kernels in the graph
     int host_syncs = 0;           // host waits in the current build
-    ac::CanonWork cw;
+    ac::CanonWork cw, cw_k3;  // K^3 has its own: it is canonicalised beside K^2
 
     ac_stats stats{};
     int res_device = -1;        // device of the cached CUDA objects below
@@ -317,7 +317,7 @@ struct ac_ctx {
     cudaStream_t side = nullptr;                    // wide-row launch, concurrent with the narrow one
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t copy = nullptr;                    // host copies of the lists (opt.host_results)
-    cudaEvent_t ev_copy = nullptr, ev_cjoin = nullptr;
+    cudaEvent_t ev_copy = nullptr, ev_cjoin = nullptr, ev_k3 = nullptr;
     bool copy_forked = false;                       // copies on the copy stream await their join
     int local_launches = 0;
 };
