@@ -141,7 +141,7 @@ struct WarpSmem : PointsD<32 * WORDS, R> {
     int n_tet, n_tri, n_edge;
     int n_tl;                         // tetrahedra pushed (the list holds the first TL_CAP)
     unsigned cand[CAND_CAP];          // triangle candidate codes (p | k << SH) of the current batch
-    static constexpr int TL_CAP = WORDS > 2 ? 256 : 128;
+    static constexpr int TL_CAP = WORDS > 4 ? 1024 : WORDS > 2 ? 256 : 128;
     unsigned tl[TL_CAP];              // tetrahedra to settle: p | k << SH | l << 2 SH [| TET_OPEN]
     int4 st_tet[STAGE];
     int4 st_tri[STAGE];
@@ -1201,6 +1201,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
                                 else atomicOr(&cnt->err, DERR_OVF_CAND);
                             }
                         }
+                    }
+                    // Long rows with many undecided lines (radii over a factor of 16: 1,000 such
+                    // tetrahedra per atom) would fill the list long before the rows are done, and what does
+                    // not fit is left to the exact kernels: 200,000 such particles 215 ms a build, 134 of them
+                    // there; 89 settled so, 83 with lists of 1,024. Rows of two words do not fill theirs.
+                    if constexpr (WORDS > 2) {
+                        __syncwarp();
+                        if (S.n_tl > SM::TL_CAP / 2) settle_tets();
                     }
                     if (!__any_sync(FULL, pass || pend || (keep && keep_it))) continue;  // nothing to append
                     const int4 item = make_int4(i, valid ? S.idx[pp] : 0, valid ? S.idx[kk] : 0, 0);
