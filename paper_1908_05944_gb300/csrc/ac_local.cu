@@ -76,7 +76,8 @@
 //     - (q_x.u)^2 with an allowance of 64 u H^2 for every rounding in it.
 // A simplex whose AC3, or whose AC2 with no decided violator, stays open is
 // appended to a pending list (the tetrahedra over an undecided triangle are
-// tested all the same). Two kernels settle the pending simplices: k_resolve_prep,
+// tested all the same: its segment's lower bound is 0, ac_reach.h, which decides
+// none of their AC3). Two kernels settle the pending simplices: k_resolve_prep,
 // one thread per simplex, takes the exact AC3 in 128-bit integers and the FP64
 // orthocentre from the exact integer minors (relative error <= 4.0001 u_64 per
 // component of y); then k_resolve_scan, a group of lanes per simplex whose AC3
@@ -109,6 +110,7 @@
 #include <math.h>
 
 #include "ac_internal.cuh"
+#include "ac_reach.h"
 
 namespace ac {
 
@@ -545,7 +547,8 @@ __device__ __forceinline__ TriLine<float> tri_line(const P4<float>& q1, const P4
     o.ey = A::mul_up(B.H, A::fma_up(2.0f, emu, A::mul_up(B.ky, A::add_up(A::abs(m1), A::abs(m2)))));
     float S, eS;
     norm2(o, B, S, eS);
-    L.ac3 = ac3_of(S, eS, T);
+    const Reach<float> t = reach_of<A>(T, S, eS);  // of T - |y|^2
+    L.ac3 = t.ac3;
     L.z0 = -2.0f * o.y0;
     L.z1 = -2.0f * o.y1;
     L.z2 = -2.0f * o.y2;
@@ -553,10 +556,8 @@ __device__ __forceinline__ TriLine<float> tri_line(const P4<float>& q1, const P4
     L.n1 = cross_c(q1.z, q2.x, q1.x, q2.z);
     L.n2 = cross_c(q1.x, q2.y, q1.y, q2.x);
     // S^2 = (T - |y|^2) / det, 1 / det between inv (1 - 64 u) (1 - rho) and inv (1 + 1.2 rho)
-    const float t_up = A::max(A::add_up(A::add_up(T, -S), eS), 0.0f);
-    const float t_lo = A::max(A::sub_dn(A::sub_dn(T, S), eS), 0.0f);
-    const float s2_up = A::mul_up(A::mul_up(t_up, inv), A::fma_up(1.2f, rho, 1.0f));
-    const float s2_lo = A::mul_dn(A::mul_dn(t_lo, A::mul_dn(inv, B.inv_lo)), A::sub_dn(1.0f, rho));
+    const float s2_up = A::mul_up(A::mul_up(t.up, inv), A::fma_up(1.2f, rho, 1.0f));
+    const float s2_lo = A::mul_dn(A::mul_dn(t.lo, A::mul_dn(inv, B.inv_lo)), A::sub_dn(1.0f, rho));
     L.s2 = 2.0f * sqrt_up(s2_up);
     L.s2lo = 2.0f * sqrt_dn(s2_lo);
     L.E = A::mul_up(A::fma_up(B.K1, o.ey, B.K0), B.up1);
