@@ -198,8 +198,8 @@ AC_API int ac_get_candidates(ac_ctx* ctx, int dim, const int32_t** d_tuples, int
  * fixed: each simplex keeps its source simplex (the one whose orthocentre is
  * its closest witness) and takes that source's OrthoSize, in FP64.
  * d_f_out[dim] receives one double per simplex of dim (device, caller-owned;
- * NULL skips that dimension, whose values, if a lower one may take some of
- * them, go to scratch of 8 bytes each). For finite-difference checks of
+ * NULL skips that dimension; a lower one's rows evaluate what they take from
+ * it themselves). Allocates nothing. For finite-difference checks of
  * ac_backward.
  * The value is the Size of Section 2.3 through its source. Errors:
  * AC_ERR_INVALID_ARG (NULL ctx or inputs), AC_ERR_STATE (no build),
