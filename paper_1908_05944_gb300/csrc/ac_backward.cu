@@ -457,7 +457,7 @@ int eval_filtration(ac_ctx* c, const double* centres, const double* radii, doubl
 //   2. k_contrib, the unattached rows: the orthocentre and barycentric
 //      coordinates of s, and for each vertex k of s the contribution
 //      (2 W_s lambda_k (p_k - c), -2 W_s lambda_k r_k).
-//   3. k_edge_sums, eight lanes per atom b: of the rows with first vertex b, the
+//   3. k_edge_sums, eight lanes per atom b (a block for one with many rows): of the rows with first vertex b, the
 //      contributions to b itself, and to each other vertex x. Such an x is the
 //      second vertex of a K^1 row with first vertex b, and its sum is written
 //      there (lane by lane in row order, so the order is fixed).
@@ -558,9 +558,45 @@ __device__ __forceinline__ double4 sum_lanes(double4 s) {
     return s;
 }
 
+// the sum of K^1 row e = (b, x): the edge's own contribution to x and those of b's triangles and tetrahedra
+__device__ __forceinline__ void edge_sum(const BackArgs& A, int64_t b, int64_t e) {
+    const int x = A.G[1][e].y;
+    double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (!A.att[1][e]) s = A.C[1][e * 2 + 1];  // the edge itself
+    for (int d = 2; d < 4; d++) {
+        const int64_t r1 = A.v0[d][b + 1];
+        for (int64_t r0 = A.v0[d][b]; r0 < r1; r0 += 32) {
+            const int cnt = (int)(r1 - r0 < 32 ? r1 - r0 : 32);
+            unsigned mask = 0u;  // of these rows, the unattached ones with vertex x
+            for (int t = 0; t < cnt; t++) {
+                const int4 g = A.G[d][r0 + t];
+                if ((g.y == x || g.z == x || g.w == x) && !A.att[d][r0 + t]) mask |= 1u << t;
+            }
+            for (; mask; mask &= mask - 1) {
+                const int64_t r = r0 + __ffs(mask) - 1;
+                const int4 g = A.G[d][r];
+                add4(s, A.C[d][r * (d + 1) + (g.y == x ? 1 : g.z == x ? 2 : 3)]);
+            }
+        }
+    }
+    A.C[1][e * 2 + 1] = s;
+}
+
+// Every edge of b goes over all of b's rows, so the work is their product: about
+// 150 for an atom of a probe globule, but 900 edges times 6,000 rows for a large
+// ball among small ones that comes before them in the input. Such atoms take the
+// whole block (each edge is still summed by one lane in row order: the same
+// numbers). Eight such balls of 900 neighbours, a whole backward: 2.6 ms; eight
+// lanes each: 21.6 ms. The line leaves the eight lanes at most 1,024 rows each, about
+// what they wait for on the other loads.
+constexpr int64_t SUM_BLOCK_WORK = 8192;
+
 __global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
+    __shared__ int64_t wide[SUM_THREADS / SUM_LANES];  // this block's atoms above the line
+    __shared__ int n_wide;
     const int sub = threadIdx.x % SUM_LANES;
     const int64_t b = ((int64_t)blockIdx.x * SUM_THREADS + threadIdx.x) / SUM_LANES;
+    if (threadIdx.x == 0) n_wide = 0;
     double4 own = make_double4(0.0, 0.0, 0.0, 0.0);
     if (b < A.n) {
         for (int d = 0; d < 4; d++)
@@ -568,30 +604,20 @@ __global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
                 if (!A.att[d][r]) add4(own, A.C[d][r * (d + 1)]);
     }
     own = sum_lanes(own);
-    if (b >= A.n) return;
-    if (sub == 0 && A.v0[0][b] < A.v0[0][b + 1]) A.C[0][A.v0[0][b]] = own;
-    for (int64_t e = A.v0[1][b] + sub; e < A.v0[1][b + 1]; e += SUM_LANES) {
-        const int x = A.G[1][e].y;
-        double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
-        if (!A.att[1][e]) s = A.C[1][e * 2 + 1];  // the edge itself
-        for (int d = 2; d < 4; d++) {
-            const int64_t r1 = A.v0[d][b + 1];
-            for (int64_t r0 = A.v0[d][b]; r0 < r1; r0 += 32) {
-                const int cnt = (int)(r1 - r0 < 32 ? r1 - r0 : 32);
-                unsigned mask = 0u;  // of these rows, the unattached ones with vertex x
-                for (int t = 0; t < cnt; t++) {
-                    const int4 g = A.G[d][r0 + t];
-                    if ((g.y == x || g.z == x || g.w == x) && !A.att[d][r0 + t]) mask |= 1u << t;
-                }
-                for (; mask; mask &= mask - 1) {
-                    const int64_t r = r0 + __ffs(mask) - 1;
-                    const int4 g = A.G[d][r];
-                    add4(s, A.C[d][r * (d + 1) + (g.y == x ? 1 : g.z == x ? 2 : 3)]);
-                }
-            }
+    __syncthreads();
+    if (b < A.n) {
+        if (sub == 0 && A.v0[0][b] < A.v0[0][b + 1]) A.C[0][A.v0[0][b]] = own;
+        const int64_t e0 = A.v0[1][b], e1 = A.v0[1][b + 1];
+        const int64_t rows = A.v0[2][b + 1] - A.v0[2][b] + A.v0[3][b + 1] - A.v0[3][b];
+        if ((e1 - e0) * rows > SUM_BLOCK_WORK) {
+            if (sub == 0) wide[atomicAdd(&n_wide, 1)] = b;
+        } else {
+            for (int64_t e = e0 + sub; e < e1; e += SUM_LANES) edge_sum(A, b, e);
         }
-        A.C[1][e * 2 + 1] = s;
     }
+    __syncthreads();
+    for (int k = 0; k < n_wide; k++)
+        for (int64_t e = A.v0[1][wide[k]] + threadIdx.x; e < A.v0[1][wide[k] + 1]; e += SUM_THREADS) edge_sum(A, wide[k], e);
 }
 
 __global__ void __launch_bounds__(SUM_THREADS) k_gather_atoms(BackArgs A, double* __restrict__ dX,
