@@ -296,7 +296,8 @@ AC_API int ac_subcomplex(ac_ctx* ctx, int dim, int64_t mol, double alpha2, uint8
  * not 0, in list order, to d_rows (count_in x (dim + 1) int32), and their
  * filtration values (as ac_filtration_values) to d_f (count_in doubles).
  * count_in is ac_subcomplex's count; rows past it are not written. Caller-owned
- * DEVICE arrays; either output may be NULL. Enqueued on stream, does not wait.
+ * DEVICE arrays; either output may be NULL. Enqueued on stream, does not wait:
+ * an ac_build on another stream has to be ordered after it by the caller.
  * Errors: AC_ERR_INVALID_ARG (bad dim/mol, NULL flags, count_in < 0),
  * AC_ERR_STATE (no build yet), AC_ERR_OOM, AC_ERR_CUDA.
  */
@@ -311,7 +312,8 @@ AC_API int ac_subcomplex_lists(ac_ctx* ctx, int dim, int64_t mol, const uint8_t*
 /*
  * Copy list `what` of (dim, mol) of the complex (Section 2.4), count rows, to dst (device or host
  * memory), enqueued on stream; does not wait (a pageable dst may make the copy
- * itself wait). count must be the list's length. Errors: AC_ERR_INVALID_ARG
+ * itself wait): an ac_build on another stream has to be ordered after it by the
+ * caller. count must be the list's length. Errors: AC_ERR_INVALID_ARG
  * (bad what/dim/mol, another count, NULL dst with rows to copy), AC_ERR_STATE,
  * AC_ERR_CUDA.
  */

@@ -341,7 +341,9 @@ class AlphaComplex:
         return flags[:m], cnt.value
 
     def subcomplex(self, alpha2: float, mol: int = -1, stream=None):
-        """The alpha complex at alpha2 <= alpha from this build: per dimension (simplices, Size values)."""
+        """The alpha complex at alpha2 <= alpha from this build: per dimension (simplices, Size values).
+
+        The reads of the context are over when it returns: a build on another stream may follow at once."""
         import torch
         index = torch.cuda.current_device()
         out = []
@@ -353,6 +355,7 @@ class AlphaComplex:
                 _check(lib().ac_subcomplex_lists(self._h, d, mol, mask.data_ptr(), n, rows.data_ptr(), f.data_ptr(),
                                                  _current_stream(torch, index)), "ac_subcomplex_lists")
             out.append((rows, f))
+        torch.cuda.current_stream(index).synchronize()
         return out
 
     def stats(self) -> dict:
