@@ -587,9 +587,11 @@ __device__ __forceinline__ void edge_sum(const BackArgs& A, int64_t b, int64_t e
 // ball among small ones that comes before them in the input. Such atoms take the
 // whole block (each edge is still summed by one lane in row order: the same
 // numbers). Eight such balls of 900 neighbours, a whole backward: 2.6 ms; eight
-// lanes each: 21.6 ms. The line leaves the eight lanes at most 1,024 rows each, about
-// what they wait for on the other loads.
-constexpr int64_t SUM_BLOCK_WORK = 8192;
+// lanes each: 21.6 ms. The line, backward in us at 2,048 / 4,096 / 8,192 / 16,384:
+// 256 balls of 300 neighbours 195 / 200 / 247 / 281, spread radii (20,000 balls)
+// 232 / 221 / 241 / 250, globules of 2,000 atoms 197 / 187 / 187 / 174 and 100,000
+// 734 / 709 / 706 / 697 (below the line no block waits for a wide atom).
+constexpr int64_t SUM_BLOCK_WORK = 4096;
 
 __global__ void __launch_bounds__(SUM_THREADS) k_edge_sums(BackArgs A) {
     __shared__ int64_t wide[SUM_THREADS / SUM_LANES];  // this block's atoms above the line
