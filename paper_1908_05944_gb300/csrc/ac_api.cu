@@ -994,6 +994,7 @@ static int capture_replay(ac_ctx* c) {
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(s, &g);
     if (rc != AC_OK || e != cudaSuccess || !g) {
+        c->os_forked = c->copy_forked = false;  // nothing of it ran
         if (g) cudaGraphDestroy(g);
         cudaGetLastError();
         return rc != AC_OK ? rc : fail(AC_ERR_CUDA, "graph capture of the build failed");
@@ -1039,6 +1040,17 @@ static int record_build(ac_ctx* c, const DevCounters& post, cudaStream_t s) {
     return AC_OK;
 }
 
+// Nothing of a build that failed half way runs on beside the next one, whatever it had forked by then: the wide tiers
+// of the per-atom pass, K^3 and the filtration on the side stream, copies of lists into page-locked blocks (which the
+// next build may hand to another context). The error it failed with stands.
+static void stop_failed_build(ac_ctx* c, cudaStream_t s) {
+    cudaStreamSynchronize(s);
+    cudaStreamSynchronize(c->side);
+    cudaStreamSynchronize(c->copy);
+    c->os_forked = false;
+    c->copy_forked = false;
+}
+
 extern "C" int ac_build(ac_ctx* c, void* stream) {
     if (!c) return fail(AC_ERR_INVALID_ARG, "ctx is NULL");
     cudaStream_t s = (cudaStream_t)stream;
@@ -1069,11 +1081,9 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
     }
     if (!replayed) {
         drop_graph(c);
+        c->rec.valid = false;  // from here the lists' sizes are this build's: no replay rests on them unless it succeeds
         const int rc = build_body(c, s);
-        if (rc != AC_OK && c->os_forked) {  // nothing of a failed build runs on beside the next one
-            cudaStreamSynchronize(c->side);
-            c->os_forked = false;
-        }
+        if (rc != AC_OK) stop_failed_build(c, s);
         AC_TRY(rc);
         AC_TRY(read_counters(c, &h, s));
     }
