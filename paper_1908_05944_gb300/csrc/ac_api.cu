@@ -1056,6 +1056,7 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     StreamScope scope(s);
     c->built = false;
+    c->deferred = false;
     c->host_syncs = 0;
     const long long launches0 = g_launch_count;
     bool replayed = false;
@@ -1082,8 +1083,14 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
     if (!replayed) {
         drop_graph(c);
         c->rec.valid = false;  // from here the lists' sizes are this build's: no replay rests on them unless it succeeds
-        const int rc = build_body(c, s);
+        int rc = build_body(c, s);
         if (rc != AC_OK) stop_failed_build(c, s);
+        if (rc == AC_ERR_OOM && c->deferred) {  // no room for lists of upper bounds: once more, waiting for their counts
+            drop_lists(c);
+            c->no_defer = true;
+            rc = build_body(c, s);
+            if (rc != AC_OK) stop_failed_build(c, s);
+        }
         AC_TRY(rc);
         AC_TRY(read_counters(c, &h, s));
     }
@@ -1096,8 +1103,10 @@ extern "C" int ac_build(ac_ctx* c, void* stream) {
         c->rec.valid = false;
         return fail(AC_ERR_TIMEOUT, "a bounded device wait (scan look-back) ran out");
     }
-    if (!replayed && c->deferred)
+    if (!replayed && c->deferred) {
         for (int d = 0; d < 3; d++) c->K[d].count = (int64_t)h.n_rows[d];
+        settle_slack(c);
+    }
     if (!replayed && !c->opt.no_graph) AC_TRY(record_build(c, h, s));
     finish_mol_rows(c);
     const DevCounters& hl = h;  // the per-atom pass wrote them; later stages add only error bits
@@ -1315,6 +1324,7 @@ extern "C" void ac_destroy(ac_ctx* c) {
         ~IdleScope() { g_release_idle = false; }
     } idle_scope(idle);
     drop_graph(c);
+    forget_slack(c);
     for (int d = 0; d < 4; d++) host_block_give(c->hres[d], c->hres_bytes[d]);
     CtxRes r;
     r.device = c->res_device;

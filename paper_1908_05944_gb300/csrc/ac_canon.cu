@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "ac_internal.cuh"
@@ -552,10 +553,63 @@ __global__ void __launch_bounds__(EW_WARPS * 32) k_edge_write(EdgeMarkArgs a, in
 
 // Up to this many atoms a build does not wait for the row counts of K^2, K^1 and
 // K^0 one after another (about 13 us each, GPU idle): their buffers and launches
-// cover an upper bound known after the per-atom pass (about 2.5 times the rows,
-// 5 KB per atom in all) and the kernels read the counts on the device. Above,
-// the memory costs more than three waits (2 % of a 100,000-atom build).
+// cover an upper bound known after the per-atom pass (about 2.5 times the rows)
+// and the kernels read the counts on the device. Above, the memory costs more
+// than three waits (2 % of a 100,000-atom build).
+//
+// A context keeps these buffers (60,000 atoms with probe radii: 413 MB in all,
+// 240 with buffers of the rows' sizes), so the bytes beyond the rows are bounded:
+// while the contexts of the process hold more than DEFER_MAX_SLACK of them, further
+// builds wait for their counts, and so does one that the device has no room for
+// (ac_build). The lists are the same either way.
 constexpr int64_t DEFER_MAX_ATOMS = 65536;
+constexpr int64_t DEFER_MAX_SLACK = (int64_t)4 << 30;
+static std::atomic<int64_t> g_slack{0};
+
+// upper bounds: a row of K^2 is a free triangle or a facet of a K^3 row; an edge
+// of K^1 joins neighbours, and is free or an edge of a K^2 row
+static int64_t tri_rows_bound(const DevCounters& h) { return (int64_t)h.n_tri_pass + 4 * (int64_t)h.n_tet_out; }
+static int64_t edge_rows_bound(const ac_ctx* c, int64_t tri_rows) {
+    return std::min((c->nb_total + 1) / 2, (int64_t)c->hc.n_edge_pass + 3 * tri_rows);
+}
+
+// bytes per row of list d (0..2): indices, flag, two values, source, canonical row, coface key and argmin, facet rows
+static int64_t list_row_bytes(int d) { return 4 * (d + 1) + 1 + 2 * 8 + 9 + 16 + 2 * 8 + (d > 0 ? 8 * (d + 1) : 0); }
+
+static bool may_defer(ac_ctx* c) {
+    if (c->replaying || c->opt.host_results || c->no_defer || c->n > DEFER_MAX_ATOMS) return false;
+    const int64_t tri = tri_rows_bound(c->hc);
+    const int64_t all = c->n * list_row_bytes(0) + edge_rows_bound(c, tri) * list_row_bytes(1) + tri * list_row_bytes(2);
+    const int64_t more = all - c->slack;  // as if there were no rows, until they are counted
+    if (g_slack.fetch_add(more) + more > DEFER_MAX_SLACK) {
+        g_slack.fetch_sub(more);
+        return false;
+    }
+    c->slack = all;
+    return true;
+}
+
+void settle_slack(ac_ctx* c) {
+    int64_t now = 0;
+    for (int d = 0; d < 3; d++) now += (c->K[d].cap - c->K[d].count) * list_row_bytes(d);
+    g_slack.fetch_add(now - c->slack);
+    c->slack = now;
+}
+
+void forget_slack(ac_ctx* c) {
+    g_slack.fetch_sub(c->slack);
+    c->slack = 0;
+}
+
+void drop_lists(ac_ctx* c) {
+    for (int d = 0; d < 3; d++) {
+        SimplexList& L = c->K[d];
+        for (DevBuf* b : {&L.tuples, &L.attached, &L.f, &L.orthosize, &L.src_dim, &L.src_idx, &c->Gbuf[d], &c->fkey[d],
+                          &c->fargs[d], &c->frows[d]})
+            *b = DevBuf{};
+    }
+    forget_slack(c);
+}
 
 // The row count of a list whose total the scan left at d_total (at most bound).
 static int list_rows(ac_ctx* c, SimplexList& L, const int64_t* d_total, int64_t bound, cudaStream_t s) {
@@ -601,8 +655,7 @@ static int canon_edges_by_marks(ac_ctx* c, cudaStream_t s) {
     }
     int64_t* uoff = L.v0_off.as<int64_t>();
     AC_TRY(scan_exclusive_i64(c, cnt, uoff, n, s));
-    // an edge of K^1 joins neighbours, and is free or an edge of a K^2 row
-    AC_TRY(list_rows(c, L, uoff + n, std::min((c->nb_total + 1) / 2, (int64_t)h.n_edge_pass + 3 * c->K[2].cap), s));
+    AC_TRY(list_rows(c, L, uoff + n, edge_rows_bound(c, c->K[2].cap), s));
     const int64_t count = L.cap;
     const size_t rows = (size_t)(count > 0 ? count : 1);
     AC_TRY(L.tuples.reserve(rows * 2 * sizeof(int32_t), s));
@@ -866,8 +919,7 @@ static int canon_tris_by_marks(ac_ctx* c, cudaStream_t s) {
     const unsigned wb = (unsigned)((n + TW_WARPS - 1) / TW_WARPS);
     int64_t* uoff = L.v0_off.as<int64_t>();
     AC_TRY(scan_exclusive_i64(c, cnt, uoff, n, s));
-    // a row of K^2 is a free triangle or a facet of a K^3 row
-    AC_TRY(list_rows(c, L, uoff + n, (int64_t)h.n_tri_pass + 4 * c->K[3].count, s));
+    AC_TRY(list_rows(c, L, uoff + n, tri_rows_bound(h), s));
     const int64_t count = L.cap;
     const size_t rows = (size_t)(count > 0 ? count : 1);
     AC_TRY(L.tuples.reserve(rows * 3 * sizeof(int32_t), s));
@@ -953,7 +1005,7 @@ int canonicalise(ac_ctx* c, cudaStream_t s) {
         return fail(AC_ERR_CAPACITY, "per-atom output overflow");
     Work& w = c->cw;
     const int64_t n = c->n;
-    c->deferred = !c->replaying && !c->opt.host_results && n <= DEFER_MAX_ATOMS;
+    c->deferred = may_defer(c);
     // K^3: its facets are marked from the tetrahedra as emitted, so K^2 does not wait for its rows, only the
     // filtration does, which runs on the side stream too
     const bool beside = n <= K3_BESIDE_MAX_ATOMS;

@@ -286,6 +286,8 @@ struct ac_ctx {
     bool os_forked = false;  // k_orthosize launches on the side stream await their join
     int64_t pair_words = 0;  // words of the triangle pair masks (recorded for replays)
     bool deferred = false;        // this build reads the rows of K^0..K^2 with its last wait
+    bool no_defer = false;        // set when the memory for that was not there
+    int64_t slack = 0;            // bytes its lists hold beyond their rows, as counted against DEFER_MAX_SLACK
     uint8_t* endpoint = nullptr;  // K^1's endpoint flags by input index (within scratch[2], this build's)
     ac::DevBuf pair_moff;    // first pair-mask word of each sorted position (n + 1)
     ac::DevBuf scan_tmp, scan_tmp_side;  // scans on the build's stream and on the side stream
@@ -344,6 +346,9 @@ int build_grid(ac_ctx* c, cudaStream_t s);
 int build_neighbours(ac_ctx* c, cudaStream_t s);
 int run_local(ac_ctx* c, cudaStream_t s);
 int canonicalise(ac_ctx* c, cudaStream_t s);
+void settle_slack(ac_ctx* c);   // after a deferred build: the lists' counts are known
+void drop_lists(ac_ctx* c);     // gives up the buffers of K^0..K^2, idle by now
+void forget_slack(ac_ctx* c);
 int compute_filtration(ac_ctx* c, cudaStream_t s);
 int eval_filtration(ac_ctx* c, const double* centres, const double* radii, double* const f_out[4], cudaStream_t s);
 int eval_filtration_f32(ac_ctx* c, float* const f_out[4], cudaStream_t s);
