@@ -58,7 +58,10 @@ extern "C" {
 
 /* precision of the predicate evaluation; every mode decides every predicate exactly */
 #define AC_PRECISION_FILTERED 0  /* FP32 with a forward error bound -> FP64 -> exact integers */
-#define AC_PRECISION_PLAIN_FP64 1 /* FP64 with a forward error bound -> exact integers */
+#define AC_PRECISION_PLAIN_FP64 1 /* FP64 with a forward error bound -> exact integers. What one ball rules out for
+                                     good (an edge, a triangle or a tetrahedron that no complex can hold) is told in
+                                     FP32 with a bound on the safe side, and so are the bounds themselves; every
+                                     simplex that this leaves is decided in FP64 or exact integers */
 
 /* which value ac_filtration_values returns */
 #define AC_FILTRATION_SIZE 0      /* Size (Section 2.3): radius^2 of the smallest empty orthosphere */
@@ -92,10 +95,12 @@ typedef struct {
     int64_t neighbour_pairs; /* ordered pairs of atoms whose grown balls meet */
     int32_t max_degree;
     int32_t grid_dims[3];
-    /* predicate decisions by the level that settled them: [0] FP32, [1] FP64, [2] exact */
+    /* AC2 tests by the level that settled them: [0] FP32, [1] FP64, [2] exact. AC_PRECISION_FILTERED counts the tests
+       that rule a simplex out for good among [0]; AC_PRECISION_PLAIN_FP64 does not count them (its [0] is 0): a simplex
+       ruled out so has no other test */
     int64_t ac2_tests_tet[3];
     int64_t ac2_tests_tri[3];
-    int64_t ac2_tests_edge; /* exact 64-bit integers */
+    int64_t ac2_tests_edge; /* all levels together */
     int64_t ac3_tests[4];   /* AC3 tests per dimension (edges: exact 64-bit integers) */
     int64_t ac3_exact;      /* triangle/tetrahedron AC3 tests the filter left to exact integers */
     double ms_total;        /* device time of the last ac_build (CUDA events) */
