@@ -271,7 +271,7 @@ int eval_filtration_f32(ac_ctx* c, float* const f_out[4], cudaStream_t s) {
 // at moved atoms of a 2,000-atom globule: 330 us, now 157).
 constexpr int EVAL_THREADS = 128;
 constexpr int EVAL_TILE = 512, EVAL_TILE_SHORT = 128;
-constexpr int64_t EVAL_SHORT_ROWS = 2 * 152 * EVAL_TILE;  // two blocks of EVAL_TILE rows per SM
+constexpr int64_t EVAL_SHORT_ROWS = 2 * 152 * EVAL_TILE;  // two blocks of EVAL_TILE rows for each of 152 SMs
 
 // indices (from first) of the rows of a tile with !skip(row), in no particular order
 template <int TILE, class F>

@@ -86,7 +86,7 @@
 // of k_local keeps its register budget small.
 // Edge AC3 and the vertex test are exact 64-bit integers in every mode.
 //
-// What bounds it in FP32: instruction issue (81 % of the issue slots, 18 of 32 lanes).
+// What bounds it in FP32: instruction issue (83 % of the issue slots, 18 of 32 lanes).
 // 100,000-atom probe globule, 64-bit rows: 727 us and 7,380 warp instructions per
 // atom, of which loading and ranking 670, adjacency rows 650, edges 1,020, lines
 // and enumeration 1,290, segments 1,580, AC3 on the lines 1,600, tetrahedra 560
@@ -182,8 +182,7 @@ struct LocalArgs {
     const int32_t* work;
     int counter;
     // rows of 8 words or more: the per-warp working sets in global memory (one
-    // per warp of the launch), where shared memory would hold too few of them;
-    // rows of more than 16 words always (they do not fit shared memory)
+    // per warp of the launch), where shared memory would hold too few of them
     void* gws;
     PredConst pc;
     Bounds<float> b32;
@@ -773,10 +772,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_local(LocalArgs
     constexpr bool is32 = sizeof(R) == 4;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    // working set: shared memory, or (rows of 8 words or more when the launch
-    // provides them, always beyond 16 words) one per warp in global memory
-    constexpr bool may_global = WORDS >= 8;
-    SM& S = (WORDS > 16 || (may_global && A.gws))
+    // working set: shared memory, or (rows of 8 words or more) one per warp in global memory
+    SM& S = WORDS >= 8
                 ? reinterpret_cast<SM*>(A.gws)[(size_t)blockIdx.x * (blockDim.x >> 5) + wib]
                 : reinterpret_cast<SM*>(smem_raw)[wib];
     DevCounters* cnt = A.cnt;
@@ -1620,10 +1617,6 @@ static int launch_local(ac_ctx* c, const LocalArgs& a, int64_t max_items, int wa
     return AC_OK;
 }
 
-// Atoms with 513..1024 neighbours: rows of 32 words, each warp's working set
-// (about 300 KB) in global memory, one warp per atom up to 16 per SM (the
-// kernel waits on memory: warps hide it), 2 GB of working sets at most;
-// blocks of two warps.
 // A launch whose per-warp working sets live in global memory (rows of 8 words
 // or more): as many warps as can be resident (two-warp blocks, 64 registers:
 // 32 warps per SM) where shared memory would allow 2 to 8, their working sets
@@ -1647,13 +1640,12 @@ static int launch_global(ac_ctx* c, LocalArgs a, cudaStream_t s) {
     return AC_OK;
 }
 
+// Rows of 1, 2 or 4 words: working sets in shared memory.
 template <class R>
 static int launch_words(ac_ctx* c, int words, const LocalArgs& a, int warps, cudaStream_t s) {
-    return words == 1 ? launch_local<1, R>(c, a, a.n, warps, s)
+    return words == 1   ? launch_local<1, R>(c, a, a.n, warps, s)
            : words == 2 ? launch_local<2, R>(c, a, a.n, warps, s)
-           : words == 4 ? launch_local<4, R>(c, a, a.n, warps, s)
-           : words == 8 ? launch_local<8, R>(c, a, a.n, warps, s)
-                        : launch_local<16, R>(c, a, a.n, warps, s);
+                        : launch_local<4, R>(c, a, a.n, warps, s);
 }
 
 // One per-atom pass over the work order (decreasing neighbour count). When
