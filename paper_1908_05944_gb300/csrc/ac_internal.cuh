@@ -288,6 +288,7 @@ struct ac_ctx {
     bool deferred = false;        // this build reads the rows of K^0..K^2 with its last wait
     bool no_defer = false;        // set when the memory for that was not there
     int64_t slack = 0;            // bytes its lists hold beyond their rows, as counted against DEFER_MAX_SLACK
+    int64_t slack_lists = 0;      // ... and with them
     uint8_t* endpoint = nullptr;  // K^1's endpoint flags by input index (within scratch[2], this build's)
     ac::DevBuf pair_moff;    // first pair-mask word of each sorted position (n + 1)
     ac::DevBuf scan_tmp, scan_tmp_side;  // scans on the build's stream and on the side stream
